@@ -215,8 +215,8 @@ int kin_energy_dissipation_noalloc(const double* u, int N, double nu, double* ou
  * the buffer, side and first changed byte (a kernel wrote outside the state).
  * Synchronous.
  * kin_debug_status: *is_debug (may be NULL) = 1 when this library was built
- * with KIN_DEBUG, whose stencil kernels check every global offset and the
- * shared-memory slot and row indices before use, skip an access that fails
+ * with KIN_DEBUG, whose stencil kernels check every global offset
+ * and row index before use, skip an access that fails
  * and record the first failure (bits 40..47: check site, bits 0..39: the
  * offending value) instead of trapping.  *word (may be NULL) receives that
  * record, 0 if every check passed (always 0 in the release build); reset != 0
@@ -238,14 +238,13 @@ int kin_num_shells(int N);
  *            LBE step (used up to 256) and of the two-launch DUGKS form
  *            (up to 128); with FP16/BF16 storage and even N an LBE thread
  *            takes 4 cells, or 2 when N % 4 != 0
- *   tile_y   DUGKS fused kernel: rows per tile, 4 or 8
+ *   tile_y   DUGKS fused kernel: rows per tile, 4 or 8 (by default 5, 8 or 11,
+ *            chosen with zchunk)
  *   zchunk   DUGKS fused kernel: planes each thread block marches through
- *            (default: when a plane's tile columns fill fewer than 1.5
- *            waves of blocks, the length with the shortest list schedule of
- *            the grid; otherwise about two waves of blocks)
- *   variant  DUGKS: 0 = fused single launch, f-tilde staged in shared
- *            memory by cp.async copies two planes ahead (default); 1 = two
- *            launches (pre-step into scratch, then flux + update)
+ *            (default: the tile height and length whose schedule on the
+ *            device's multiprocessors ends first)
+ *   variant  DUGKS: 0 = fused single launch (default); 1 = two launches
+ *            (pre-step into scratch, then flux + update)
  * The fused step's results do not depend on tile_y or zchunk (bitwise); the
  * two-launch form sums the same terms in another order (rounding only).
  * Other variant values return KIN_EINVAL. */
@@ -285,7 +284,7 @@ void kin_destroy(kin_sim* sim);
  * 256 steps when there are LBE members): a persistent, cooperative kernel
  * runs every step of the DUGKS members, and, on a parallel stream of the same
  * graph, one batched launch per step and storage type updates all LBE
- * members, its blocks sharing the SMs with the DUGKS blocks.  Each member's
+ * members.  Each member's
  * results are bitwise identical to stepping it alone with kin_step (a cell's
  * arithmetic does not depend on the tile shape or the launch).  There is no
  * counterpart of this batching in the paper, which runs one simulation.
@@ -296,9 +295,9 @@ typedef struct kin_ensemble kin_ensemble;
  * keeps ownership and must destroy the ensemble before any member). */
 int kin_ensemble_create(kin_sim* const* members, int n, kin_ensemble** out);
 
-/* Work decomposition: tile_y (4, 6 or 8; default 6 when the ensemble holds
- * both schemes, so that LBE blocks fit beside each DUGKS block, else 8) and
- * zchunk of the DUGKS tiles, lbe_block (a multiple of 32, at most 128) threads
+/* Work decomposition: tile_y (4, 6 or 8; the default is 5-row tiles) and
+ * zchunk of the DUGKS tiles (by default chosen for the members), lbe_block
+ * (a multiple of 32, at most 128) threads
  * per block of the batched LBE launches; values <= 0 keep the setting. */
 int kin_ensemble_set_tuning(kin_ensemble* ens, int tile_y, int zchunk, int lbe_block);
 

@@ -23,6 +23,7 @@ struct DugksCoef {
     Pr<C> c1p;       // (1 - c2, 1 - c2)
     Pr<C> third;     // (1/3, 1/3)
     Pr<C> dts;       // (-dt, dt)
+    Pr<C> h2, mh2, mhq2;  // h, -h and -h/4 in both members
 };
 
 // Interface flux through the face normal to axis A between L (the stencil

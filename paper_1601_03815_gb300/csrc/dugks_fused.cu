@@ -1,4 +1,5 @@
 // Standalone launch of the fused DUGKS step (tile code in dugks_tile.cuh).
+#include <algorithm>
 #include <atomic>
 
 #include "dugks_tile.cuh"
@@ -6,19 +7,23 @@
 
 namespace kin {
 
+// Blocks of TY-row tiles that share an SM.  Two 6-warp blocks (TY <= 5, held to
+// 168 registers a thread) run out of step, so one's exchanges overlap the
+// other's arithmetic: 0.773 ms at 256^3 against 0.93 for one 9-warp block of
+// 8-row tiles and 0.777 for one 12-warp block of 11-row tiles.
+constexpr int blocks_per_sm(int ty) { return ty <= 5 ? 2 : 1; }
+
 // VEL: also write the velocity of the new state to uvel (FP32-computed storage).
-// EVEN = false: odd N with 2-byte storage, whose tile reads f-tilde from global
-// memory directly instead of staging it.
-template <typename S, int TY, bool VEL, bool EVEN>
-__global__ void __launch_bounds__(32 * (TY + 2), 1)
+template <typename S, int TY, bool VEL>
+__global__ void __launch_bounds__(32 * (TY + 1), sizeof(typename Traits<S>::C) == 4 ? blocks_per_sm(TY) : 1)
     dugks_fused_kernel(const S* __restrict__ src, S* __restrict__ dst, int N, int zchunk,
                        DugksCoef<typename Traits<S>::C> kc, float* __restrict__ uvel) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    dugks_tile<S, TY, VEL, EVEN>(src, dst, N, blockIdx.x, blockIdx.y, blockIdx.z, zchunk, kc, smem_raw, uvel);
+    dugks_tile<S, TY, VEL>(src, dst, N, blockIdx.x, blockIdx.y, blockIdx.z, zchunk, kc, smem_raw, uvel);
 }
 
-template <typename S, int TY, bool VEL, bool EVEN>
-static cudaError_t launch_fused_e(const void* src, void* dst, int N, int zchunk,
+template <typename S, int TY, bool VEL>
+static cudaError_t launch_fused_t(const void* src, void* dst, int N, int zchunk,
                                   const DugksCoef<typename Traits<S>::C>& k, float* uvel, cudaStream_t stream) {
     const size_t smem = fused_smem_bytes<S, TY>();
     // the shared-memory limit is a per-device attribute of the kernel: set it
@@ -29,26 +34,33 @@ static cudaError_t launch_fused_e(const void* src, void* dst, int N, int zchunk,
     if (e != cudaSuccess) return e;
     const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
     if (!bit || !(configured.load() & bit)) {
-        e = cudaFuncSetAttribute(dugks_fused_kernel<S, TY, VEL, EVEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(dugks_fused_kernel<S, TY, VEL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem);
         if (e != cudaSuccess) return e;
         configured.fetch_or(bit);
     }
     if (zchunk <= 0) zchunk = 32;
     if (zchunk > N) zchunk = N;
-    dim3 block(32, TY + 2);
+    dim3 block(32, TY + 1);
     dim3 grid((N + 29) / 30, (N + TY - 1) / TY, (N + zchunk - 1) / zchunk);
-    dugks_fused_kernel<S, TY, VEL, EVEN><<<grid, block, smem, stream>>>((const S*)src, (S*)dst, N, zchunk, k, uvel);
+    dugks_fused_kernel<S, TY, VEL><<<grid, block, smem, stream>>>((const S*)src, (S*)dst, N, zchunk, k, uvel);
     return cudaGetLastError();
 }
 
-template <typename S, int TY, bool VEL>
-static cudaError_t launch_fused_t(const void* src, void* dst, int N, int zchunk,
-                                  const DugksCoef<typename Traits<S>::C>& k, float* uvel, cudaStream_t stream) {
-    if constexpr (sizeof(S) == 2) {
-        if (N % 2) return launch_fused_e<S, TY, VEL, false>(src, dst, N, zchunk, k, uvel, stream);
+template <typename S, bool VEL>
+static cudaError_t launch_fused_v(const void* src, void* dst, int N, const DugksCoef<typename Traits<S>::C>& k,
+                                  int ty, int zchunk, float* uvel, cudaStream_t stream) {
+    if constexpr (sizeof(typename Traits<S>::C) == 8) {
+        return launch_fused_t<S, 4, VEL>(src, dst, N, zchunk, k, uvel, stream);
+    } else {
+        switch (ty) {
+            case 4: return launch_fused_t<S, 4, VEL>(src, dst, N, zchunk, k, uvel, stream);
+            case 5: return launch_fused_t<S, 5, VEL>(src, dst, N, zchunk, k, uvel, stream);
+            case 8: return launch_fused_t<S, 8, VEL>(src, dst, N, zchunk, k, uvel, stream);
+            case 11: return launch_fused_t<S, 11, VEL>(src, dst, N, zchunk, k, uvel, stream);
+        }
+        return cudaErrorInvalidValue;
     }
-    return launch_fused_e<S, TY, VEL, true>(src, dst, N, zchunk, k, uvel, stream);
 }
 
 template <typename S>
@@ -58,15 +70,10 @@ static cudaError_t launch_fused(const void* src, void* dst, int N, double nu, do
     const DugksCoef<C> k = dugks_coef<C>(nu, dt);
     if constexpr (sizeof(C) == 8) {
         if (uvel) return cudaErrorInvalidValue;  // FP64 storage keeps the FP64 statistics path
-        return launch_fused_t<S, 4, false>(src, dst, N, zchunk, k, nullptr, stream);
     } else {
-        if (uvel) {
-            if (ty == 4) return launch_fused_t<S, 4, true>(src, dst, N, zchunk, k, uvel, stream);
-            return launch_fused_t<S, 8, true>(src, dst, N, zchunk, k, uvel, stream);
-        }
-        if (ty == 4) return launch_fused_t<S, 4, false>(src, dst, N, zchunk, k, nullptr, stream);
-        return launch_fused_t<S, 8, false>(src, dst, N, zchunk, k, nullptr, stream);
+        if (uvel) return launch_fused_v<S, true>(src, dst, N, k, ty, zchunk, uvel, stream);
     }
+    return launch_fused_v<S, false>(src, dst, N, k, ty, zchunk, nullptr, stream);
 }
 
 KIN_DEBUG_ACCESSOR(debug_word_dugks)
@@ -80,6 +87,85 @@ cudaError_t dugks_step_fused(int storage, const void* src, void* dst, int N, dou
         case ST_F64: return launch_fused<double>(src, dst, N, nu, dt, ty, zchunk, uvel, stream);
     }
     return cudaErrorInvalidValue;
+}
+
+namespace {
+
+// What the launch shape is chosen among, with the measured time of one plane
+// of a block (FP32, us): alone on its SM and with the SM's blocks all there.
+struct TileShape {
+    int ty, per_sm;
+    double alone, shared;
+};
+constexpr TileShape kShapes[] = {{4, 2, 1.5, 1.85}, {5, 2, 1.28, 2.0}, {8, 1, 1.76, 1.76}, {11, 1, 2.1, 2.1}};
+
+// Time (us) of the fused DUGKS launch with tiles of shape t and z chunks of zc
+// planes: blocks are issued chunk by chunk (the grid's z index varies slowest),
+// each to the SM slot that frees first, and occupy it for their planes plus
+// about 1.1 plane-times of prologue (two pre-steps and one record before the
+// first face).  All chunks but the last are equal, so whole waves are counted
+// and only the last chunk's blocks are placed, on the slots of the last
+// incomplete wave that are free earlier.
+double makespan(int N, const TileShape& t, int zc, int nsm) {
+    constexpr double kPrologue = 1.1;
+    const long long cols = (long long)((N + 29) / 30) * ((N + t.ty - 1) / t.ty);
+    const int full = N / zc, rest = N - full * zc;
+    const double plane = cols * (full + (rest > 0)) <= nsm ? t.alone : t.shared;
+    const double a = (zc + kPrologue) * plane, b = (rest + kPrologue) * plane;
+    const long long slots = (long long)nsm * t.per_sm;
+    const long long late = cols * full % slots;  // slots one wave ahead of the others
+    double early_at = (double)(cols * full / slots) * a, late_at = early_at + a;
+    double end = late > 0 ? late_at : early_at;
+    for (long long left = rest > 0 ? cols : 0; left > 0;) {
+        if (late == 0 || early_at <= late_at) {
+            left -= slots - late;
+            early_at += b;
+            end = std::max(end, early_at);
+        } else {
+            left -= late;
+            late_at += b;
+            end = std::max(end, late_at);
+        }
+    }
+    return end;
+}
+
+}  // namespace
+
+// The step lasts as long as its busiest SM, so a chunk length that leaves the
+// last wave nearly empty costs up to a third of it.  Every tile height and
+// chunk length is scored by the schedule above and the shortest taken (the
+// longest chunk among those within 0.5 %: fewer halo planes).  Measured against
+// sweeps of all shapes: 32^3 8 x 2 planes 8.2 us (5 x 3: 10.2), 48^3 8 x 4 12.3
+// us (5 x 8: 14.4), 64^3 11 x 8 22.5 us (8 x 11: 23.8), 97^3 11 x 25 61.6 us
+// (5 x 13: 66.6), 128^3 11 x 26 117 us (5 x 19: 119), 256^3 11 x 37 0.777 ms
+// (5 x 52: 0.773).
+void dugks_fused_shape(int storage, int N, int nsm, int want_ty, int want_zc, int* ty, int* zc) {
+    constexpr long long kMaxBlocks = 20000;
+    const TileShape f64{4, 1, 1.0, 1.0};
+    double best = -1.0;
+    auto consider = [&](const TileShape& t) {
+        const long long cols = (long long)((N + 29) / 30) * ((N + t.ty - 1) / t.ty);
+        for (int c = want_zc > 0 ? std::min(want_zc, N) : N; c >= 1; --c) {
+            const int nz = (N + c - 1) / c;
+            if (want_zc <= 0 && nz > 1 && (nz > 64 || cols * nz > kMaxBlocks)) break;
+            // of the lengths that give nz chunks, the smallest is the most even
+            if (want_zc <= 0 && c > 1 && (N + c - 2) / (c - 1) == nz) continue;
+            const double m = makespan(N, t, c, nsm);
+            if (best < 0.0 || m < best * (1.0 - 0.005)) {
+                best = m;
+                *ty = t.ty;
+                *zc = c;
+            }
+            if (want_zc > 0) break;
+        }
+    };
+    if (storage == ST_F64) {
+        consider(f64);
+        return;
+    }
+    for (const TileShape& t : kShapes)
+        if (want_ty > 0 ? t.ty == want_ty : t.ty != 4) consider(t);
 }
 
 }  // namespace kin

@@ -2,16 +2,11 @@
 // of f-tilde per cell.
 //
 // Each CTA owns a 30 x TY column of cells and marches along z through a chunk
-// of planes.  Its 32 x (TY + 2) threads cover the columns plus a one-cell halo;
-// every thread runs the cell pre-step (Eq. 19) of its own column for the next
-// plane into a three-plane ring of f-bar-plus in shared memory, fed by
-// cp.async copies of f-tilde issued two planes ahead (by four of the warps
-// for every row; an issuer waits for its copies at the end of a plane and
-// the next barrier publishes them).  Two block barriers per plane: one before
-// the plane's work, whose first part is the pre-step of the next plane (only
-// this thread reads the slot it fills until the next barrier, so its
-// arithmetic interleaves with the faces of this plane), and one before the
-// y faces.
+// of planes.  Warps 0..TY-1 own one row each (lanes 0 and 31 are the x halo);
+// warp TY serves both halo rows, 0 and TY + 1, which need about half of a row's
+// work (f-bar-plus and one y record), so that the TY + 1 warps are evenly
+// loaded.  A thread keeps its column's f-bar-plus of planes z and z + 1 in
+// registers and prefetches f-tilde of the plane after them.
 //
 // Interface reconstruction splits exactly between the two cells of a face.
 // With G_i^t(X) = fbp_i(X + e_t) - fbp_i(X - e_t) the Eq. 13/15/16 value at the
@@ -20,20 +15,40 @@
 //   P_i^a = (1/2 + h xi_ia) X_i - (h/4) sum_{t != a} xi_it G_i^t,
 //   M_i^a = (1/2 - h xi_ia) X_i - (h/4) sum_{t != a} xi_it G_i^t,
 // where X = fbp at the cell; summed over i, the face moments (Eq. 17) split the
-// same way through the moments of X and their tangential differences.  A cell
+// same way through the moments of X and their tangential differences.  The
+// moments of X follow from those of f-tilde (Eq. 19 conserves density and
+// momentum and relaxes Pi), so a cell forms them once, and a neighbour's
+// difference needs four of them instead of sums over its populations; of the
+// populations only the diagonal pairs have a tangential direction.  A cell
 // builds a "side record" per axis and sign (the 5 velocity pairs crossing the
 // face plus density and momentum); a face (Eqs. 17, 7, 18, 10) needs one
 // record from each neighbour: x neighbours exchange records by warp shuffles,
 // y neighbours through shared memory, z neighbours are the same thread one
 // plane apart.
 //
-// Updates lag one plane so the z face uses one cell view per plane.
+// Updates lag one plane so the z face uses one cell view per plane.  Two block
+// barriers per plane: one publishes f-bar-plus of plane z + 1 and the y records
+// of plane z, the other the y-face values.
 //
 // Opposite populations (2p+1, 2p+2) travel as one pair (pair_math.cuh): both
 // always undergo the same operation with a fixed coefficient pattern, so one
 // packed FP32x2 instruction serves both.  Flux sums are kept sign-folded,
 // Dhat_p = (D_{2p+1}, -D_{2p+2}), so a face adds the same signed value to
 // both members.
+//
+// What bounds it, 128^3 FP32: the shared-memory and shuffle pipe, 67 % of its
+// wavefront rate (FMA pipe 40 %, issue 45 %); every row's exchange is ~200
+// wavefronts a plane.  Against the form that staged f-tilde in shared memory
+// and summed the moments of every difference: 96.3 -> 59 M warp instructions,
+// 154 -> 117 us at 128^3, 0.961 -> 0.773 ms at 256^3 (2.65 -> 3.30 TB/s
+// algorithmic).  The steps of that: moments from f-tilde and f-tilde kept in
+// registers 0.961 -> 0.928; two 6-warp blocks on an SM, which drift apart so that
+// one's exchange overlaps the other's arithmetic, instead of one of 10 warps
+// -> 0.84; one base address per thread and the z loop unrolled by two (no
+// register moves), one warp for both halo rows -> 0.797; the own y-face
+// values kept in registers -> 0.773.  Not kept: mbarriers between neighbouring
+// rows in place of the block barriers (1.10), 16 warps at 128 registers (1.09:
+// spills go to L2, the shared memory leaves no L1).
 #pragma once
 
 #include <type_traits>
@@ -99,157 +114,166 @@ __device__ __forceinline__ C pdot(C x, C y, C z) {
 }
 
 // ------------------------------------------------------------------ shared memory
+// Four values that one thread writes or reads together: two pairs.
+template <typename C>
+struct alignas(16) Quad {
+    Pr<C> a, b;
+};
+
+constexpr int NXQ = 5;  // quads of a cell's exchange record
+constexpr int NBQ = 5;  // quads of an update base (19 values)
+
+// Quad (or pair) arrays, all indexed [..][row][lane] with the same row and lane
+// strides, so that every access of a thread is one base address plus a constant.
+//   XCH   [2 slots][5]: f-bar-plus of planes z and z + 1, what neighbours read of
+//         it: the diagonal pairs (3, 4), (5, 6), (7, 8) and the moments that the
+//         x and y differences need, (j_x, Pi_xx, Pi_xy, Pi_xz) and
+//         (j_y, Pi_yx, Pi_yy, Pi_yz)
+//   MY    [4]: y-face M records: pairs (0, 1), (2, 3), (4, moments 0-1), (moments 2-3, -)
+//   FY    [3]: y-face values: pairs (0, 1), (2, 3), (4, -)
+//   BASE  [2 slots][5]: f-tilde-plus of planes z - 1 and z (Eq. 20), each column's
+//         own; rows 1..TY
 template <typename C, int TY>
 struct FusedSmem {
-    Pr<C> ring[3][NPAIR][TY + 2][32];  // f-bar-plus pairs of planes z - 1, z, z + 1
-    Pr<C> my[NC][TY + 2][32];          // y-face M records (pairs)
-    Pr<C> fy[NC][TY + 1][32];          // y-face values
-    C ring0[3][TY + 2][32];            // rest population of the ring
-    C mym[4][TY + 2][32];              // y-face M records (density, momentum)
+    static constexpr int ROW = 32 * (int)sizeof(Quad<C>);
+    static constexpr int QX = (TY + 2) * ROW, QB = TY * ROW;
+    static constexpr int PAD = (int)sizeof(Quad<C>);  // lane 0 of row 0 reads one quad to its left
+    static constexpr int XCH = PAD, MY = XCH + 2 * NXQ * QX, FY = MY + 4 * QX, BASE = FY + 3 * QX - ROW,
+                         BYTES = BASE + ROW + 2 * NBQ * QB;
 };
 
-// Raw f-tilde staging for FP32 storage, filled by 4-byte cp.async copies:
-// planes z - 1 and z (awaiting their update), z + 1 (next pre-step) and z + 2
-// (in flight while plane z is computed).  One population per 128-byte row, so
-// a warp's copy instruction fills one row without bank conflicts and touches
-// one population plane; the pre-step and update read the two members of a
-// pair with two 4-byte loads.  FP64 storage reads global memory directly.
-template <int TY>
-struct RawStage {
-    float raw[4][Q][TY + 2][32];
-};
-
-template <typename S>
-constexpr bool kAsyncStage = std::is_same<S, float>::value;
-
-// Raw staging of 2-byte storage (FP16, BF16) for even N: lanes 0..16 of a
-// row's warp copy the row of each population as 17 aligned 4-byte words, the
-// 34 elements from x0 - 2; thread `lane` reads element lane + 1.  Odd N (a
-// word would straddle the periodic wrap) reads global memory directly, in a
-// separate instantiation (template flag EVEN = false) so that the even-N code
-// carries neither the branch nor the registers of that path.
-template <typename S, int TY>
-struct RawStage16 {
-    S raw[4][Q][TY + 2][34];
-};
-template <typename S>
-constexpr bool kStage16 = sizeof(S) == 2;
-
-template <typename S>
-__device__ __forceinline__ float to_float(S v) {
-    if constexpr (std::is_same<S, __half>::value) return __half2float(v);
-    else return __bfloat162float(v);
+// One quad or pair at shared-memory address a + OFF.  volatile: ordered with
+// the barriers.
+template <int OFF>
+__device__ __forceinline__ void lds(unsigned a, Quad<float>& q) {
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4 + %5];"
+                 : "=f"(q.a.x), "=f"(q.a.y), "=f"(q.b.x), "=f"(q.b.y)
+                 : "r"(a), "n"(OFF) : "memory");
 }
-
-__device__ __forceinline__ void cp_async4(void* smem_dst, const void* gsrc) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(gsrc) : "memory");
+template <int OFF>
+__device__ __forceinline__ void lds(unsigned a, float2& q) {
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2 + %3];" : "=f"(q.x), "=f"(q.y) : "r"(a), "n"(OFF) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+template <int OFF>
+__device__ __forceinline__ void lds(unsigned a, double2& q) {
+    asm volatile("ld.shared.v2.f64 {%0, %1}, [%2 + %3];" : "=d"(q.x), "=d"(q.y) : "r"(a), "n"(OFF) : "memory");
+}
+template <int OFF>
+__device__ __forceinline__ void lds(unsigned a, Quad<double>& q) {
+    lds<OFF>(a, q.a);
+    lds<OFF + 16>(a, q.b);
+}
+template <int OFF>
+__device__ __forceinline__ void sts(unsigned a, float2 p, float2 q) {
+    asm volatile("st.shared.v4.f32 [%0 + %1], {%2, %3, %4, %5};" ::"r"(a), "n"(OFF), "f"(p.x), "f"(p.y), "f"(q.x), "f"(q.y) : "memory");
+}
+template <int OFF>
+__device__ __forceinline__ void sts(unsigned a, float2 p) {
+    asm volatile("st.shared.v2.f32 [%0 + %1], {%2, %3};" ::"r"(a), "n"(OFF), "f"(p.x), "f"(p.y) : "memory");
+}
+template <int OFF>
+__device__ __forceinline__ void sts(unsigned a, double2 p) {
+    asm volatile("st.shared.v2.f64 [%0 + %1], {%2, %3};" ::"r"(a), "n"(OFF), "d"(p.x), "d"(p.y) : "memory");
+}
+template <int OFF>
+__device__ __forceinline__ void sts(unsigned a, double2 p, double2 q) {
+    sts<OFF>(a, p);
+    sts<OFF + 16>(a, q);
+}
 
 template <typename S, int TY>
 constexpr size_t fused_smem_bytes() {
-    using C = typename Traits<S>::C;
-    return sizeof(FusedSmem<C, TY>) +
-           (kAsyncStage<S> ? sizeof(RawStage<TY>) : kStage16<S> ? sizeof(RawStage16<S, TY>) : 0);
+    return FusedSmem<typename Traits<S>::C, TY>::BYTES;
 }
 
-// ------------------------------------------------------------------ cell view
-template <typename C>
-struct CellView {
-    Pr<C> X[NPAIR];   // f-bar-plus pairs at the cell
-    C X0;             // rest population
-    Pr<C> G[3][NC];   // G[t][k] = X(+e_t) - X(-e_t) for pair cross_pair(t, k)
-    C drho, j[3], pi[3][3];
-    C hrho, hj[3];    // drho / 2, j / 2
-    C DJ[3];          // DJ_t = sum_i xi_it G_i^t
-    C DP[3][3];       // DP[c][t] = sum_i xi_ic xi_it G_i^t
+// ------------------------------------------------------------------ global loads
+// f-tilde is read once, in L2 (the persistent ensemble kernel reads what other
+// blocks wrote earlier in the same launch, so never through the read-only
+// path), and kept raw until the pre-step.
+template <typename S>
+struct RawOf {
+    using T = S;
+    static __device__ __forceinline__ T load(const S* p) { return __ldcg(p); }
+    static __device__ __forceinline__ typename Traits<S>::C get(T v) { return v; }
+    template <typename P>
+    static __device__ __forceinline__ P store2(S* p0, S* p1, P v) {
+        __stcg(p0, v.x);
+        __stcg(p1, v.y);
+        return v;
+    }
+};
+template <>
+struct RawOf<__half> {
+    using T = unsigned short;
+    static __device__ __forceinline__ T load(const __half* p) {
+        return __ldcg(reinterpret_cast<const unsigned short*>(p));
+    }
+    static __device__ __forceinline__ float get(T v) { return __half2float(__ushort_as_half(v)); }
+    static __device__ __forceinline__ float2 store2(__half* p0, __half* p1, float2 v) {
+        const __half2 h = __floats2half2_rn(v.x, v.y);
+        __stcg(reinterpret_cast<unsigned short*>(p0), __half_as_ushort(__low2half(h)));
+        __stcg(reinterpret_cast<unsigned short*>(p1), __half_as_ushort(__high2half(h)));
+        return make_float2(__low2float(h), __high2float(h));
+    }
+};
+template <>
+struct RawOf<__nv_bfloat16> {
+    using T = unsigned short;
+    static __device__ __forceinline__ T load(const __nv_bfloat16* p) {
+        return __ldcg(reinterpret_cast<const unsigned short*>(p));
+    }
+    static __device__ __forceinline__ float get(T v) { return __bfloat162float(__ushort_as_bfloat16(v)); }
+    static __device__ __forceinline__ float2 store2(__nv_bfloat16* p0, __nv_bfloat16* p1, float2 v) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
+        __stcg(reinterpret_cast<unsigned short*>(p0), __bfloat16_as_ushort(__low2bfloat16(h)));
+        __stcg(reinterpret_cast<unsigned short*>(p1), __bfloat16_as_ushort(__high2bfloat16(h)));
+        return make_float2(__low2float(h), __high2float(h));
+    }
 };
 
-// Moments of X (delta-rho, j, Pi = sum xi xi X) via pair sums and differences.
+// ------------------------------------------------------------------ cells
+// f-bar-plus of one cell with its moments.
 template <typename C>
-__device__ __forceinline__ void view_moments(CellView<C>& v) {
-    C a[NPAIR], b[NPAIR];
-#pragma unroll
-    for (int p = 0; p < NPAIR; ++p) {
-        a[p] = v.X[p].x + v.X[p].y;
-        b[p] = v.X[p].x - v.X[p].y;
-    }
-    const C s34 = a[3] + a[4], s56 = a[5] + a[6], s78 = a[7] + a[8];
-    v.drho = v.X0 + (((a[0] + a[1]) + a[2]) + ((s34 + s56) + s78));
-    v.j[0] = (b[0] + b[3]) + (b[4] + (b[5] + b[6]));
-    v.j[1] = (b[1] + b[3]) - (b[4] - (b[7] + b[8]));
-    v.j[2] = (b[2] + b[5]) - (b[6] - (b[7] - b[8]));
-    v.pi[0][0] = a[0] + (s34 + s56);
-    v.pi[1][1] = a[1] + (s34 + s78);
-    v.pi[2][2] = a[2] + (s56 + s78);
-    v.pi[0][1] = v.pi[1][0] = a[3] - a[4];
-    v.pi[0][2] = v.pi[2][0] = a[5] - a[6];
-    v.pi[1][2] = v.pi[2][1] = a[7] - a[8];
-    v.hrho = C(0.5) * v.drho;
-    v.hj[0] = C(0.5) * v.j[0];
-    v.hj[1] = C(0.5) * v.j[1];
-    v.hj[2] = C(0.5) * v.j[2];
-}
+struct Cell {
+    Pr<C> X[NPAIR];
+    Pr<C> rj, jj;       // halves: (delta-rho, j_x) / 2, (j_y, j_z) / 2
+    Quad<C> m[3];       // m[a] = (j_a, Pi_a0, Pi_a1, Pi_a2)
+};
 
-// Coefficient of term k in a difference sum of axis T: W = 3 gives DJ_T
-// (weight e_pT on G.x - G.y), W = c gives DP[c][T] (weight e_pc e_pT on
-// G.x + G.y).
-template <int T, int W>
-__host__ __device__ constexpr int dcoef(int k) {
-    return W == 3 ? pe(cross_pair(T, k), T) : pe(cross_pair(T, k), W) * pe(cross_pair(T, k), T);
+// Differences across a cell along one axis T: the two diagonal pairs named and
+// (DJ_T, DP_0T, DP_1T, DP_2T).
+template <typename C>
+__device__ __forceinline__ Quad<C> qsub(const Quad<C>& p, const Quad<C>& m) {
+    return Quad<C>{psub(p.a, m.a), psub(p.b, m.b)};
 }
-// Signed sum of vals[k] over the nonzero coefficients, starting from the first
-// term (no addition of zero).
-template <int T, int W, int K, bool STARTED, typename C>
-__device__ __forceinline__ C dsum(const C (&vals)[NC], C acc) {
-    if constexpr (K == NC) {
-        return acc;
-    } else {
-        constexpr int cf = dcoef<T, W>(K);
-        if constexpr (cf == 0) {
-            return dsum<T, W, K + 1, STARTED>(vals, acc);
-        } else if constexpr (!STARTED) {
-            return dsum<T, W, K + 1, true>(vals, cf > 0 ? vals[K] : -vals[K]);
-        } else {
-            return dsum<T, W, K + 1, true>(vals, cf > 0 ? acc + vals[K] : acc - vals[K]);
-        }
-    }
-}
-
-// DJ and DP for the tangential directions T in MASK (bit t set).
-template <int MASK, typename C>
-__device__ __forceinline__ void view_diffs(CellView<C>& v) {
-    static_for<0, 3>([&](auto tc) {
-        constexpr int T = decltype(tc)::value;
-        if constexpr ((MASK >> T) & 1) {
-            C sg[NC], dg[NC];
-#pragma unroll
-            for (int k = 0; k < NC; ++k) {
-                sg[k] = v.G[T][k].x + v.G[T][k].y;
-                dg[k] = v.G[T][k].x - v.G[T][k].y;
-            }
-            v.DJ[T] = dsum<T, 3, 0, false>(dg, C(0));
-            v.DP[0][T] = dsum<T, 0, 0, false>(sg, C(0));
-            v.DP[1][T] = dsum<T, 1, 0, false>(sg, C(0));
-            v.DP[2][T] = dsum<T, 2, 0, false>(sg, C(0));
-        }
-    });
+template <typename C>
+__device__ __forceinline__ Quad<C> qadd(const Quad<C>& p, const Quad<C>& m) {
+    return Quad<C>{padd(p.a, m.a), padd(p.b, m.b)};
 }
 
 // ------------------------------------------------------------------ side records
 template <typename C>
 struct Rec {
-    Pr<C> r[NC];  // pairs crossing the face, in cross_pair order
-    C m[4];       // density, momentum
+    Pr<C> r[NC];   // pairs crossing the face, in cross_pair order
+    Pr<C> m0, m1;  // (density, momentum x), (momentum y, z)
 };
 
 // P (cell on the lower side of the face along A) and M (upper side) records.
+// g[k], k = 1..4: the tangential difference of diagonal pair cross_pair(A, k);
+// d: the sum of the moment differences along the two tangential axes.
 template <int A, bool WANT_P, bool WANT_M, typename C>
-__device__ __forceinline__ void side_records(const CellView<C>& v, const DugksCoef<C>& k, Rec<C>& P,
-                                             Rec<C>& M) {
-    constexpr int T1 = (A + 1) % 3, T2 = (A + 2) % 3;
+__device__ __forceinline__ void side_records(const Cell<C>& v, const Pr<C> (&g)[NC], const Quad<C>& d,
+                                             const DugksCoef<C>& k, Rec<C>& P, Rec<C>& M) {
+    const Pr<C> b0 = pfma(k.mhq2, d.a, v.rj);
+    const Pr<C> b1 = pfma(k.mhq2, d.b, v.jj);
+    if constexpr (WANT_P) {
+        P.m0 = pfma(k.h2, v.m[A].a, b0);
+        P.m1 = pfma(k.h2, v.m[A].b, b1);
+    }
+    if constexpr (WANT_M) {
+        M.m0 = pfma(k.mh2, v.m[A].a, b0);
+        M.m1 = pfma(k.mh2, v.m[A].b, b1);
+    }
     static_for<0, NC>([&](auto kc) {
         constexpr int K = decltype(kc)::value;
         constexpr int p = cross_pair(A, K);
@@ -258,25 +282,19 @@ __device__ __forceinline__ void side_records(const CellView<C>& v, const DugksCo
         [[maybe_unused]] const Pr<C> cP = sg > 0 ? k.cpp : k.cpm;
         [[maybe_unused]] const Pr<C> cM = sg > 0 ? k.cpm : k.cpp;
         if constexpr (p < 3) {
+            // the axis pair (K = 0): M carries fbp, the face scales it, so that no
+            // product feeds a plain addition (which the compiler may contract in one
+            // inlined copy and not in another)
             if constexpr (WANT_P) P.r[K] = pmul(cP, v.X[p]);
-            if constexpr (WANT_M) M.r[K] = pmul(cM, v.X[p]);
+            if constexpr (WANT_M) M.r[K] = v.X[p];
         } else {
             constexpr int T = tang_axis(p, A);
             constexpr int tau = pe(p, T);
             // -(h/4) xi_iT G_i^T for both members
-            const Pr<C> ht = pmul(tau > 0 ? k.hqp : k.hqm, v.G[T][cross_index(T, p)]);
+            const Pr<C> ht = pmul(tau > 0 ? k.hqp : k.hqm, g[K]);
             if constexpr (WANT_P) P.r[K] = pfma(cP, v.X[p], ht);
             if constexpr (WANT_M) M.r[K] = pfma(cM, v.X[p], ht);
         }
-    });
-    const C br = fma(-k.hq, v.DJ[T1] + v.DJ[T2], v.hrho);
-    if constexpr (WANT_P) P.m[0] = fma(k.h, v.j[A], br);
-    if constexpr (WANT_M) M.m[0] = fma(-k.h, v.j[A], br);
-    static_for<0, 3>([&](auto ccn) {
-        constexpr int CC = decltype(ccn)::value;
-        const C bc = fma(-k.hq, v.DP[CC][T1] + v.DP[CC][T2], v.hj[CC]);
-        if constexpr (WANT_P) P.m[1 + CC] = fma(k.h, v.pi[A][CC], bc);
-        if constexpr (WANT_M) M.m[1 + CC] = fma(-k.h, v.pi[A][CC], bc);
     });
 }
 
@@ -285,8 +303,8 @@ __device__ __forceinline__ void side_records(const CellView<C>& v, const DugksCo
 template <int A, typename C>
 __device__ __forceinline__ void face_values(const Rec<C>& P, const Rec<C>& M, const DugksCoef<C>& k,
                                             Pr<C> (&ff)[NC]) {
-    const C rho = P.m[0] + M.m[0];
-    const C ux = P.m[1] + M.m[1], uy = P.m[2] + M.m[2], uz = P.m[3] + M.m[3];
+    const Pr<C> m0 = padd(P.m0, M.m0), m1 = padd(P.m1, M.m1);
+    const C rho = m0.x, ux = m0.y, uy = m1.x, uz = m1.y;
     const C a0 = fma(C(-1.5), fma(uz, uz, fma(uy, uy, ux * ux)), rho);
     const C wa_ax = k.qw[0] * a0, wa_dg = k.qw[1] * a0;
     static_for<0, NC>([&](auto kc) {
@@ -295,8 +313,9 @@ __device__ __forceinline__ void face_values(const Rec<C>& P, const Rec<C>& M, co
         constexpr int cls = p < 3 ? 0 : 1;
         const C s = pdot<p>(ux, uy, uz);
         const C q = fma(k.qk[cls] * s, s, cls == 0 ? wa_ax : wa_dg);  // c2 W (a0 + 9/2 s^2)
-        const C l = k.ql[cls] * s;                                   // c2 3W s
-        ff[K] = pfma(k.c1p, padd(P.r[K], M.r[K]), pmk(q + l, q - l));
+        // +/- c2 3W s
+        const Pr<C> fb = K == 0 ? pfma(k.cpm, M.r[K], P.r[K]) : padd(P.r[K], M.r[K]);
+        ff[K] = pfma(k.c1p, fb, pmk(fma(k.ql[cls], s, q), fma(-k.ql[cls], s, q)));
     });
 }
 
@@ -309,6 +328,11 @@ __device__ __forceinline__ Pr<C> pshfl_up1(Pr<C> v) {
     return pmk(__shfl_up_sync(0xffffffffu, v.x, 1), __shfl_up_sync(0xffffffffu, v.y, 1));
 }
 
+template <typename T>
+__device__ __forceinline__ T opaque(T v) {
+    asm volatile("" : "+r"(v));
+    return v;
+}
 __device__ __forceinline__ int wrapc(int v, int n) {
     v %= n;
     return v < 0 ? v + n : v;
@@ -316,309 +340,277 @@ __device__ __forceinline__ int wrapc(int v, int n) {
 
 // ------------------------------------------------------------------ the tile
 // One tile (tile coordinates bx, by, bz) of the fused step, run by a
-// 32 x (TY + 2) thread block with fused_smem_bytes<S, TY>() of dynamic shared
+// 32 x (TY + 1) thread block with fused_smem_bytes<S, TY>() of dynamic shared
 // memory at smem_raw (16-byte aligned).  Also called by the persistent
 // ensemble kernel.  With VEL (FP32-computed storage) the tile also writes
 // rho0 u = sum xi f of the stored new state (Eq. 8) to uvel[3][N^3], summed in
 // population order.
-template <typename S, int TY, bool VEL = false, bool EVEN = true>
+template <typename S, int TY, bool VEL = false>
 __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restrict__ dst, int N,
                                            int bx, int by, int bz, int zchunk,
                                            const DugksCoef<typename Traits<S>::C>& kc,
                                            unsigned char* smem_raw, float* __restrict__ uvel = nullptr) {
     using C = typename Traits<S>::C;
     using P2 = Pr<C>;
+    using Q4 = Quad<C>;
+    using SM = FusedSmem<C, TY>;
     static_assert(!VEL || std::is_same<C, float>::value, "the fused velocity serves FP32-computed storage");
-    FusedSmem<C, TY>& sm = *reinterpret_cast<FusedSmem<C, TY>*>(smem_raw);
-    RawStage<TY>* stage = reinterpret_cast<RawStage<TY>*>(smem_raw + sizeof(FusedSmem<C, TY>));
-    RawStage16<S, TY>* stage16 = reinterpret_cast<RawStage16<S, TY>*>(smem_raw + sizeof(FusedSmem<C, TY>));
 
-    const int lane = threadIdx.x, row = threadIdx.y;
-    const int x0 = bx * 30, y0 = by * TY, z0 = bz * zchunk;
+    // read once: recomputed from the special registers and the layout, the
+    // shared-memory addresses cost ~20 instructions a plane
+    const int lane = opaque((int)threadIdx.x);
+    const bool halo = threadIdx.y == TY;
+    const int row = opaque(halo ? 0 : (int)threadIdx.y + 1);
+    if (!KIN_CHECK((int)threadIdx.y <= TY && lane < 32, DBG_DUGKS_ROW, threadIdx.y)) return;
+    const unsigned own = opaque((unsigned)__cvta_generic_to_shared(smem_raw) + row * SM::ROW + lane * (int)sizeof(Q4));
+    const int z0 = bz * zchunk;
     const int zend = min(z0 + zchunk, N);
-    const int gxr = x0 - 1 + lane, gyr = y0 - 1 + row;
+    const int gxr = bx * 30 - 1 + lane, gyr = by * TY - 1 + row;
     const int gx = wrapc(gxr, N), gy = wrapc(gyr, N);
-    const bool xin = lane >= 1 && lane <= 30;
-    const bool yin = row >= 1 && row <= TY;
-    const bool interior = xin && yin;
-    const bool valid = interior && gxr < N && gyr < N;
+    const bool valid = lane >= 1 && lane <= 30 && gxr < N && gyr < N;
     const size_t plane = (size_t)N * N * N;
-    const size_t colidx = (size_t)gx + (size_t)N * gy;
-    const size_t nn = (size_t)N * N;
-    // x neighbours, clamped so the two halo lanes can run the interior code
-    // path (their x differences are never used)
-    const int lp = min(lane + 1, 31), lm = max(lane - 1, 0);
+    // cell indices fit in 32 bits (N <= 1024)
+    const unsigned nn32 = (unsigned)N * N, col32 = (unsigned)gx + (unsigned)N * gy;
 
     auto zwrap = [&](int z) { return z < 0 ? z + N : (z >= N ? z - N : z); };
-    auto rslot_of = [&](int z) { return (z - z0 + 4) & 3; };
 
-    // 2-byte staging (EVEN: the caller guarantees an even N): this lane's word
-    // starts at element x0 - 2 + 2 lane (even, so it never straddles the wrap)
-    constexpr bool use16 = kStage16<S> && EVEN;
-    const size_t rowidx = (size_t)N * gy + (size_t)wrapc(x0 - 2 + 2 * lane, N);
-
-    // The staging copies of all rows are issued by the warps of rows r with
-    // r % 4 >= 2 (rows 2, 3, 6, 7 of a 10-row block; warps are dealt to the
-    // SM's four schedulers in turn, so these sit on the two that hold two
-    // warps instead of three).  Row r2's copies go to issuer r2 % NI; an
-    // issuer takes at most KR rows.  Measured against every thread copying
-    // its own column: FP32 unchanged (0.961 vs 0.964 ms at 256^3), FP16 and
-    // BF16 3 % faster (a 2-byte row is copied by 17 of the 32 lanes).
-    constexpr int NW = TY + 2;
-    constexpr int NI = (NW / 4) * 2 + (NW % 4 > 2 ? NW % 4 - 2 : 0);
-    constexpr int KR = (NW + NI - 1) / NI;
-    const bool issuer = (row & 3) >= 2;
-    const int iidx = (row >> 2) * 2 + (row & 3) - 2;  // rank among the issuers (issuers only)
-    unsigned icol[KR];  // y + N x part of each assigned row's column (x from this lane)
+    // raw f-tilde of this thread's column at plane z
+    using Raw = typename RawOf<S>::T;
+    auto load_plane = [&](int z, unsigned col, Raw (&fr)[Q]) {
+        const unsigned o = (unsigned)zwrap(z) * nn32 + col;
+        if (!KIN_CHECK(o < plane, DBG_DUGKS_LOAD, o)) return;
 #pragma unroll
-    for (int k = 0; k < KR; ++k) {
-        const int r2 = iidx + k * NI;
-        const int gy2 = wrapc(y0 - 1 + (r2 < NW ? r2 : 0), N);
-        if constexpr (use16) icol[k] = (unsigned)N * gy2 + (unsigned)wrapc(x0 - 2 + 2 * lane, N);
-        else icol[k] = (unsigned)gx + (unsigned)N * gy2;
-    }
-
-    // issuers only: the copies of plane z for their assigned rows
-    auto issue_plane = [&](int z) {
-        const int s = rslot_of(z);
-#pragma unroll
-        for (int k = 0; k < KR; ++k) {
-            const int r2 = iidx + k * NI;
-            if (r2 >= NW) continue;
-            const size_t o = (size_t)zwrap(z) * nn + icol[k];
-            if constexpr (use16) {
-                if (lane <= 16) {
-#pragma unroll
-                    for (int i = 0; i < Q; ++i)
-                        if (KIN_CHECK(o + i * plane + 1 < Q * plane, DBG_DUGKS_LOAD, o + i * plane + 1) &&
-                            KIN_CHECK(s >= 0 && s < 4, DBG_DUGKS_SLOT, s))
-                            cp_async4(&stage16->raw[s][i][r2][2 * lane], src + o + i * plane);
-                }
-            }
-            if constexpr (kAsyncStage<S>) {
-#pragma unroll
-                for (int i = 0; i < Q; ++i)
-                    if (KIN_CHECK(o + i * plane < Q * plane, DBG_DUGKS_LOAD, o + i * plane) &&
-                        KIN_CHECK(s >= 0 && s < 4, DBG_DUGKS_SLOT, s))
-                        cp_async4(&stage->raw[s][i][r2][lane], src + o + i * plane);
-            }
-        }
-        cp_async_commit();
-    };
-    auto raw_pair = [&](int z, int q) -> P2 {
-        if constexpr (kAsyncStage<S>) {
-            const int s = rslot_of(z);
-            return pmk(stage->raw[s][2 * q + 1][row][lane], stage->raw[s][2 * q + 2][row][lane]);
-        } else if constexpr (use16) {
-            const int s = rslot_of(z);
-            return pmk(to_float(stage16->raw[s][2 * q + 1][row][lane + 1]),
-                       to_float(stage16->raw[s][2 * q + 2][row][lane + 1]));
-        } else {
-            const size_t o = (size_t)zwrap(z) * nn + colidx;
-            if (!KIN_CHECK(o + (2 * q + 2) * plane < Q * plane, DBG_DUGKS_LOAD, o + (2 * q + 2) * plane))
-                return pmk(C(0), C(0));
-            return pmk(Traits<S>::load(src + o + (2 * q + 1) * plane), Traits<S>::load(src + o + (2 * q + 2) * plane));
-        }
-    };
-    auto raw_rest = [&](int z) -> C {
-        if constexpr (kAsyncStage<S>) {
-            return stage->raw[rslot_of(z)][0][row][lane];
-        } else if constexpr (use16) {
-            return to_float(stage16->raw[rslot_of(z)][0][row][lane + 1]);
-        } else {
-            const size_t o = (size_t)zwrap(z) * nn + colidx;
-            if (!KIN_CHECK(o < plane, DBG_DUGKS_LOAD, o)) return C(0);
-            return Traits<S>::load(src + o);
-        }
+        for (int i = 0; i < Q; ++i) fr[i] = RawOf<S>::load(src + i * plane + o);
     };
 
-    // Eq. 19 for this thread's column at plane z into ring slot s:
-    // fbp = f + b (f_eq - f), f_eq of a pair = q +/- l (Eq. 7).
-    auto prestep = [&](int z, int s) {
+    // Eq. 19 of the column's raw values: fbp = f + b (f_eq - f), f_eq of a pair
+    // = q +/- l (Eq. 7), with the moments of fbp: delta-rho and j are those of
+    // f, Pi = Pi_f + b (Pi_eq - Pi_f) with Pi_eq = delta-rho / 3 I + j j.  The
+    // exchange record goes to slot SL.  With KEEP also f-tilde-plus = 4/3 fbp -
+    // 1/3 f-tilde (Eq. 20), kept in the column's own slot until the update.
+    auto prestep = [&](auto slc, auto keepc, unsigned own, const Raw (&fr)[Q], Cell<C>& n) {
+        constexpr int SL = decltype(slc)::value;
+        constexpr bool keep = decltype(keepc)::value;
         P2 f[NPAIR];
 #pragma unroll
-        for (int q = 0; q < NPAIR; ++q) f[q] = raw_pair(z, q);
-        const C f0 = raw_rest(z);
+        for (int q = 0; q < NPAIR; ++q) f[q] = pmk(RawOf<S>::get(fr[2 * q + 1]), RawOf<S>::get(fr[2 * q + 2]));
+        const C f0 = RawOf<S>::get(fr[0]);
         C a[NPAIR], b[NPAIR];
 #pragma unroll
         for (int q = 0; q < NPAIR; ++q) {
             a[q] = f[q].x + f[q].y;
             b[q] = f[q].x - f[q].y;
         }
-        const C drho = f0 + (((a[0] + a[1]) + a[2]) + (((a[3] + a[4]) + (a[5] + a[6])) + (a[7] + a[8])));
+        const C s34 = a[3] + a[4], s56 = a[5] + a[6], s78 = a[7] + a[8];
+        const C drho = f0 + (((a[0] + a[1]) + a[2]) + ((s34 + s56) + s78));
         const C jx = (b[0] + b[3]) + (b[4] + (b[5] + b[6]));
         const C jy = (b[1] + b[3]) - (b[4] - (b[7] + b[8]));
         const C jz = (b[2] + b[5]) - (b[6] - (b[7] - b[8]));
+        const C r3 = mul_rn(drho, C(1) / C(3));
+        auto relax = [&](C pf, C ja, C jb, C r) { return fma(kc.b, fma(ja, jb, r - pf), pf); };
+        const C pxx = relax(a[0] + (s34 + s56), jx, jx, r3);
+        const C pyy = relax(a[1] + (s34 + s78), jy, jy, r3);
+        const C pzz = relax(a[2] + (s56 + s78), jz, jz, r3);
+        const C pxy = relax(a[3] - a[4], jx, jy, C(0));
+        const C pxz = relax(a[5] - a[6], jx, jz, C(0));
+        const C pyz = relax(a[7] - a[8], jy, jz, C(0));
+        n.rj = pmk(C(0.5) * drho, C(0.5) * jx);
+        n.jj = pmk(C(0.5) * jy, C(0.5) * jz);
+        n.m[0] = Q4{pmk(jx, pxx), pmk(pxy, pxz)};
+        n.m[1] = Q4{pmk(jy, pxy), pmk(pyy, pyz)};
+        n.m[2] = Q4{pmk(jz, pxz), pmk(pyz, pzz)};
+        constexpr int X = SM::XCH + SL * NXQ * SM::QX;
+        constexpr int B = SM::BASE + SL * NBQ * SM::QB;
+        sts<X + 3 * SM::QX>(own, n.m[0].a, n.m[0].b);
+        sts<X + 4 * SM::QX>(own, n.m[1].a, n.m[1].b);
         const C a0 = fma(C(-1.5), fma(jz, jz, fma(jy, jy, jx * jx)), drho);
         const C wa_ax = (C(2) / C(36)) * a0, wa_dg = (C(1) / C(36)) * a0;
+        P2 t[NPAIR];
         static_for<0, NPAIR>([&](auto pc) {
             constexpr int PP = decltype(pc)::value;
             constexpr bool AX = PP < 3;
             const C sd = pdot<PP>(jx, jy, jz);
             // W (a0 + 9/2 s^2) with 9/2 W = 1/4 (axis) or 1/8 (diagonal)
             const C q = fma(C(AX ? 0.25 : 0.125) * sd, sd, AX ? wa_ax : wa_dg);
-            const C l = lin3w<C>(AX ? 1 : 2) * sd;
-            sm.ring[s][PP][row][lane] = pfma(kc.b2, psub(pmk(q + l, q - l), f[PP]), f[PP]);
-        });
-        sm.ring0[s][row][lane] = fma(kc.b, (C(12) / C(36)) * a0 - f0, f0);
-    };
-
-    // Cell view at ring slot s0 with the tangential differences in MASK.
-    auto gather = [&](int s0, int sm1, int sp1, auto maskc, CellView<C>& v) {
-        constexpr int MASK = decltype(maskc)::value;
-#pragma unroll
-        for (int q = 0; q < NPAIR; ++q) v.X[q] = sm.ring[s0][q][row][lane];
-        v.X0 = sm.ring0[s0][row][lane];
-        static_for<0, 3>([&](auto tc) {
-            constexpr int T = decltype(tc)::value;
-            if constexpr ((MASK >> T) & 1) {
-                static_for<0, NC>([&](auto kc2) {
-                    constexpr int K = decltype(kc2)::value;
-                    constexpr int p = cross_pair(T, K);
-                    if constexpr (T == 0) {
-                        v.G[0][K] = psub(sm.ring[s0][p][row][lp], sm.ring[s0][p][row][lm]);
-                    } else if constexpr (T == 1) {
-                        if (KIN_CHECK(row >= 1 && row <= TY, DBG_DUGKS_ROW, row))
-                            v.G[1][K] = psub(sm.ring[s0][p][row + 1][lane], sm.ring[s0][p][row - 1][lane]);
-                    } else {
-                        v.G[2][K] = psub(sm.ring[sp1][p][row][lane], sm.ring[sm1][p][row][lane]);
-                    }
-                });
+            constexpr C w3 = lin3w<C>(AX ? 1 : 2);
+            n.X[PP] = pfma(kc.b2, psub(pmk(fma(w3, sd, q), fma(-w3, sd, q)), f[PP]), f[PP]);
+            t[PP] = pfma(kc.third, psub(n.X[PP], f[PP]), n.X[PP]);
+            if constexpr (PP == 4) sts<X>(own, n.X[3], n.X[4]);
+            if constexpr (PP == 6) sts<X + SM::QX>(own, n.X[5], n.X[6]);
+            if constexpr (PP == 8) sts<X + 2 * SM::QX>(own, n.X[7], n.X[8]);
+            if constexpr (PP % 2 == 1) {
+                if constexpr (keep) sts<B + (PP / 2) * SM::QB>(own, t[PP - 1], t[PP]);
             }
         });
-        view_moments(v);
-        view_diffs<MASK>(v);
-    };
-
-    // ring slots of planes z - 1, z, z + 1 (rotated every plane)
-    int s_m1 = 2, s_0 = 0, s_p1 = 1;
-
-    // Copies become visible to every thread by the issuer's wait followed by a
-    // block barrier: the copies of plane z + 2, issued right after the first
-    // barrier of plane z, are waited for at the end of plane z.
-    constexpr bool staged = kAsyncStage<S> || use16;
-    if constexpr (staged) {
-        if (issuer) {
-            issue_plane(z0 - 1);
-            issue_plane(z0);
-            if (z0 + 1 <= zend) issue_plane(z0 + 1);
-            cp_async_wait_all();
+        if constexpr (keep) {
+            const C X0 = fma(kc.b, fma(C(12) / C(36), a0, -f0), f0);
+            sts<B + 4 * SM::QB>(own, t[8], pmk(fma(C(1.0 / 3.0), X0 - f0, X0), C(0)));
         }
-        __syncthreads();
-    }
-    prestep(z0 - 1, s_m1);
-    prestep(z0, s_0);
-    __syncthreads();
+    };
 
-    Rec<C> Pz;        // P^z record of the plane below the current one
-    P2 Dprev[NPAIR];  // sign-folded flux sums of plane z - 1, still missing its +z face
-    P2 Dcur[NPAIR];
+    // differences of quad K of exchange slot SL along x and y.  The outer lanes
+    // read past their row: their x differences are never used.
+    auto diff_x = [&](auto slc, auto kc2, unsigned own) {
+        constexpr int O = SM::XCH + decltype(slc)::value * NXQ * SM::QX + decltype(kc2)::value * SM::QX;
+        Q4 p, m;
+        lds<O + (int)sizeof(Q4)>(own, p);
+        lds<O - (int)sizeof(Q4)>(own, m);
+        return qsub<C>(p, m);
+    };
+    auto diff_y = [&](auto slc, auto kc2) {
+        constexpr int O = SM::XCH + decltype(slc)::value * NXQ * SM::QX + decltype(kc2)::value * SM::QX;
+        Q4 p, m;
+        lds<O + SM::ROW>(own, p);
+        lds<O - SM::ROW>(own, m);
+        return qsub<C>(p, m);
+    };
+    constexpr auto k0 = std::integral_constant<int, 0>{};
+    constexpr auto k1 = std::integral_constant<int, 1>{};
+    constexpr auto k2 = std::integral_constant<int, 2>{};
+    constexpr auto k3 = std::integral_constant<int, 3>{};
+    constexpr auto k4 = std::integral_constant<int, 4>{};
+
+    auto y_face = [&](const Rec<C>& Py, unsigned own, P2 (&ffy)[NC]) {
+        // face between this row and the one above
+        Rec<C> Mu;
+        Q4 q0, q1, q2;
+        lds<SM::MY + SM::ROW>(own, q0);
+        lds<SM::MY + SM::QX + SM::ROW>(own, q1);
+        lds<SM::MY + 2 * SM::QX + SM::ROW>(own, q2);
+        lds<SM::MY + 3 * SM::QX + SM::ROW>(own, Mu.m1);
+        Mu.r[0] = q0.a, Mu.r[1] = q0.b, Mu.r[2] = q1.a, Mu.r[3] = q1.b, Mu.r[4] = q2.a;
+        Mu.m0 = q2.b;
+        face_values<1>(Py, Mu, kc, ffy);
+        sts<SM::FY>(own, ffy[0], ffy[1]);
+        sts<SM::FY + SM::QX>(own, ffy[2], ffy[3]);
+        sts<SM::FY + 2 * SM::QX>(own, ffy[4]);
+    };
+    auto sync = [] { asm volatile("bar.sync 0, %0;" ::"n"(32 * (TY + 1)) : "memory"); };
+
+    if (halo) {
+        // rows 0 and TY + 1: f-bar-plus for their neighbours, the P record of row
+        // 0 with its y face, the M record of row TY + 1
+        const unsigned ownr[2] = {own, own + (TY + 1) * SM::ROW};
+        const unsigned col[2] = {col32, (unsigned)gx + (unsigned)N * wrapc(by * TY + TY, N)};
+        Cell<C> A[2], B[2];
+        Raw fr[2][Q];
 #pragma unroll
-    for (int q = 0; q < NPAIR; ++q) {
-        Dprev[q] = pmk(C(0), C(0));
-        Dcur[q] = pmk(C(0), C(0));
+        for (int r = 0; r < 2; ++r) {
+            load_plane(z0 - 1, col[r], fr[r]);
+            prestep(k1, std::false_type{}, ownr[r], fr[r], B[r]);
+            load_plane(z0, col[r], fr[r]);
+            prestep(k0, std::false_type{}, ownr[r], fr[r], A[r]);
+            if (z0 + 1 <= zend) load_plane(z0 + 1, col[r], fr[r]);
+        }
+        sync();
+        auto advance = [&](auto slc, int z, Cell<C> (&cur)[2], Cell<C> (&nxt)[2]) -> bool {
+            constexpr auto other = std::integral_constant<int, decltype(slc)::value ^ 1>{};
+            sync();
+            if (z == zend) return true;
+            Rec<C> Py, My, unused;
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const Q4 zp78{nxt[r].X[7], nxt[r].X[8]}, zpm = nxt[r].m[2];
+                prestep(other, std::false_type{}, ownr[r], fr[r], nxt[r]);
+                const Q4 z78 = qsub<C>(Q4{nxt[r].X[7], nxt[r].X[8]}, zp78), zm = qsub<C>(nxt[r].m[2], zpm);
+                if (z + 2 <= zend) load_plane(z + 2, col[r], fr[r]);
+                const Q4 xp = diff_x(slc, k0, ownr[r]), xm = diff_x(slc, k3, ownr[r]);
+                const P2 g[NC] = {P2{}, xp.a, xp.b, z78.a, z78.b};
+                if (r == 0) {
+                    side_records<1, true, false>(cur[r], g, qadd<C>(xm, zm), kc, Py, unused);
+                } else {
+                    side_records<1, false, true>(cur[r], g, qadd<C>(xm, zm), kc, unused, My);
+                    sts<SM::MY>(ownr[r], My.r[0], My.r[1]);
+                    sts<SM::MY + SM::QX>(ownr[r], My.r[2], My.r[3]);
+                    sts<SM::MY + 2 * SM::QX>(ownr[r], My.r[4], My.m0);
+                    sts<SM::MY + 3 * SM::QX>(ownr[r], My.m1);
+                }
+            }
+            sync();
+            P2 ffy[NC];
+            y_face(Py, ownr[0], ffy);
+            return false;
+        };
+        for (int z = z0;; z += 2) {
+            if (advance(k0, z, A, B)) return;
+            if (advance(k1, z + 1, B, A)) return;
+        }
     }
-    if (interior) {
-        CellView<C> v;
+
+    Cell<C> A, B;          // planes z and z - 1, in turn
+    Raw fr[Q];
+    Rec<C> Pz;             // P^z record of plane z - 1
+    P2 ffy[NC] = {};       // upper y-face values of plane z - 1
+    P2 D[NPAIR];           // sign-folded flux sums of plane z - 1, still missing z and y faces
+#pragma unroll
+    for (int q = 0; q < NPAIR; ++q) D[q] = pmk(C(0), C(0));
+
+    // prologue: planes z0 - 1 (slot 1) and z0 (slot 0)
+    load_plane(z0 - 1, col32, fr);
+    prestep(k1, std::false_type{}, own, fr, B);
+    load_plane(z0, col32, fr);
+    prestep(k0, std::true_type{}, own, fr, A);
+    if (z0 + 1 <= zend) load_plane(z0 + 1, col32, fr);
+    sync();
+    {
+        const Q4 xq = diff_x(k1, k1, own), xm = diff_x(k1, k3, own), yq = diff_y(k1, k2), ym = diff_y(k1, k4);
+        const P2 g[NC] = {P2{}, xq.a, xq.b, yq.a, yq.b};
         Rec<C> unused;
-        gather(s_m1, s_m1, s_m1, std::integral_constant<int, 3>{}, v);
-        side_records<2, true, false>(v, kc, Pz, unused);
+        side_records<2, true, false>(B, g, qadd<C>(xm, ym), kc, Pz, unused);
     }
 
-    for (int z = z0; z <= zend; ++z) {
+    // One plane: cur is plane z (exchange slot SL), nxt holds plane z - 1 and
+    // leaves with plane z + 1.
+    auto advance = [&](auto slc, int z, Cell<C>& cur, Cell<C>& nxt) -> bool {
+        constexpr int SL = decltype(slc)::value;
+        constexpr auto other = std::integral_constant<int, SL ^ 1>{};
         const bool last = z == zend;
-        if (!KIN_CHECK(s_m1 >= 0 && s_m1 < 3 && s_0 >= 0 && s_0 < 3 && s_p1 >= 0 && s_p1 < 3, DBG_DUGKS_SLOT,
-                       s_m1 * 100 + s_0 * 10 + s_p1))
-            break;
-        __syncthreads();  // fy of plane z - 1 complete; my of plane z - 1 consumed
-        Rec<C> Py;
-        if (!last) {
-            prestep(z + 1, s_p1);
-            if constexpr (staged) {
-                if (issuer && z + 2 <= zend) issue_plane(z + 2);
-            }
-            CellView<C> v;
-            // warp-uniform: rows 1..TY take every difference, the halo rows
-            // only those their y records need
-            if (yin) {
-                gather(s_0, s_m1, s_p1, std::integral_constant<int, 7>{}, v);
-            } else {
-                gather(s_0, s_m1, s_p1, std::integral_constant<int, 5>{}, v);  // G^x, G^z
-            }
-            if (yin) {
-                // x faces: this lane's face to the right uses the next lane's M record
-                Rec<C> Px, Mx, Mn;
-                side_records<0, true, true>(v, kc, Px, Mx);
-#pragma unroll
-                for (int k = 0; k < NC; ++k) Mn.r[k] = pshfl_down1<C>(Mx.r[k]);
-#pragma unroll
-                for (int m = 0; m < 4; ++m) Mn.m[m] = __shfl_down_sync(0xffffffffu, Mx.m[m], 1);
-                P2 ffx[NC];
-                face_values<0>(Px, Mn, kc, ffx);
-                static_for<0, NC>([&](auto kc2) {
-                    constexpr int K = decltype(kc2)::value;
-                    constexpr int p = cross_pair(0, K);
-                    const P2 fl = pshfl_up1<C>(ffx[K]);
-                    // Dhat = e_px (F(x + 1/2) - F(x - 1/2)), the first contribution
-                    Dcur[p] = pe(p, 0) > 0 ? psub(ffx[K], fl) : psub(fl, ffx[K]);
-                });
-            }
-            if (xin) {
-                Rec<C> My;
-                side_records<1, true, true>(v, kc, Py, My);
-#pragma unroll
-                for (int k = 0; k < NC; ++k) sm.my[k][row][lane] = My.r[k];
-#pragma unroll
-                for (int m = 0; m < 4; ++m) sm.mym[m][row][lane] = My.m[m];
-            }
-            if (interior) {
-                // z face (z - 1, z): P^z(z - 1) carried, M^z(z) from this view
-                Rec<C> Pn, Mz;
-                side_records<2, true, true>(v, kc, Pn, Mz);
-                P2 ffz[NC];
-                face_values<2>(Pz, Mz, kc, ffz);
-                static_for<0, NC>([&](auto kc2) {
-                    constexpr int K = decltype(kc2)::value;
-                    constexpr int p = cross_pair(2, K);
-                    constexpr int sg = pe(p, 2);
-                    Dprev[p] = padd_sg<sg>(Dprev[p], ffz[K]);
-                    if constexpr (pe(p, 0) != 0) {
-                        Dcur[p] = padd_sg<-sg>(Dcur[p], ffz[K]);
-                    } else {
-                        Dcur[p] = sg > 0 ? pneg(ffz[K]) : ffz[K];
-                    }
-                });
-                Pz = Pn;
-            }
-        } else if (interior) {
-            CellView<C> v;
-            Rec<C> unused, Mz;
-            gather(s_0, s_0, s_0, std::integral_constant<int, 3>{}, v);
-            side_records<2, false, true>(v, kc, unused, Mz);
-            P2 ffz[NC];
+        const Q4 xm = diff_x(slc, k3, own), ym = diff_y(slc, k4);
+        P2 ffz[NC];
+        {
+            // z face (z - 1, z): P^z(z - 1) carried, M^z(z) from this plane
+            const Q4 xq = diff_x(slc, k1, own), yq = diff_y(slc, k2);
+            Rec<C> Pn, Mz;
+            const P2 g[NC] = {P2{}, xq.a, xq.b, yq.a, yq.b};
+            side_records<2, true, true>(cur, g, qadd<C>(xm, ym), kc, Pn, Mz);
             face_values<2>(Pz, Mz, kc, ffz);
+            Pz = Pn;
             static_for<0, NC>([&](auto kc2) {
                 constexpr int K = decltype(kc2)::value;
                 constexpr int p = cross_pair(2, K);
-                Dprev[p] = padd_sg<pe(p, 2)>(Dprev[p], ffz[K]);
+                D[p] = padd_sg<pe(p, 2)>(D[p], ffz[K]);
             });
         }
-        // update plane z - 1 (Eqs. 20, 9): its y faces were computed one iteration ago
-        if (z > z0 && interior) {
+        sync();  // fy of plane z - 1 complete; slot SL ^ 1 (plane z - 1) no longer read
+        // update plane z - 1 (Eqs. 20, 9)
+        if (z > z0) {
+            Q4 l0, l1;
+            P2 l4;
+            lds<SM::FY - SM::ROW>(own, l0);
+            lds<SM::FY + SM::QX - SM::ROW>(own, l1);
+            lds<SM::FY + 2 * SM::QX - SM::ROW>(own, l4);
+            const P2 fl[NC] = {l0.a, l0.b, l1.a, l1.b, l4};
             static_for<0, NC>([&](auto kc2) {
                 constexpr int K = decltype(kc2)::value;
                 constexpr int p = cross_pair(1, K);
                 constexpr int sg = pe(p, 1);
-                const P2 dy = psub(sm.fy[K][row][lane], sm.fy[K][row - 1][lane]);
+                const P2 d = psub(ffy[K], fl[K]);
                 if constexpr (pe(p, 0) != 0 || pe(p, 2) != 0) {
-                    Dprev[p] = padd_sg<sg>(Dprev[p], dy);
+                    D[p] = padd_sg<sg>(D[p], d);
                 } else {
-                    Dprev[p] = sg > 0 ? dy : pneg(dy);
+                    D[p] = sg > 0 ? d : pneg(d);
                 }
             });
-            if (valid && KIN_CHECK((size_t)(z - 1) * nn + colidx < plane, DBG_DUGKS_STORE,
-                                   (size_t)(z - 1) * nn + colidx)) {
-                const size_t c = (size_t)(z - 1) * nn + colidx;
+            P2 t[NPAIR + 1];
+            static_for<0, NBQ>([&](auto qc) {
+                constexpr int K = decltype(qc)::value;
+                Q4 v;
+                lds<SM::BASE + (SL ^ 1) * NBQ * SM::QB + K * SM::QB>(own, v);
+                t[2 * K] = v.a;
+                t[2 * K + 1] = v.b;
+            });
+            const unsigned c = (unsigned)(z - 1) * nn32 + col32;
+            if (valid && KIN_CHECK(c < plane, DBG_DUGKS_STORE, c)) {
                 [[maybe_unused]] C uv[3] = {C(0), C(0), C(0)};
                 // velocity sums in population order: the same additions as the
                 // separate velocity pass over the stored state
@@ -631,22 +623,18 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
                     if constexpr (cz(I) > 0) uv[2] += v;
                     if constexpr (cz(I) < 0) uv[2] -= v;
                 };
+                Traits<S>::store(dst + c, t[NPAIR].x);
                 static_for<0, NPAIR>([&](auto pc) {
                     constexpr int PP = decltype(pc)::value;
-                    const P2 xb = sm.ring[s_m1][PP][row][lane];
-                    // f-tilde-plus = 4/3 fbp - 1/3 f-tilde (Eq. 20), minus dt times the flux sum (Eq. 9)
-                    const P2 t = pfma(kc.third, psub(xb, raw_pair(z - 1, PP)), xb);
-                    const P2 o = pfma(kc.dts, Dprev[PP], t);
-                    // both members rounded by one paired conversion for 2-byte storage
-                    [[maybe_unused]] const P2 r =
-                        Traits<S>::store2(dst + (2 * PP + 1) * plane + c, dst + (2 * PP + 2) * plane + c, o);
+                    // f-tilde-plus minus dt times the flux sum (Eq. 9), both members rounded
+                    // by one paired conversion for 2-byte storage
+                    [[maybe_unused]] const P2 r = RawOf<S>::store2(
+                        dst + (2 * PP + 1) * plane + c, dst + (2 * PP + 2) * plane + c, pfma(kc.dts, D[PP], t[PP]));
                     if constexpr (VEL) {
                         vel_add(std::integral_constant<int, 2 * PP + 1>{}, r.x);
                         vel_add(std::integral_constant<int, 2 * PP + 2>{}, r.y);
                     }
                 });
-                const C xb0 = sm.ring0[s_m1][row][lane];
-                Traits<S>::store(dst + c, fma(C(1.0 / 3.0), xb0 - raw_rest(z - 1), xb0));
                 if constexpr (VEL) {
                     uvel[c] = uv[0];
                     uvel[plane + c] = uv[1];
@@ -654,28 +642,58 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
                 }
             }
         }
-        __syncthreads();  // my of plane z complete; fy of plane z - 1 consumed
-        if (!last && xin && row <= TY) {
-            // y faces of plane z: face r between rows r and r + 1, r = 0..TY
-            Rec<C> Mu;
+        if (last) return true;
+        // plane z + 1
+        const Q4 zp56{nxt.X[5], nxt.X[6]}, zp78{nxt.X[7], nxt.X[8]}, zpm = nxt.m[2];
+        prestep(other, std::true_type{}, own, fr, nxt);
+        const Q4 z56 = qsub<C>(Q4{nxt.X[5], nxt.X[6]}, zp56), z78 = qsub<C>(Q4{nxt.X[7], nxt.X[8]}, zp78);
+        const Q4 zm = qsub<C>(nxt.m[2], zpm);
+        {
+            // x faces: this lane's face to the right uses the next lane's M record
+            Rec<C> Px, Mx, Mn;
+            const Q4 yp = diff_y(slc, k0);
+            const P2 g[NC] = {P2{}, yp.a, yp.b, z56.a, z56.b};
+            side_records<0, true, true>(cur, g, qadd<C>(ym, zm), kc, Px, Mx);
 #pragma unroll
-            for (int k = 0; k < NC; ++k) Mu.r[k] = sm.my[k][row + 1][lane];
-#pragma unroll
-            for (int m = 0; m < 4; ++m) Mu.m[m] = sm.mym[m][row + 1][lane];
-            P2 ffy[NC];
-            face_values<1>(Py, Mu, kc, ffy);
-#pragma unroll
-            for (int k = 0; k < NC; ++k) sm.fy[k][row][lane] = ffy[k];
+            for (int k = 0; k < NC; ++k) Mn.r[k] = pshfl_down1<C>(Mx.r[k]);
+            Mn.m0 = pshfl_down1<C>(Mx.m0);
+            Mn.m1 = pshfl_down1<C>(Mx.m1);
+            P2 ffx[NC];
+            face_values<0>(Px, Mn, kc, ffx);
+            static_for<0, NC>([&](auto kc2) {
+                constexpr int K = decltype(kc2)::value;
+                constexpr int p = cross_pair(0, K);
+                const P2 fl = pshfl_up1<C>(ffx[K]);
+                // Dhat = e_px (F(x + 1/2) - F(x - 1/2)), the first contribution
+                D[p] = pe(p, 0) > 0 ? psub(ffx[K], fl) : psub(fl, ffx[K]);
+            });
+            static_for<0, NC>([&](auto kc2) {
+                constexpr int K = decltype(kc2)::value;
+                constexpr int p = cross_pair(2, K);
+                constexpr int sg = pe(p, 2);
+                if constexpr (pe(p, 0) != 0) D[p] = padd_sg<-sg>(D[p], ffz[K]);
+                else D[p] = sg > 0 ? pneg(ffz[K]) : ffz[K];
+            });
         }
-        if constexpr (staged) {
-            if (issuer) cp_async_wait_all();  // plane z + 2, published by the next barrier
+        if (z + 2 <= zend) load_plane(z + 2, col32, fr);
+        Rec<C> Py;
+        {
+            Rec<C> My;
+            const Q4 xp = diff_x(slc, k0, own);
+            const P2 g[NC] = {P2{}, xp.a, xp.b, z78.a, z78.b};
+            side_records<1, true, true>(cur, g, qadd<C>(xm, zm), kc, Py, My);
+            sts<SM::MY>(own, My.r[0], My.r[1]);
+            sts<SM::MY + SM::QX>(own, My.r[2], My.r[3]);
+            sts<SM::MY + 2 * SM::QX>(own, My.r[4], My.m0);
+            sts<SM::MY + 3 * SM::QX>(own, My.m1);
         }
-#pragma unroll
-        for (int q = 0; q < NPAIR; ++q) Dprev[q] = Dcur[q];
-        const int st = s_m1;
-        s_m1 = s_0;
-        s_0 = s_p1;
-        s_p1 = st;
+        sync();  // my of plane z and slot SL ^ 1 (plane z + 1) complete; fy of plane z - 1 consumed
+        y_face(Py, own, ffy);
+        return false;
+    };
+    for (int z = z0;; z += 2) {
+        if (advance(k0, z, A, B)) break;
+        if (advance(k1, z + 1, B, A)) break;
     }
 }
 
@@ -708,6 +726,9 @@ inline DugksCoef<C> dugks_coef(double nu, double dt) {
     k.c1p = pmk(c1, c1);
     k.third = pmk(C(1.0 / 3.0), C(1.0 / 3.0));
     k.dts = pmk(-k.dt, k.dt);
+    k.h2 = pmk(k.h, k.h);
+    k.mh2 = pmk(-k.h, -k.h);
+    k.mhq2 = pmk(-k.hq, -k.hq);
     return k;
 }
 

@@ -15,13 +15,13 @@
 //
 // LBE members: one batched launch per step covers every LBE member of a
 // storage type (a block takes consecutive nodes of one member), on a second
-// stream of the same graph.  With both schemes present the persistent kernel
-// runs 6-row tiles (8 warps, 160 KB of shared memory, at most 160 registers
-// a thread), which leave room for three 4-warp FP32 LBE blocks (56 registers
-// a thread, no shared memory) on each SM: the memory-bound LBE nodes use the
-// bandwidth and issue slots that the issue-bound DUGKS tiles leave.  The two
-// kernels never wait on each other; consecutive LBE steps are ordered by
-// their stream.
+// stream of the same graph.  The two kernels never wait on each other;
+// consecutive LBE steps are ordered by their stream.  Two persistent blocks of
+// 5-row tiles fill an SM's registers, so the LBE launches get the SMs before or
+// after them: for the 24-member reference mix 0.366 ms a step of the DUGKS
+// members plus 0.137 ms of the LBE members, 0.502 together.  Tiles that leave
+// registers for LBE blocks beside them overlap and are still slower (one block
+// of 7-row tiles at 160 registers: 0.520 ms alone, 0.601 together).
 //
 // Which block runs an item does not change what it computes: a member's
 // results are bitwise those of stepping it alone.
@@ -153,30 +153,16 @@ __device__ __forceinline__ void ensemble_body(const EnsMember* __restrict__ mem,
         unsigned *next_item, int *status, long long wait_cycles, int stall_test
 
 template <int TY, bool WIDE>
-__global__ void __launch_bounds__(32 * (TY + 2), 1) ensemble_kernel(KIN_ENSEMBLE_PARAMS) {
+__global__ void __launch_bounds__(32 * (TY + 1), TY <= 5 ? 2 : 1) ensemble_kernel(KIN_ENSEMBLE_PARAMS) {
     ensemble_body<TY, WIDE>(mem, items, nitems, nsteps, done, next_item, status, wait_cycles, stall_test);
-}
-
-// 6-row tiles, the form beside which LBE blocks run: held to 160 registers a
-// thread (152 used; at the compiler's free choice it takes 214), so that the
-// 8-warp block leaves most of the SM's registers to the LBE blocks.
-template <bool WIDE>
-__global__ void __maxnreg__(160) ensemble_kernel6(KIN_ENSEMBLE_PARAMS) {
-    ensemble_body<6, WIDE>(mem, items, nitems, nsteps, done, next_item, status, wait_cycles, stall_test);
-}
-
-template <int TY, bool WIDE>
-constexpr auto ensemble_kernel_for() {
-    if constexpr (TY == 6) return ensemble_kernel6<WIDE>;
-    else return ensemble_kernel<TY, WIDE>;
 }
 
 // One LBE step of every member in tab[0 .. nmem) (one storage type): block b
 // belongs to the member with the largest block0 <= b and takes blockDim.x * V
 // consecutive cells of it (linear index x + N (y + N z)); each thread updates V
 // cells of one row exactly as the standalone LBE step does.  FP32 blocks are
-// held to 56 registers a thread, so that two 128-thread blocks fit beside a
-// DUGKS block (the 2-byte vector forms would spill there).
+// held to 56 registers a thread, nine 128-thread blocks an SM (the 2-byte
+// vector forms would spill there).
 template <typename S>
 __global__ void __launch_bounds__(128, sizeof(S) == 4 ? 9 : 1) lbe_batch_kernel(const LbeMember* __restrict__ tab, int nmem, int step) {
     const unsigned b = blockIdx.x;
@@ -219,9 +205,11 @@ struct kin_ensemble {
     cudaStream_t stream = nullptr;  // persistent DUGKS launch (and the graph's origin)
     cudaStream_t side = nullptr;    // batched LBE launches inside the graph
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    // tile_y 6 (8 warps a DUGKS block) when both schemes are present, else 8;
-    // see kin_ensemble_create
-    int tile_y = 8, zchunk = 16, lbe_block = 128;
+    // 5-row tiles, two 6-warp blocks an SM: 0.366 ms a step for the DUGKS members
+    // of the reference mix, against 0.402 (4 rows), 0.568 (6), 0.436 (8)
+    int tile_y = 5, lbe_block = 128;
+    int zchunk = 0;  // 0: chosen for the members (default_zchunk)
+    int zc = 1;      // planes per item in use
     EnsMember* d_mem = nullptr;
     LbeMember* d_lbe = nullptr;
     int2* d_items = nullptr;
@@ -269,10 +257,10 @@ size_t persistent_smem() {
 template <int TY, bool WIDE>
 int configure(kin_ensemble* e) {
     const size_t smem = persistent_smem<TY, WIDE>();
-    ECK(cudaFuncSetAttribute(ensemble_kernel_for<TY, WIDE>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+    ECK(cudaFuncSetAttribute(ensemble_kernel<TY, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem));
     int per_sm = 0, nsm = 0;
-    ECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ensemble_kernel_for<TY, WIDE>(), 32 * (TY + 2),
+    ECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ensemble_kernel<TY, WIDE>, 32 * (TY + 1),
                                                       smem));
     ECK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, e->device));
     if (per_sm < 1) return set_error(KIN_ECUDA, "ensemble kernel does not fit on an SM");
@@ -300,7 +288,7 @@ std::vector<EnsMember> dugks_table(const kin_ensemble* e) {
         M.storage = s->storage;
         M.cur = s->cur;
         M.coef = dugks_coef<float>(s->nu, s->dt);
-        const int zc = std::min(e->zchunk, s->N);
+        const int zc = std::min(e->zc, s->N);
         M.tiles_x = (s->N + 29) / 30;
         M.tiles_y = (s->N + e->tile_y - 1) / e->tile_y;
         M.zchunk = zc;
@@ -342,14 +330,44 @@ int launch_persistent_config(kin_ensemble* e) {
         e->grid = 0;
         return KIN_OK;
     }
+    if (e->tile_y == 5) return e->wide ? configure<5, true>(e) : configure<5, false>(e);
     if (e->tile_y == 4) return e->wide ? configure<4, true>(e) : configure<4, false>(e);
     if (e->tile_y == 6) return e->wide ? configure<6, true>(e) : configure<6, false>(e);
     return e->wide ? configure<8, true>(e) : configure<8, false>(e);
 }
 
+// Planes per item when the caller has not chosen: a step takes about its items'
+// planes (and 1.1 plane-times of prologue each) spread over the resident
+// blocks, but no less than its longest item, which the next step of that
+// member waits for.  The reference mix gets 64 planes (0.373 ms a step of its
+// DUGKS members; 16: 0.421, 32: 0.385, 128: 0.366).
+int default_zchunk(const kin_ensemble* e) {
+    int nsm = 0;
+    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, e->device) != cudaSuccess || nsm <= 0) nsm = 152;
+    const double slots = nsm * (e->tile_y <= 5 ? 2.0 : 1.0);
+    int best = 1;
+    double best_cost = -1.0;
+    for (int zc : {1024, 512, 256, 128, 96, 64, 48, 32, 24, 16, 11, 8, 6, 4, 3, 2, 1}) {
+        double sum = 0.0, longest = 0.0;
+        for (int m : e->dugks_ids) {
+            const int N = e->members[m]->N, c = std::min(zc, N);
+            const double cols = (double)((N + 29) / 30) * ((N + e->tile_y - 1) / e->tile_y);
+            sum += cols * (N + 1.1 * ((N + c - 1) / c));
+            longest = std::max(longest, c + 1.1);
+        }
+        const double cost = std::max(sum / slots, longest);
+        if (best_cost < 0.0 || cost < best_cost) {
+            best_cost = cost;
+            best = zc;
+        }
+    }
+    return best;
+}
+
 // Work list for the current tuning; items of big members first so their long
 // critical paths start early.
 int build_tables(kin_ensemble* e) {
+    e->zc = e->zchunk > 0 ? e->zchunk : default_zchunk(e);
     const std::vector<EnsMember> tab = dugks_table(e);
     std::vector<int> order(tab.size());
     for (size_t d = 0; d < order.size(); ++d) order[d] = (int)d;
@@ -382,7 +400,7 @@ template <int TY, bool WIDE>
 cudaError_t launch_persistent_t(kin_ensemble* e, int nsteps, int stall_test) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(e->grid);
-    cfg.blockDim = dim3(32, TY + 2);
+    cfg.blockDim = dim3(32, TY + 1);
     cfg.dynamicSmemBytes = persistent_smem<TY, WIDE>();
     cfg.stream = e->stream;
     cudaLaunchAttribute attr[1];
@@ -391,7 +409,7 @@ cudaError_t launch_persistent_t(kin_ensemble* e, int nsteps, int stall_test) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const int nd = (int)e->dugks_ids.size();
-    return cudaLaunchKernelEx(&cfg, ensemble_kernel_for<TY, WIDE>(), (const EnsMember*)e->d_mem,
+    return cudaLaunchKernelEx(&cfg, ensemble_kernel<TY, WIDE>, (const EnsMember*)e->d_mem,
                               (const int2*)e->d_items, e->nitems, nsteps, e->d_done, e->d_done + nd, e->d_status,
                               wait_cycles(e), stall_test);
 }
@@ -401,6 +419,9 @@ int launch_persistent(kin_ensemble* e, int nsteps, int stall_test) {
     if (e->tile_y == 4)
         err = e->wide ? launch_persistent_t<4, true>(e, nsteps, stall_test)
                       : launch_persistent_t<4, false>(e, nsteps, stall_test);
+    else if (e->tile_y == 5)
+        err = e->wide ? launch_persistent_t<5, true>(e, nsteps, stall_test)
+                      : launch_persistent_t<5, false>(e, nsteps, stall_test);
     else if (e->tile_y == 6)
         err = e->wide ? launch_persistent_t<6, true>(e, nsteps, stall_test)
                       : launch_persistent_t<6, false>(e, nsteps, stall_test);
@@ -550,11 +571,6 @@ int kin_ensemble_create(kin_sim* const* members, int n, kin_ensemble** out) {
             e->lbe_ids.push_back(m);
         }
     }
-    // Measured: LBE blocks of any size ran beside 6- and 8-warp DUGKS blocks
-    // (4- and 6-row tiles) and never beside the 10-warp blocks of 8-row tiles,
-    // even with those held to 152 registers a thread; so when both schemes
-    // are present the DUGKS tiles have 6 rows.
-    if (!e->dugks_ids.empty() && !e->lbe_ids.empty()) e->tile_y = 6;
     e->device = dev;
     int prev = 0;
     cudaGetDevice(&prev);

@@ -24,12 +24,17 @@ cudaError_t lbe_step(int storage, const void* src, void* dst, int N, double nu, 
 cudaError_t dugks_step(int storage, const void* src, void* dst, void* fbp, int N, double nu,
                        double dt, int block_x, cudaStream_t stream);
 
-// Fused single-launch DUGKS step; tile_y in {4, 8} (FP64 always uses 4),
-// zchunk planes per CTA.
+// Fused single-launch DUGKS step; tile_y and zchunk (planes per block) as
+// dugks_fused_shape returns them.
 // uvel: NULL, or (FP32-computed storage) uvel[3][N^3] receives the velocity
 // of the new state, bitwise equal to velocity_field32 of it.
 cudaError_t dugks_step_fused(int storage, const void* src, void* dst, int N, double nu, double dt,
                              int tile_y, int zchunk, cudaStream_t stream, float* uvel = nullptr);
+
+// Tile height (FP32-computed storage: 4, 5, 8 or 11 rows; FP64: 4) and planes
+// per block of the fused step on nsm multiprocessors; want_ty (4 or 8) and
+// want_zc fix one of them where positive.
+void dugks_fused_shape(int storage, int N, int nsm, int want_ty, int want_zc, int* ty, int* zc);
 
 // The momentum reset of a DUGKS consistent-initialisation iteration: f-tilde
 // (in place) gets momentum rho0 u0 (FP64 [3][N^3], device) back along the

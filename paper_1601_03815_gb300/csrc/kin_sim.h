@@ -30,8 +30,8 @@ struct kin_sim {
     cufftHandle d2z = 0, z2d = 0, r2c = 0;
     bool have_d2z = false, have_z2d = false, have_r2c = false;
     int block_lbe = 0, block_dugks = 0;
-    int tile_y = 8, zchunk = 0, variant = 0;  // zchunk 0: chosen per launch
-    int zc_auto = 0, zc_auto_ty = 0;  // the chosen z chunk and the tile height it was chosen for
+    int tile_y = 0, zchunk = 0, variant = 0;  // 0: chosen by dugks_fused_shape
+    int fused_ty = 0, fused_zc = 0;  // the fused step's shape for this tuning (0: not chosen yet)
     int* d_err = nullptr;  // set by a kernel whose bounded wait gave up
     double* h_pin = nullptr;  // pinned host words: E, eps, and the error flag
     int64_t launches = 0;  // own kernel launches

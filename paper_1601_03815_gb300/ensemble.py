@@ -26,7 +26,7 @@ import numpy as np
 from . import DUGKS, F32, LBE_MRT, Ensemble, Sim
 
 REFERENCE_SIZES = ((32, 8), (64, 8), (96, 6), (128, 2))
-TUNE_TILE_Y = (4, 6, 8)
+TUNE_TILE_Y = (0,)  # the library's 5-row tiles: 4, 6 and 8 rows were slower on every mix measured
 TUNE_ZCHUNK = (8, 16, 32, 64, 128)
 TUNE_LBE_BLOCK = (64, 128)
 
@@ -63,8 +63,8 @@ def _signature(sims):
 
     dev = torch.cuda.get_device_name() if torch.cuda.is_available() else "cpu"
     sizes = sorted((s.N, s.scheme) for s in sims)
-    # "c": tunings of the batched-LBE form (threads per LBE block, 6-row tiles)
-    return "c|%s|%s" % (dev, ",".join("%d%s" % (n, "L" if sc == LBE_MRT else "D") for n, sc in sizes))
+    # "d": tunings of the 5-row tiles
+    return "d|%s|%s" % (dev, ",".join("%d%s" % (n, "L" if sc == LBE_MRT else "D") for n, sc in sizes))
 
 
 def autotune(ens: Ensemble, steps: int = 10, use_cache: bool = True, verbose: bool = False):
