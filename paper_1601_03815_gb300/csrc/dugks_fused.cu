@@ -4,6 +4,7 @@
 
 #include "dugks_tile.cuh"
 #include "kin_internal.h"
+#include "kin_launch.cuh"
 
 namespace kin {
 
@@ -19,6 +20,7 @@ __global__ void __launch_bounds__(32 * (TY + 1), sizeof(typename Traits<S>::C) =
     dugks_fused_kernel(const S* __restrict__ src, S* __restrict__ dst, int N, int zchunk,
                        DugksCoef<typename Traits<S>::C> kc, float* __restrict__ uvel) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    grid_begin();
     dugks_tile<S, TY, VEL>(src, dst, N, blockIdx.x, blockIdx.y, blockIdx.z, zchunk, kc, smem_raw, uvel);
 }
 
@@ -43,8 +45,8 @@ static cudaError_t launch_fused_t(const void* src, void* dst, int N, int zchunk,
     if (zchunk > N) zchunk = N;
     dim3 block(32, TY + 1);
     dim3 grid((N + 29) / 30, (N + TY - 1) / TY, (N + zchunk - 1) / zchunk);
-    dugks_fused_kernel<S, TY, VEL><<<grid, block, smem, stream>>>((const S*)src, (S*)dst, N, zchunk, k, uvel);
-    return cudaGetLastError();
+    return launch_next(dugks_fused_kernel<S, TY, VEL>, grid, block, smem, stream, (const S*)src, (S*)dst, N, zchunk, k,
+                       uvel);
 }
 
 template <typename S, bool VEL>

@@ -361,7 +361,7 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
     const int lane = opaque((int)threadIdx.x);
     const bool halo = threadIdx.y == TY;
     const int row = opaque(halo ? 0 : (int)threadIdx.y + 1);
-    if (!KIN_CHECK((int)threadIdx.y <= TY && lane < 32, DBG_DUGKS_ROW, threadIdx.y)) return;
+    (void)KIN_CHECK((int)threadIdx.y <= TY && lane < 32, DBG_DUGKS_ROW, threadIdx.y);
     const unsigned own = opaque((unsigned)__cvta_generic_to_shared(smem_raw) + row * SM::ROW + lane * (int)sizeof(Q4));
     const int z0 = bz * zchunk;
     const int zend = min(z0 + zchunk, N);

@@ -1,6 +1,7 @@
 // Standalone launch of the MRT-LBE step (node update in lbe_node.cuh).
 // HBM traffic per node: 19 loads + 19 stores of the storage type.
 #include "kin_internal.h"
+#include "kin_launch.cuh"
 #include "lbe_node.cuh"
 
 #include <algorithm>
@@ -13,6 +14,7 @@ __global__ void __launch_bounds__(256) lbe_step_kernel(const S* __restrict__ src
                                                        S* __restrict__ dst, int N, size_t plane,
                                                        MrtRates<typename Traits<S>::C> rates) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    grid_begin();
     if (x >= N) return;
     lbe_node<S, false>(src, dst, N, plane, x, blockIdx.y, blockIdx.z, rates);
 }
@@ -21,6 +23,7 @@ template <typename S, int V>
 __global__ void __launch_bounds__(256) lbe_stepv_kernel(const S* __restrict__ src, S* __restrict__ dst,
                                                         int N, size_t plane, MrtRates<float> rates) {
     const int x = V * (blockIdx.x * blockDim.x + threadIdx.x);
+    grid_begin();
     if (x >= N) return;
     lbe_vnode<S, V>(src, dst, N, plane, x, blockIdx.y, blockIdx.z, rates);
 }
@@ -33,6 +36,7 @@ template <typename S>
 __global__ void __maxnreg__(96) lbe_stepv4_kernel(const S* __restrict__ src, S* __restrict__ dst, int N,
                                                   size_t plane, MrtRates<float> rates) {
     const int x = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+    grid_begin();
     if (x >= N) return;
     lbe_vnode4p<S>(src, dst, N, plane, x, blockIdx.y, blockIdx.z, rates);
 }
@@ -44,9 +48,9 @@ static cudaError_t launch_lbe_v(const S* src, S* dst, int N, const MrtRates<floa
     int b = bx > 0 ? std::min(bx, 256) : 128;
     if (b > nv) b = ((nv + 31) / 32) * 32;
     dim3 block(b), grid((nv + b - 1) / b, N, N);
-    if constexpr (V == 4) lbe_stepv4_kernel<S><<<grid, block, 0, stream>>>(src, dst, N, (size_t)N * N * N, r);
-    else lbe_stepv_kernel<S, V><<<grid, block, 0, stream>>>(src, dst, N, (size_t)N * N * N, r);
-    return cudaGetLastError();
+    const size_t plane = (size_t)N * N * N;
+    if constexpr (V == 4) return launch_next(lbe_stepv4_kernel<S>, grid, block, 0, stream, src, dst, N, plane, r);
+    else return launch_next(lbe_stepv_kernel<S, V>, grid, block, 0, stream, src, dst, N, plane, r);
 }
 
 template <typename S>
@@ -62,9 +66,7 @@ static cudaError_t launch_lbe(const void* src, void* dst, int N, double nu, int 
     if (bx > 256) bx = 256;  // the kernel's launch bounds
     if (bx > N) bx = ((N + 31) / 32) * 32;
     dim3 block(bx), grid((N + bx - 1) / bx, N, N);
-    lbe_step_kernel<S><<<grid, block, 0, stream>>>((const S*)src, (S*)dst, N,
-                                                    (size_t)N * N * N, r);
-    return cudaGetLastError();
+    return launch_next(lbe_step_kernel<S>, grid, block, 0, stream, (const S*)src, (S*)dst, N, (size_t)N * N * N, r);
 }
 
 // One iteration of the consistent initialisation (Sec. IV.A, after Mei et

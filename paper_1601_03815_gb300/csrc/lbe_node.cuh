@@ -42,8 +42,7 @@ __device__ __forceinline__ void lbe_gather(const S* __restrict__ src, int N, siz
         constexpr int I = decltype(ic)::value;
         const int idx = xo[1 - cx(I)] + yo[1 - cy(I)] + zo[1 - cz(I)];
         if (!KIN_CHECK(idx >= 0 && (size_t)idx < plane, DBG_LBE_LOAD, idx)) f[I] = C(0);
-        else if constexpr (COHERENT) f[I] = (C)src[(size_t)I * plane + idx];
-        else f[I] = Traits<S>::load(src + (size_t)I * plane + idx);
+        else f[I] = Traits<S>::load_l2(src + (size_t)I * plane + idx);
     });
 }
 
@@ -139,11 +138,11 @@ struct Pair2<__nv_bfloat16> {
 template <typename S, int V>
 __device__ __forceinline__ void vload(const S* p, float (&o)[V]) {
     if constexpr (V == 2) {
-        const float2 a = Pair2<S>::unpack(__ldg(reinterpret_cast<const unsigned*>(p)));
+        const float2 a = Pair2<S>::unpack(__ldcg(reinterpret_cast<const unsigned*>(p)));
         o[0] = a.x;
         o[1] = a.y;
     } else {
-        const uint2 w = __ldg(reinterpret_cast<const uint2*>(p));
+        const uint2 w = __ldcg(reinterpret_cast<const uint2*>(p));
         const float2 a = Pair2<S>::unpack(w.x), b = Pair2<S>::unpack(w.y);
         o[0] = a.x;
         o[1] = a.y;
@@ -202,16 +201,16 @@ __device__ __forceinline__ void lbe_vnode4p(const S* __restrict__ src, S* __rest
         uint2 own = make_uint2(0u, 0u);
         if (KIN_CHECK((size_t)(yo[1 - cy(I)] + zo[1 - cz(I)]) + x + 4 <= plane && xm < N && xp < N, DBG_LBE_LOAD,
                       yo[1 - cy(I)] + zo[1 - cz(I)] + x))
-            own = __ldg(reinterpret_cast<const uint2*>(row + x));
+            own = __ldcg(reinterpret_cast<const uint2*>(row + x));
         if constexpr (cx(I) == 0) {
             w[I][0] = own.x;
             w[I][1] = own.y;
         } else if constexpr (cx(I) > 0) {  // cells x - 1 .. x + 2
-            const unsigned l = __ldg(reinterpret_cast<const unsigned short*>(row + xm));
+            const unsigned l = __ldcg(reinterpret_cast<const unsigned short*>(row + xm));
             w[I][0] = __byte_perm(l, own.x, 0x5410);
             w[I][1] = __byte_perm(own.x, own.y, 0x5432);
         } else {  // cells x + 1 .. x + 4
-            const unsigned r = __ldg(reinterpret_cast<const unsigned short*>(row + xp));
+            const unsigned r = __ldcg(reinterpret_cast<const unsigned short*>(row + xp));
             w[I][0] = __byte_perm(own.x, own.y, 0x5432);
             w[I][1] = __byte_perm(own.y, r, 0x5432);
         }
@@ -253,13 +252,13 @@ __device__ __forceinline__ void lbe_vnode(const S* __restrict__ src, S* __restri
 #pragma unroll
             for (int k = 0; k < V; ++k) f[k][I] = own[k];
         } else if constexpr (cx(I) > 0) {
-            f[0][I] = Traits<S>::load(row + xm);
+            f[0][I] = Traits<S>::load_l2(row + xm);
 #pragma unroll
             for (int k = 1; k < V; ++k) f[k][I] = own[k - 1];
         } else {
 #pragma unroll
             for (int k = 0; k < V - 1; ++k) f[k][I] = own[k + 1];
-            f[V - 1][I] = Traits<S>::load(row + xp);
+            f[V - 1][I] = Traits<S>::load_l2(row + xp);
         }
     });
 #pragma unroll
