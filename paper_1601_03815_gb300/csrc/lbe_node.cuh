@@ -28,9 +28,9 @@ inline MrtRates<C> lbe_rates(double nu) {
     return r;
 }
 
-// COHERENT selects plain loads (data written earlier in the same launch by
-// other thread blocks, read after an acquire) instead of the read-only path.
-template <typename S, bool COHERENT>
+// Loads go to L2: the step may start while the kernel that wrote src ends
+// (kin_launch.cuh), so not through the read-only path; 256^3 measures the same.
+template <typename S>
 __device__ __forceinline__ void lbe_gather(const S* __restrict__ src, int N, size_t plane, int x, int y,
                                            int z, typename Traits<S>::C (&f)[Q]) {
     using C = typename Traits<S>::C;
@@ -55,43 +55,16 @@ __device__ __forceinline__ void lbe_scatter(S* __restrict__ dst, int N, size_t p
     for (int i = 0; i < Q; ++i) Traits<S>::store(dst + (size_t)i * plane + c, f[i]);
 }
 
-template <typename S, bool COHERENT>
+template <typename S>
 __device__ __forceinline__ void lbe_node(const S* __restrict__ src, S* __restrict__ dst, int N,
                                          size_t plane, int x, int y, int z,
                                          const MrtRates<typename Traits<S>::C>& rates) {
     using C = typename Traits<S>::C;
     C f[Q];
-    lbe_gather<S, COHERENT>(src, N, plane, x, y, z, f);
+    lbe_gather<S>(src, N, plane, x, y, z, f);
     C drho, jx, jy, jz;
     mrt_collide(f, rates, drho, jx, jy, jz);
     lbe_scatter<S>(dst, N, plane, x, y, z, f);
-}
-
-// K nodes (cells c[0..K-1], linear index x + N (y + N z)) with every gather
-// issued before the first collision, so that a thread keeps K times the loads
-// in flight (used where few warps share an SM).
-template <int K, typename S, bool COHERENT>
-__device__ __forceinline__ void lbe_nodes(const S* __restrict__ src, S* __restrict__ dst, int N,
-                                          size_t plane, const int (&c)[K],
-                                          const MrtRates<typename Traits<S>::C>& rates) {
-    using C = typename Traits<S>::C;
-    C f[K][Q];
-    int xyz[K][3];
-    const int nn = N * N;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        xyz[k][2] = c[k] / nn;
-        xyz[k][1] = (c[k] - xyz[k][2] * nn) / N;
-        xyz[k][0] = c[k] - xyz[k][2] * nn - xyz[k][1] * N;
-        lbe_gather<S, COHERENT>(src, N, plane, xyz[k][0], xyz[k][1], xyz[k][2], f[k]);
-    }
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        C drho, jx, jy, jz;
-        mrt_collide(f[k], rates, drho, jx, jy, jz);
-    }
-#pragma unroll
-    for (int k = 0; k < K; ++k) lbe_scatter<S>(dst, N, plane, xyz[k][0], xyz[k][1], xyz[k][2], f[k]);
 }
 
 // 2-byte storage moves a cell's 19 values as 38 bytes, so one element per
