@@ -162,13 +162,20 @@ int launch_step(kin_sim* s, float* uvel = nullptr) {
     return KIN_OK;
 }
 
-// Enqueue E and eps of the current state into red_out[0..1] (device).
-int enqueue_energy_dissipation(kin_sim* s) {
+// Enqueue E and eps of the current state into red_out[0..1] (device) and, where
+// host is not NULL, into that device-accessible host memory (with_err: followed
+// by the error word).
+int enqueue_energy_dissipation(kin_sim* s, double* host, bool with_err) {
     if (int r = ensure_u(s)) return r;
+    EdSink sink;
+    sink.out = s->red_out;
+    sink.counter = reinterpret_cast<unsigned*>(s->d_err + 1);
+    sink.host = host;
+    if (with_err) sink.err = s->d_err;
     if (s->storage == ST_F64) {
         CK(velocity_field(s->storage, s->buf[s->cur], shifted(s), s->N, s->u, s->stream));
-        CK(energy_dissipation(s->u, s->N, s->nu, s->red, s->red_out, s->stream));
-        s->launches += 3;
+        CK(energy_dissipation(s->u, s->N, s->nu, s->red, sink, s->stream));
+        s->launches += 2;
     } else {
         // FP32 arithmetic per cell (FP64 on this GPU runs at a small fraction
         // of the FP32 rate), FP64 sums; the velocity pass is skipped when u32
@@ -180,10 +187,23 @@ int enqueue_energy_dissipation(kin_sim* s) {
             s->launches += 1;
             s->u32_epoch = s->epoch;
         }
-        CK(energy_dissipation32(s->u32, s->N, s->nu, s->red, s->red_out, s->stream));
-        s->launches += 2;
+        CK(energy_dissipation32(s->u32, s->N, s->nu, s->red, sink, s->stream));
+        s->launches += 1;
     }
     return KIN_OK;
+}
+
+// The address under which kernels may write doubles to this host memory, or
+// NULL: aligned page-locked memory of this process.  Looked up on every call
+// (the memory may have been released and the address reused since).
+double* device_view(double* host) {
+    if (reinterpret_cast<uintptr_t>(host) % sizeof(double)) return nullptr;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return a.type == cudaMemoryTypeHost ? static_cast<double*>(a.devicePointer) : nullptr;
 }
 
 }  // namespace
@@ -266,9 +286,9 @@ int kin_create(int N, int scheme, double nu, double Ma, double dt, int storage, 
         if (e != cudaSuccess) return bail(fail(KIN_ECUDA, "memset: %s", cudaGetErrorString(e)));
     }
     {
-        cudaError_t e = cudaMalloc(&s->d_err, sizeof(int));
+        cudaError_t e = cudaMalloc(&s->d_err, 2 * sizeof(int));
         if (e != cudaSuccess) return bail(fail(KIN_ENOMEM, "error flag: %s", cudaGetErrorString(e)));
-        e = cudaMemsetAsync(s->d_err, 0, sizeof(int), s->stream);
+        e = cudaMemsetAsync(s->d_err, 0, 2 * sizeof(int), s->stream);
         if (e != cudaSuccess) return bail(fail(KIN_ECUDA, "memset: %s", cudaGetErrorString(e)));
         e = cudaMallocHost(&s->h_pin, 4 * sizeof(double));
         if (e != cudaSuccess) return bail(fail(KIN_ENOMEM, "pinned words: %s", cudaGetErrorString(e)));
@@ -478,8 +498,11 @@ int kin_stats_async(kin_sim* s, double* out) {
     if (int r = usable(s)) return r;
     if (!out) return fail(KIN_EINVAL, "NULL output");
     DeviceGuard g(s->device);
-    if (int r = enqueue_energy_dissipation(s)) return r;
-    CK(cudaMemcpyAsync(out, s->red_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
+    // page-locked memory is written by the reduction itself (a copy of 16 bytes is
+    // a stream operation of ~4 us between two steps)
+    double* view = device_view(out);
+    if (int r = enqueue_energy_dissipation(s, view, false)) return r;
+    if (!view) CK(cudaMemcpyAsync(out, s->red_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
     return KIN_OK;
 }
 
@@ -552,10 +575,9 @@ int kin_stats(kin_sim* s, double* E, double* eps, double* Ek) {
     NvtxRange nvtx_("kin_stats");
     if (int r = usable(s)) return r;
     DeviceGuard g(s->device);
-    if (int r = enqueue_energy_dissipation(s)) return r;
-    // E, eps and the step kernels' error flag in one synchronisation
-    CK(cudaMemcpyAsync(s->h_pin, s->red_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
-    CK(cudaMemcpyAsync(s->h_pin + 2, s->d_err, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+    // E, eps and the step kernels' error flag in one synchronisation, written to
+    // the page-locked words by the reduction
+    if (int r = enqueue_energy_dissipation(s, s->h_pin, true)) return r;
     CK(cudaStreamSynchronize(s->stream));
     const double ed[2] = {s->h_pin[0], s->h_pin[1]};
     int flag = 0;
@@ -614,10 +636,13 @@ int kin_derived_stats(kin_sim* s, double* out, double* D) {
     const int N = s->N;
     const size_t n = ncell(s), nm = nmode(s);
     CK(velocity_field(s->storage, s->buf[s->cur], shifted(s), N, s->u, s->stream));
-    CK(energy_dissipation(s->u, N, s->nu, s->red, s->red_out, s->stream));
-    double ed[2];
-    CK(cudaMemcpyAsync(ed, s->red_out, sizeof(ed), cudaMemcpyDeviceToHost, s->stream));
+    EdSink sink;
+    sink.out = s->red_out;
+    sink.counter = reinterpret_cast<unsigned*>(s->d_err + 1);
+    sink.host = s->h_pin;
+    CK(energy_dissipation(s->u, N, s->nu, s->red, sink, s->stream));
     CK(cudaStreamSynchronize(s->stream));
+    const double ed[2] = {s->h_pin[0], s->h_pin[1]};
     if (!std::isfinite(ed[0]))
         return fail(KIN_ENONFINITE, "non-finite statistics at step %lld", (long long)s->step);
     if (!s->have_d2z) {
@@ -648,7 +673,7 @@ int kin_derived_stats(kin_sim* s, double* out, double* D) {
     double m[9];
     CK(cudaMemcpyAsync(m, s->red_out, sizeof(m), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
-    s->launches += 10;  // velocity, 2 + 2 reductions, 3 multiplies, 2 moment passes
+    s->launches += 9;  // velocity, 1 + 2 reductions, 3 multiplies, 2 moment passes
     const double kf = 2.0 * 3.14159265358979323846 / N, nu = s->nu;
     double eps = 0.0;
     for (int k = 0; k < nsh; ++k) {

@@ -57,21 +57,32 @@ size_t dugks_scratch_bytes(int storage);
 cudaError_t velocity_field(int storage, const void* state, bool shifted, int N, double* u,
                            cudaStream_t stream);
 
-// E and eps sums: partials[2 * nblocks] then out[2] = {E, eps} (FP64, fixed
-// order).  nblocks = stats_blocks(N) <= kStatsMaxBlocks (8 per SM on 152 SMs).
+// Where E and eps go: out[0..1] (device).  counter: a zeroed device word of this
+// caller's, or NULL (the total is then a launch of its own).  host: NULL, or
+// device-accessible host memory that also receives them; with err also the
+// device error word, in the int at host + 2.
+struct EdSink {
+    double* out = nullptr;
+    unsigned* counter = nullptr;
+    double* host = nullptr;
+    const int* err = nullptr;
+};
+
+// E and eps sums: partials[2 * nblocks], FP64, summed in a fixed order.
+// nblocks <= stats_blocks(N) <= kStatsMaxBlocks (8 per SM on 152 SMs).
 constexpr int kStatsMaxBlocks = 1216;
 int stats_blocks(int N);
 // FP32 statistics path for storage types computed in FP32 (F32, F16, BF16).
 cudaError_t velocity_field32(int storage, const void* state, bool shifted, int N, float* u,
                              cudaStream_t stream);
-cudaError_t energy_dissipation32(const float* u, int N, double nu, double* partials, double* out,
+cudaError_t energy_dissipation32(const float* u, int N, double nu, double* partials, const EdSink& sink,
                                  cudaStream_t stream);
 // Derived statistics: spectral derivative of one component in place, and the
 // moments <d^p> (p = 2, 3, 4) of three derivative fields d[3][N^3] -> out[9].
 cudaError_t derivative_multiply(double2* uh, int N, int axis, cudaStream_t stream);
 cudaError_t derivative_moments(const double* d, int N, double* partial, double* out, cudaStream_t stream);
 int deriv_moment_blocks(int N);
-cudaError_t energy_dissipation(const double* u, int N, double nu, double* partials, double* out,
+cudaError_t energy_dissipation(const double* u, int N, double nu, double* partials, const EdSink& sink,
                                cudaStream_t stream);
 
 // Shell sums of |inv * X|^2 / 2 over the half-complex arrays X of the three

@@ -32,7 +32,7 @@ struct kin_sim {
     int block_lbe = 0, block_dugks = 0;
     int tile_y = 0, zchunk = 0, variant = 0;  // 0: chosen by dugks_fused_shape
     int fused_ty = 0, fused_zc = 0;  // the fused step's shape for this tuning (0: not chosen yet)
-    int* d_err = nullptr;  // set by a kernel whose bounded wait gave up
+    int* d_err = nullptr;  // [0] set by a kernel whose bounded wait gave up, [1] blocks of a reduction done
     double* h_pin = nullptr;  // pinned host words: E, eps, and the error flag
     int64_t launches = 0;  // own kernel launches
     // state version: bumped by every step and every write of the state; u32

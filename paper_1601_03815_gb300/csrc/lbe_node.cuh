@@ -156,18 +156,15 @@ struct Half1<__nv_bfloat16> {
     }
 };
 
-// Four consecutive cells with their populations held packed (two cells a
-// word) between the loads and the stores; each cell is unpacked, relaxed and
-// packed back in turn, so the thread holds 38 words and one cell's 19 floats
-// instead of four cells' 76.  Same arithmetic per cell as lbe_node.
+// The pulled populations of four consecutive cells, held packed (two cells a
+// word).
 template <typename S>
-__device__ __forceinline__ void lbe_vnode4p(const S* __restrict__ src, S* __restrict__ dst, int N, size_t plane,
-                                            int x, int y, int z, const MrtRates<float>& rates) {
+__device__ __forceinline__ void lbe_gather4p(const S* __restrict__ src, int N, size_t plane, int x, int y, int z,
+                                             unsigned (&w)[Q][2]) {
     const int xm = x == 0 ? N - 1 : x - 1;
     const int xp = x + 4 == N ? 0 : x + 4;
     const int yo[3] = {wrap_dec(y, N) * N, y * N, wrap_inc(y, N) * N};
     const int zo[3] = {wrap_dec(z, N) * N * N, z * N * N, wrap_inc(z, N) * N * N};
-    unsigned w[Q][2];
     static_for<0, Q>([&](auto ic) {
         constexpr int I = decltype(ic)::value;
         const S* row = src + (size_t)I * plane + (yo[1 - cy(I)] + zo[1 - cz(I)]);
@@ -188,6 +185,17 @@ __device__ __forceinline__ void lbe_vnode4p(const S* __restrict__ src, S* __rest
             w[I][1] = __byte_perm(own.y, r, 0x5432);
         }
     });
+}
+
+// Four consecutive cells with their populations held packed (two cells a
+// word) between the loads and the stores; each cell is unpacked, relaxed and
+// packed back in turn, so the thread holds 38 words and one cell's 19 floats
+// instead of four cells' 76.  Same arithmetic per cell as lbe_node.
+template <typename S>
+__device__ __forceinline__ void lbe_vnode4p(const S* __restrict__ src, S* __restrict__ dst, int N, size_t plane,
+                                            int x, int y, int z, const MrtRates<float>& rates) {
+    unsigned w[Q][2];
+    lbe_gather4p<S>(src, N, plane, x, y, z, w);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         float f[Q];

@@ -5,7 +5,10 @@
 //   ed_partial_kernel      per-block FP64 sums of |u|^2 and s_ab s_ab
 //   ed32_partial_kernel    the same from FP32 u: per-cell terms in FP32,
 //                          per-thread and block sums in FP64
-//   ed_final_kernel        fixed-order sum of the block partials -> {E, eps}
+//                          (the last block of either to finish sums the
+//                          partials in a fixed order -> {E, eps})
+//   ed_final_kernel        that sum as a kernel, for callers without the
+//                          counter that tells the last block
 //   shell_partial_kernel   per-block shell sums of |u_hat|^2 / 2 (Eq. 27)
 //   shell_final_kernel     fixed-order sum over blocks
 // Every reduction runs in a fixed order for a given N, so results are
@@ -13,11 +16,13 @@
 #include "kin.h"
 #include "kin_common.cuh"
 #include "kin_internal.h"
+#include "kin_launch.cuh"
 #include "kin_sim.h"
+#include "lbe_node.cuh"
 
 #include <cufft.h>
 
-#include <mutex>
+#include <algorithm>
 
 namespace kin {
 
@@ -56,55 +61,103 @@ template <typename S>
 __global__ void velocity_kernel(const S* __restrict__ st, bool shifted, int N, size_t plane,
                                 double* __restrict__ u) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    grid_begin();
     if (x >= N) return;
     const int y = blockIdx.y, z = blockIdx.z;
-    double jx = 0.0, jy = 0.0, jz = 0.0;
-    static_for<0, Q>([&](auto ic) {
-        constexpr int I = decltype(ic)::value;
-        const double v = (double)Traits<S>::load(st + I * plane + stored_index<I>(x, y, z, N, shifted));
-        if constexpr (cx(I) != 0) jx += cx(I) * v;
-        if constexpr (cy(I) != 0) jy += cy(I) * v;
-        if constexpr (cz(I) != 0) jz += cz(I) * v;
+    // 21 FP64 additions: an opposite pair enters as its difference
+    double b[NPAIR];
+    static_for<0, NPAIR>([&](auto pc) {
+        constexpr int P = decltype(pc)::value, I = 2 * P + 1;
+        b[P] = (double)Traits<S>::load_l2(st + I * plane + stored_index<I>(x, y, z, N, shifted)) -
+               (double)Traits<S>::load_l2(st + (I + 1) * plane + stored_index<I + 1>(x, y, z, N, shifted));
     });
+    const double jx = (b[0] + b[3]) + (b[4] + (b[5] + b[6]));
+    const double jy = (b[1] + b[3]) - (b[4] - (b[7] + b[8]));
+    const double jz = (b[2] + b[5]) - (b[6] - (b[7] - b[8]));
     const size_t c = (size_t)x + (size_t)N * (y + (size_t)N * z);
     u[c] = jx;
     u[plane + c] = jy;
     u[2 * plane + c] = jz;
 }
 
-// FP32 storage, FP32 arithmetic: u in FP32 (the per-cell sums of 19 terms
-// carry the storage's own rounding; the FP64 path above serves FP64 storage).
-template <typename S>
-__global__ void velocity32_kernel(const S* __restrict__ st, bool shifted, int N, size_t plane,
-                                  float* __restrict__ u) {
+// u in FP32 for storage computed in FP32, the populations of a cell added in
+// their order (the fused DUGKS step forms the same sums).  SHIFTED: the LBE
+// pull layout; its row offsets are formed once per cell, which with the index
+// arithmetic of stored_index took as long as the loads (256^3 LBE: FP32
+// 250 -> 218 us, FP16 254 -> 130 us with four cells a thread).
+template <int I>
+__device__ __forceinline__ void add_velocity(float (&j)[3], float v) {
+    if constexpr (cx(I) > 0) j[0] += v;
+    if constexpr (cx(I) < 0) j[0] -= v;
+    if constexpr (cy(I) > 0) j[1] += v;
+    if constexpr (cy(I) < 0) j[1] -= v;
+    if constexpr (cz(I) > 0) j[2] += v;
+    if constexpr (cz(I) < 0) j[2] -= v;
+}
+
+template <typename S, bool SHIFTED>
+__global__ void velocity32_kernel(const S* st, int N, size_t plane, float* __restrict__ u) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    grid_begin();
     if (x >= N) return;
     const int y = blockIdx.y, z = blockIdx.z;
-    float j[3] = {0.0f, 0.0f, 0.0f};
-    static_for<0, Q>([&](auto ic) {
-        constexpr int I = decltype(ic)::value;
-        const float v = (float)Traits<S>::load(st + I * plane + stored_index<I>(x, y, z, N, shifted));
-        if constexpr (cx(I) > 0) j[0] += v;
-        if constexpr (cx(I) < 0) j[0] -= v;
-        if constexpr (cy(I) > 0) j[1] += v;
-        if constexpr (cy(I) < 0) j[1] -= v;
-        if constexpr (cz(I) > 0) j[2] += v;
-        if constexpr (cz(I) < 0) j[2] -= v;
-    });
     const size_t c = (size_t)x + (size_t)N * (y + (size_t)N * z);
+    float f[Q];
+    if constexpr (SHIFTED) {
+        lbe_gather<S>(st, N, plane, x, y, z, f);
+    } else {
+#pragma unroll
+        for (int i = 1; i < Q; ++i) f[i] = Traits<S>::load_l2(st + i * plane + c);
+    }
+    float j[3] = {0.0f, 0.0f, 0.0f};
+    static_for<1, Q>([&](auto ic) { add_velocity<decltype(ic)::value>(j, f[decltype(ic)::value]); });
     u[c] = j[0];
     u[plane + c] = j[1];
     u[2 * plane + c] = j[2];
 }
 
+// 2-byte storage, N % 4 == 0: four x-neighbouring cells a thread, read as aligned
+// 8-byte words (as the LBE step does), the same sums per cell.
+template <typename S, bool SHIFTED>
+__global__ void __launch_bounds__(128) velocity32v4_kernel(const S* st, int N, size_t plane, float* __restrict__ u) {
+    const int x = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+    grid_begin();
+    if (x >= N) return;
+    const int y = blockIdx.y, z = blockIdx.z;
+    unsigned w[Q][2];
+    if constexpr (SHIFTED) {
+        lbe_gather4p<S>(st, N, plane, x, y, z, w);
+    } else {
+        const size_t c = (size_t)x + (size_t)N * (y + (size_t)N * z);
+#pragma unroll
+        for (int i = 1; i < Q; ++i) {
+            const uint2 v = __ldcg(reinterpret_cast<const uint2*>(st + i * plane + c));
+            w[i][0] = v.x;
+            w[i][1] = v.y;
+        }
+    }
+    float j[4][3];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        j[k][0] = j[k][1] = j[k][2] = 0.0f;
+        static_for<1, Q>([&](auto ic) {
+            constexpr int I = decltype(ic)::value;
+            add_velocity<I>(j[k], Half1<S>::get(w[I][k >> 1], k & 1));
+        });
+    }
+    float* o = u + ((size_t)x + (size_t)N * (y + (size_t)N * z));
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+        *reinterpret_cast<float4*>(o + a * plane) = make_float4(j[0][a], j[1][a], j[2][a], j[3][a]);
+}
+
 constexpr int RED_THREADS = 256;
 
+// One cell a thread and pass (FP64 arithmetic runs at 1/64 of the FP32 rate, so
+// a small box has to reach every SM: 32^3 FP64 in 16 blocks took 27 us).
 int stats_blocks(int N) {
-    long long n = (long long)N * N * N;
-    long long b = (n + RED_THREADS * 8 - 1) / (RED_THREADS * 8);
-    if (b > kStatsMaxBlocks) b = kStatsMaxBlocks;
-    if (b < 1) b = 1;
-    return (int)b;
+    const long long n = (long long)N * N * N;
+    return (int)std::min<long long>((n + RED_THREADS - 1) / RED_THREADS, kStatsMaxBlocks);
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -113,56 +166,113 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// Block-then-warp reduction of |u|^2 and s_ab s_ab; each thread walks a fixed
-// grid-stride sequence of cells.
-__global__ void __launch_bounds__(RED_THREADS)
-    ed_partial_kernel(const double* __restrict__ u, int N, double* __restrict__ partial) {
-    const size_t n = (size_t)N * N * N;
-    double se = 0.0, ss = 0.0;
-    for (size_t c = (size_t)blockIdx.x * RED_THREADS + threadIdx.x; c < n;
-         c += (size_t)gridDim.x * RED_THREADS) {
-        const int x = (int)(c % N), y = (int)((c / N) % N), z = (int)(c / ((size_t)N * N));
-        const size_t nb[3][2] = {
-            {(size_t)wrap_inc(x, N) + (size_t)N * (y + (size_t)N * z),
-             (size_t)wrap_dec(x, N) + (size_t)N * (y + (size_t)N * z)},
-            {(size_t)x + (size_t)N * (wrap_inc(y, N) + (size_t)N * z),
-             (size_t)x + (size_t)N * (wrap_dec(y, N) + (size_t)N * z)},
-            {(size_t)x + (size_t)N * (y + (size_t)N * wrap_inc(z, N)),
-             (size_t)x + (size_t)N * (y + (size_t)N * wrap_dec(z, N))}};
-        double g[3][3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) g[a][b] = 0.5 * (u[b * n + nb[a][0]] - u[b * n + nb[a][1]]);
-        double s2 = 0.0;
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                const double sab = 0.5 * (g[a][b] + g[b][a]);
-                s2 += sab * sab;
-            }
-        ss += s2;
-        se += u[c] * u[c] + u[n + c] * u[n + c] + u[2 * n + c] * u[2 * n + c];
-    }
+// Sums of a and b over the block, in thread 0 (warps, then the block, in order).
+__device__ __forceinline__ void block_sum2(double& a, double& b) {
     __shared__ double sh[2][RED_THREADS / 32];
-    se = warp_sum(se);
-    ss = warp_sum(ss);
+    a = warp_sum(a);
+    b = warp_sum(b);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __syncthreads();
     if (lane == 0) {
-        sh[0][wid] = se;
-        sh[1][wid] = ss;
+        sh[0][wid] = a;
+        sh[1][wid] = b;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double a = 0.0, b = 0.0;
+        a = b = 0.0;
         for (int w = 0; w < RED_THREADS / 32; ++w) {
             a += sh[0][w];
             b += sh[1][w];
         }
+    }
+}
+
+// Fixed-order sum of the block partials {sum |u|^2, sum s_ab s_ab} by one block:
+// thread t takes partials t, t + RED_THREADS, ..., then block_sum2.
+__device__ __forceinline__ void ed_total(const double* partial, int nblocks, size_t n, double nu, const EdSink& sink) {
+    double a = 0.0, b = 0.0;
+    for (int i = threadIdx.x; i < nblocks; i += RED_THREADS) {
+        a += __ldcg(partial + 2 * i);
+        b += __ldcg(partial + 2 * i + 1);
+    }
+    block_sum2(a, b);
+    if (threadIdx.x == 0) {
+        const double E = 0.5 * a / (double)n, eps = 2.0 * nu * b / (double)n;
+        sink.out[0] = E;
+        sink.out[1] = eps;
+        if (sink.host) {
+            sink.host[0] = E;
+            sink.host[1] = eps;
+            if (sink.err) *reinterpret_cast<int*>(sink.host + 2) = __ldcg(sink.err);
+        }
+    }
+}
+
+// A block's sums into its partial; the last block to get here (counter, which
+// wraps to zero for the next call) forms the total.  One launch instead of two:
+// the one-block total took 6 us of its own.
+__device__ __forceinline__ void ed_block_done(double a, double b, double* partial, size_t n, double nu,
+                                              const EdSink& sink) {
+    block_sum2(a, b);
+    if (threadIdx.x == 0) {
         partial[2 * blockIdx.x] = a;
         partial[2 * blockIdx.x + 1] = b;
     }
+    if (!sink.counter) return;
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicInc(sink.counter, gridDim.x - 1) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    ed_total(partial, gridDim.x, n, nu, sink);
+}
+
+// Reduction of |u|^2 and s_ab s_ab in FP64; each thread walks a fixed
+// grid-stride sequence of cells.  With g_ab = u_b(+e_a) - u_b(-e_a),
+// s_ab s_ab = sum_a g_aa^2 / 4 + sum_{a<b} (g_ab + g_ba)^2 / 8: 21 FP64
+// operations a cell (they are what bounds the kernel), the factors exact.
+__global__ void __launch_bounds__(RED_THREADS)
+    ed_partial_kernel(const double* u, int N, double nu, double* partial, EdSink sink) {
+    grid_begin();
+    const size_t n = (size_t)N * N * N;
+    const double* U[3] = {u, u + n, u + 2 * n};
+    double se = 0.0, sd = 0.0, so = 0.0;
+    // N <= 1024: cell indices fit in 32 bits
+    const unsigned un = (unsigned)N, nn = un * un;
+    for (unsigned c = blockIdx.x * RED_THREADS + threadIdx.x; c < (unsigned)n; c += gridDim.x * RED_THREADS) {
+        const unsigned z = c / nn, r = c - z * nn, y = r / un, x = r - y * un;
+        const unsigned up[3] = {x + 1 == un ? c - x : c + 1, y + 1 == un ? c - y * un : c + un,
+                                z + 1 == un ? c - z * nn : c + nn};
+        const unsigned dn[3] = {x == 0 ? c + un - 1 : c - 1, y == 0 ? c + nn - un : c - un,
+                                z == 0 ? c + (un - 1) * nn : c - nn};
+        double g[3][3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) g[a][b] = U[b][up[a]] - U[b][dn[a]];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            sd = fma(g[a][a], g[a][a], sd);
+            const double o = g[a][(a + 1) % 3] + g[(a + 1) % 3][a];
+            so = fma(o, o, so);
+            const double v = U[a][c];
+            se = fma(v, v, se);
+        }
+    }
+    ed_block_done(se, 0.25 * sd + 0.125 * so, partial, n, nu, sink);
+}
+
+// One cell's |u|^2 and s_ab s_ab in FP32 (the form of ed_partial_kernel), formed
+// before they are added to the running sums.
+__device__ __forceinline__ void add_cell(const float (&g)[3][3], const float (&u)[3], float& fe, float& fs) {
+    const float d = fmaf(g[2][2], g[2][2], fmaf(g[1][1], g[1][1], g[0][0] * g[0][0]));
+    const float xy = g[0][1] + g[1][0], yz = g[1][2] + g[2][1], zx = g[2][0] + g[0][2];
+    const float o = fmaf(zx, zx, fmaf(yz, yz, xy * xy));
+    fs += fmaf(0.5f, o, d) * 0.25f;
+    fe += fmaf(u[2], u[2], fmaf(u[1], u[1], u[0] * u[0]));
 }
 
 // FP32 counterpart of ed_partial_kernel: block b takes the rows (y, z) =
@@ -170,10 +280,11 @@ __global__ void __launch_bounds__(RED_THREADS)
 // |u|^2 and s_ab s_ab are formed in FP32, summed in FP32 over at most 8 rows
 // and then in FP64, in a fixed order.
 __global__ void __launch_bounds__(RED_THREADS)
-    ed32_partial_kernel(const float* __restrict__ u, int N, double* __restrict__ partial) {
+    ed32_partial_kernel(const float* u, int N, double nu, double* partial, EdSink sink) {
+    grid_begin();
     const size_t n = (size_t)N * N * N;
     // component bases; offsets inside a component fit in 32 bits (N <= 1024)
-    const float* __restrict__ U[3] = {u, u + n, u + 2 * n};
+    const float* U[3] = {u, u + n, u + 2 * n};
     double se = 0.0, ss = 0.0;
     float fe = 0.0f, fs = 0.0f;
     int rows_in_chunk = 0;
@@ -192,45 +303,19 @@ __global__ void __launch_bounds__(RED_THREADS)
                                 {N * (y + N * wrap_inc(z, N)), N * (y + N * wrap_dec(z, N))}};
         for (int x = threadIdx.x; x < N; x += RED_THREADS) {
             const int xs[3][2] = {{wrap_inc(x, N), wrap_dec(x, N)}, {x, x}, {x, x}};
-            float g[3][3];  // g[a][b] = d u_b / d x_a, central differences
+            float g[3][3];  // g[a][b] = 2 d u_b / d x_a, central differences
 #pragma unroll
             for (int a = 0; a < 3; ++a)
 #pragma unroll
                 for (int b = 0; b < 3; ++b)
-                    g[a][b] = 0.5f * (__ldg(U[b] + rows[a][0] + xs[a][0]) - __ldg(U[b] + rows[a][1] + xs[a][1]));
-            float s2 = 0.0f;
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-#pragma unroll
-                for (int b = 0; b < 3; ++b) {
-                    const float sab = 0.5f * (g[a][b] + g[b][a]);
-                    s2 += sab * sab;
-                }
-            const float u0 = __ldg(U[0] + row + x), u1 = __ldg(U[1] + row + x), u2 = __ldg(U[2] + row + x);
-            fe += u0 * u0 + u1 * u1 + u2 * u2;
-            fs += s2;
+                    g[a][b] = U[b][rows[a][0] + xs[a][0]] - U[b][rows[a][1] + xs[a][1]];
+            const float v[3] = {U[0][row + x], U[1][row + x], U[2][row + x]};
+            add_cell(g, v, fe, fs);
         }
     }
     se += (double)fe;
     ss += (double)fs;
-    __shared__ double sh[2][RED_THREADS / 32];
-    se = warp_sum(se);
-    ss = warp_sum(ss);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) {
-        sh[0][wid] = se;
-        sh[1][wid] = ss;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0.0, b = 0.0;
-        for (int w = 0; w < RED_THREADS / 32; ++w) {
-            a += sh[0][w];
-            b += sh[1][w];
-        }
-        partial[2 * blockIdx.x] = a;
-        partial[2 * blockIdx.x + 1] = b;
-    }
+    ed_block_done(se, ss, partial, n, nu, sink);
 }
 
 // The same for N a multiple of 4, four cells per thread: a thread reads its
@@ -240,9 +325,10 @@ __global__ void __launch_bounds__(RED_THREADS)
 // terms of a thread's cells are summed in cell order, in FP32 over at most 8
 // row groups and then in FP64.
 __global__ void __launch_bounds__(RED_THREADS)
-    ed32v4_partial_kernel(const float* __restrict__ u, int N, double* __restrict__ partial) {
+    ed32v4_partial_kernel(const float* u, int N, double nu, double* partial, EdSink sink) {
+    grid_begin();
     const size_t n = (size_t)N * N * N;
-    const float* __restrict__ U[3] = {u, u + n, u + 2 * n};
+    const float* U[3] = {u, u + n, u + 2 * n};
     const int gpr = N / 4, rpi = RED_THREADS / gpr;
     const int rsub = threadIdx.x / gpr, x = 4 * (threadIdx.x % gpr);
     const bool active = rsub < rpi;
@@ -265,28 +351,28 @@ __global__ void __launch_bounds__(RED_THREADS)
         const int row = N * r;
         const int ryp = N * (wrap_inc(y, N) + N * z), rym = N * (wrap_dec(y, N) + N * z);
         const int rzp = N * (y + N * wrap_inc(z, N)), rzm = N * (y + N * wrap_dec(z, N));
-        float g[4][3][3];  // g[cell][a][b] = d u_b / d x_a
+        float g[4][3][3];  // g[cell][a][b] = 2 d u_b / d x_a
         float c[4][3];
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
-            const float4 cc = __ldg(reinterpret_cast<const float4*>(U[b] + row + x));
-            const float4 yp = __ldg(reinterpret_cast<const float4*>(U[b] + ryp + x));
-            const float4 ym = __ldg(reinterpret_cast<const float4*>(U[b] + rym + x));
-            const float4 zp = __ldg(reinterpret_cast<const float4*>(U[b] + rzp + x));
-            const float4 zm = __ldg(reinterpret_cast<const float4*>(U[b] + rzm + x));
-            const float l = __ldg(U[b] + row + xm), rr = __ldg(U[b] + row + xp);
-            g[0][0][b] = 0.5f * (cc.y - l);
-            g[1][0][b] = 0.5f * (cc.z - cc.x);
-            g[2][0][b] = 0.5f * (cc.w - cc.y);
-            g[3][0][b] = 0.5f * (rr - cc.z);
-            g[0][1][b] = 0.5f * (yp.x - ym.x);
-            g[1][1][b] = 0.5f * (yp.y - ym.y);
-            g[2][1][b] = 0.5f * (yp.z - ym.z);
-            g[3][1][b] = 0.5f * (yp.w - ym.w);
-            g[0][2][b] = 0.5f * (zp.x - zm.x);
-            g[1][2][b] = 0.5f * (zp.y - zm.y);
-            g[2][2][b] = 0.5f * (zp.z - zm.z);
-            g[3][2][b] = 0.5f * (zp.w - zm.w);
+            const float4 cc = *reinterpret_cast<const float4*>(U[b] + row + x);
+            const float4 yp = *reinterpret_cast<const float4*>(U[b] + ryp + x);
+            const float4 ym = *reinterpret_cast<const float4*>(U[b] + rym + x);
+            const float4 zp = *reinterpret_cast<const float4*>(U[b] + rzp + x);
+            const float4 zm = *reinterpret_cast<const float4*>(U[b] + rzm + x);
+            const float l = U[b][row + xm], rr = U[b][row + xp];
+            g[0][0][b] = cc.y - l;
+            g[1][0][b] = cc.z - cc.x;
+            g[2][0][b] = cc.w - cc.y;
+            g[3][0][b] = rr - cc.z;
+            g[0][1][b] = yp.x - ym.x;
+            g[1][1][b] = yp.y - ym.y;
+            g[2][1][b] = yp.z - ym.z;
+            g[3][1][b] = yp.w - ym.w;
+            g[0][2][b] = zp.x - zm.x;
+            g[1][2][b] = zp.y - zm.y;
+            g[2][2][b] = zp.z - zm.z;
+            g[3][2][b] = zp.w - zm.w;
             c[0][b] = cc.x;
             c[1][b] = cc.y;
             c[2][b] = cc.z;
@@ -294,92 +380,38 @@ __global__ void __launch_bounds__(RED_THREADS)
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            float s2 = 0.0f;
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-#pragma unroll
-                for (int b = 0; b < 3; ++b) {
-                    const float sab = 0.5f * (g[j][a][b] + g[j][b][a]);
-                    s2 += sab * sab;
-                }
-            fe += c[j][0] * c[j][0] + c[j][1] * c[j][1] + c[j][2] * c[j][2];
-            fs += s2;
+            add_cell(g[j], c[j], fe, fs);
         }
     }
     se += (double)fe;
     ss += (double)fs;
-    __shared__ double sh[2][RED_THREADS / 32];
-    se = warp_sum(se);
-    ss = warp_sum(ss);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) {
-        sh[0][wid] = se;
-        sh[1][wid] = ss;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0.0, b = 0.0;
-        for (int w = 0; w < RED_THREADS / 32; ++w) {
-            a += sh[0][w];
-            b += sh[1][w];
-        }
-        partial[2 * blockIdx.x] = a;
-        partial[2 * blockIdx.x + 1] = b;
-    }
+    ed_block_done(se, ss, partial, n, nu, sink);
 }
 
-// One block of FIN_THREADS: thread t sums partials t, t + FIN_THREADS, ... in
-// order, then the warps and the block reduce in a fixed order.
-constexpr int FIN_THREADS = 256;
-__global__ void __launch_bounds__(FIN_THREADS)
-    ed_final_kernel(const double* __restrict__ partial, int nblocks, size_t n, double nu,
-                    double* __restrict__ out) {
-    double a = 0.0, b = 0.0;
-    for (int i = threadIdx.x; i < nblocks; i += FIN_THREADS) {
-        a += partial[2 * i];
-        b += partial[2 * i + 1];
-    }
-    a = warp_sum(a);
-    b = warp_sum(b);
-    __shared__ double sh[2][FIN_THREADS / 32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) {
-        sh[0][wid] = a;
-        sh[1][wid] = b;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double ta = 0.0, tb = 0.0;
-        for (int w = 0; w < FIN_THREADS / 32; ++w) {
-            ta += sh[0][w];
-            tb += sh[1][w];
-        }
-        out[0] = 0.5 * ta / (double)n;
-        out[1] = 2.0 * nu * tb / (double)n;
-    }
+__global__ void __launch_bounds__(RED_THREADS)
+    ed_final_kernel(const double* partial, int nblocks, size_t n, double nu, EdSink sink) {
+    grid_begin();
+    ed_total(partial, nblocks, n, nu, sink);
 }
 
-cudaError_t energy_dissipation(const double* u, int N, double nu, double* partials, double* out,
+cudaError_t energy_dissipation(const double* u, int N, double nu, double* partials, const EdSink& sink,
                                cudaStream_t stream) {
     const int nb = stats_blocks(N);
-    ed_partial_kernel<<<nb, RED_THREADS, 0, stream>>>(u, N, partials);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    ed_final_kernel<<<1, FIN_THREADS, 0, stream>>>(partials, nb, (size_t)N * N * N, nu, out);
-    return cudaGetLastError();
+    cudaError_t e = launch_next(ed_partial_kernel, nb, RED_THREADS, 0, stream, u, N, nu, partials, sink);
+    if (e != cudaSuccess || sink.counter) return e;
+    return launch_next(ed_final_kernel, 1, RED_THREADS, 0, stream, (const double*)partials, nb, (size_t)N * N * N, nu,
+                       sink);
 }
 
-cudaError_t energy_dissipation32(const float* u, int N, double nu, double* partials, double* out,
+cudaError_t energy_dissipation32(const float* u, int N, double nu, double* partials, const EdSink& sink,
                                  cudaStream_t stream) {
-    const int nb = stats_blocks(N);
-    if (N % 4 == 0 && N / 4 <= RED_THREADS)
-        ed32v4_partial_kernel<<<nb, RED_THREADS, 0, stream>>>(u, N, partials);
-    else
-        ed32_partial_kernel<<<nb, RED_THREADS, 0, stream>>>(u, N, partials);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    ed_final_kernel<<<1, FIN_THREADS, 0, stream>>>(partials, nb, (size_t)N * N * N, nu, out);
-    return cudaGetLastError();
+    if (N % 4 == 0 && N / 4 <= RED_THREADS) {
+        const int rows = RED_THREADS / (N / 4);  // a block's rows at a time
+        const int nb = std::min(stats_blocks(N), (N * N + rows - 1) / rows);
+        return launch_next(ed32v4_partial_kernel, nb, RED_THREADS, 0, stream, u, N, nu, partials, sink);
+    }
+    return launch_next(ed32_partial_kernel, std::min(stats_blocks(N), N * N), RED_THREADS, 0, stream, u, N, nu, partials,
+                       sink);
 }
 
 // ---------------------------------------------------------------------------
@@ -403,7 +435,7 @@ int spectrum_blocks(int N) {
 template <typename CT>
 __global__ void __launch_bounds__(SPEC_THREADS)
     shell_partial_kernel(const CT* __restrict__ u0, const CT* __restrict__ u1,
-                         const CT* __restrict__ u2, int N, int nshell, double inv,
+                         const CT* __restrict__ u2, int N, int nshell, double scale,
                          int weight_n2, double* __restrict__ partial) {
     extern __shared__ double bins[];  // [SPEC_THREADS/32][nshell]
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -431,8 +463,7 @@ __global__ void __launch_bounds__(SPEC_THREADS)
             const CT a = u0[m], b = u1[m], c = u2[m];
             const double amp = (double)((a.x * a.x + a.y * a.y) + (b.x * b.x + b.y * b.y) + (c.x * c.x + c.y * c.y));
             const double w = (kx > 0 && 2 * kx < N) ? 2.0 : 1.0;
-            e = 0.5 * amp * inv * inv * w;
-            if (weight_n2) e *= (double)n2;
+            e = amp * (weight_n2 ? (double)n2 * w : w);
         }
         const unsigned same = __match_any_sync(0xffffffffu, shell);
         const int leader = __ffs(same) - 1;
@@ -450,7 +481,7 @@ __global__ void __launch_bounds__(SPEC_THREADS)
     for (int s = threadIdx.x; s < nshell; s += SPEC_THREADS) {
         double a = 0.0;
         for (int w = 0; w < SPEC_THREADS / 32; ++w) a += bins[w * nshell + s];
-        partial[(size_t)blockIdx.x * nshell + s] = a;
+        partial[(size_t)blockIdx.x * nshell + s] = a * scale;
     }
 }
 
@@ -467,7 +498,9 @@ __global__ void shell_final_kernel(const double* __restrict__ partial, int nbloc
 // Spectral derivative d_a u_a of one component: u_hat (half-complex, unscaled
 // D2Z output) times i k_a / N^3, the Nyquist wavenumber of axis a set to zero;
 // the Z2D of the result is the derivative field.
-__global__ void deriv_mult_kernel(double2* __restrict__ uh, int N, int axis) {
+// k1 = 2 pi / N / N^3 (formed on the host: a division a mode cost as much as the
+// memory traffic).
+__global__ void deriv_mult_kernel(double2* __restrict__ uh, int N, int axis, double k1) {
     const int nh = N / 2 + 1;
     const int kx = blockIdx.x * blockDim.x + threadIdx.x;
     if (kx >= nh) return;
@@ -476,8 +509,7 @@ __global__ void deriv_mult_kernel(double2* __restrict__ uh, int N, int axis) {
     int n = axis == 0 ? kx : axis == 1 ? ky : kz;
     if (axis != 0 && n > N / 2) n -= N;
     const bool nyquist = (N % 2 == 0) && (n == N / 2 || n == -N / 2);
-    const double inv = 1.0 / ((double)N * N * N);
-    const double k = nyquist ? 0.0 : 2.0 * 3.14159265358979323846 * n / N * inv;
+    const double k = nyquist ? 0.0 : (double)n * k1;
     const double2 v = uh[m];
     uh[m] = make_double2(-k * v.y, k * v.x);
 }
@@ -537,7 +569,8 @@ cudaError_t derivative_multiply(double2* uh, int N, int axis, cudaStream_t strea
     const int nh = N / 2 + 1;
     const int bx = nh < 128 ? ((nh + 31) / 32) * 32 : 128;
     dim3 g((nh + bx - 1) / bx, N, N);
-    deriv_mult_kernel<<<g, bx, 0, stream>>>(uh, N, axis);
+    const double k1 = 2.0 * 3.14159265358979323846 / N / ((double)N * N * N);
+    deriv_mult_kernel<<<g, bx, 0, stream>>>(uh, N, axis, k1);
     return cudaGetLastError();
 }
 
@@ -562,7 +595,7 @@ static cudaError_t spectrum_shells_t(const void* uh0, const void* uh1, const voi
         if (e != cudaSuccess) return e;
     }
     shell_partial_kernel<CT><<<nb, SPEC_THREADS, smem, stream>>>(
-        (const CT*)uh0, (const CT*)uh1, (const CT*)uh2, N, nshell, inv, weight_n2, partial);
+        (const CT*)uh0, (const CT*)uh1, (const CT*)uh2, N, nshell, 0.5 * inv * inv, weight_n2, partial);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     shell_final_kernel<<<(nshell + 127) / 128, 128, 0, stream>>>(partial, nb, nshell, out);
@@ -685,24 +718,35 @@ cudaError_t velocity_field(int storage, const void* state, bool shifted, int N, 
     int bx;
     dim3 g = row_grid(N, bx);
     const size_t plane = (size_t)N * N * N;
-    KIN_DISPATCH(storage, (velocity_kernel<S><<<g, bx, 0, stream>>>((const S*)state, shifted, N, plane, u)));
-    return cudaGetLastError();
+    KIN_DISPATCH(storage, return launch_next(velocity_kernel<S>, g, bx, 0, stream, (const S*)state, shifted, N, plane, u));
+    return cudaSuccess;
+}
+
+template <typename S, bool SHIFTED>
+static cudaError_t velocity32_t(const void* state, int N, float* u, cudaStream_t stream) {
+    const size_t plane = (size_t)N * N * N;
+    if constexpr (sizeof(S) == 2) {
+        if (N % 4 == 0) {
+            const int nv = N / 4, bx = nv >= 64 ? 64 : 32;
+            return launch_next(velocity32v4_kernel<S, SHIFTED>, dim3((nv + bx - 1) / bx, N, N), bx, 0, stream,
+                               (const S*)state, N, plane, u);
+        }
+    }
+    int bx;
+    const dim3 g = row_grid(N, bx);
+    return launch_next(velocity32_kernel<S, SHIFTED>, g, bx, 0, stream, (const S*)state, N, plane, u);
 }
 
 cudaError_t velocity_field32(int storage, const void* state, bool shifted, int N, float* u,
                              cudaStream_t stream) {
-    int bx;
-    dim3 g = row_grid(N, bx);
-    const size_t plane = (size_t)N * N * N;
     switch (storage) {
-        case ST_F32: velocity32_kernel<float><<<g, bx, 0, stream>>>((const float*)state, shifted, N, plane, u); break;
-        case ST_F16: velocity32_kernel<__half><<<g, bx, 0, stream>>>((const __half*)state, shifted, N, plane, u); break;
+        case ST_F32: return shifted ? velocity32_t<float, true>(state, N, u, stream) : velocity32_t<float, false>(state, N, u, stream);
+        case ST_F16: return shifted ? velocity32_t<__half, true>(state, N, u, stream) : velocity32_t<__half, false>(state, N, u, stream);
         case ST_BF16:
-            velocity32_kernel<__nv_bfloat16><<<g, bx, 0, stream>>>((const __nv_bfloat16*)state, shifted, N, plane, u);
-            break;
-        default: return cudaErrorInvalidValue;
+            return shifted ? velocity32_t<__nv_bfloat16, true>(state, N, u, stream)
+                           : velocity32_t<__nv_bfloat16, false>(state, N, u, stream);
     }
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t equilibrium_from_velocity(int storage, const double* u, bool shifted, int N,
@@ -808,7 +852,9 @@ extern "C" int kin_energy_dissipation_noalloc(const double* u, int N, double nu,
     cudaError_t e;
     double* partials = noalloc_scratch(&e);
     if (!partials) return set_error(KIN_ECUDA, "cudaGetSymbolAddress: %s", cudaGetErrorString(e));
-    e = energy_dissipation(u, N, nu, partials, out, (cudaStream_t)stream);
+    EdSink sink;
+    sink.out = out;  // no counter: overlapping calls would leave it set
+    e = energy_dissipation(u, N, nu, partials, sink, (cudaStream_t)stream);
     if (e != cudaSuccess) return set_error(KIN_ECUDA, "reduction launch: %s", cudaGetErrorString(e));
     return KIN_OK;
 }
