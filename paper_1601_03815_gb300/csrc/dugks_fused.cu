@@ -14,17 +14,21 @@ namespace kin {
 // 8-row tiles and 0.777 for one 12-warp block of 11-row tiles.
 constexpr int blocks_per_sm(int ty) { return ty <= 5 ? 2 : 1; }
 
+// Rows that a warp holds whole, where tiles of 30 columns would take two (32^3
+// FP32 6.8 -> 5.2 us a step).
+constexpr bool whole_rows(int N) { return N == 31 || N == 32; }
+
 // VEL: also write the velocity of the new state to uvel (FP32-computed storage).
-template <typename S, int TY, bool VEL>
+template <typename S, int TY, bool VEL, bool WRAP>
 __global__ void __launch_bounds__(32 * (TY + 1), sizeof(typename Traits<S>::C) == 4 ? blocks_per_sm(TY) : 1)
     dugks_fused_kernel(const S* __restrict__ src, S* __restrict__ dst, int N, int zchunk,
                        DugksCoef<typename Traits<S>::C> kc, float* __restrict__ uvel) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     grid_begin();
-    dugks_tile<S, TY, VEL>(src, dst, N, blockIdx.x, blockIdx.y, blockIdx.z, zchunk, kc, smem_raw, uvel);
+    dugks_tile<S, TY, VEL, WRAP>(src, dst, N, blockIdx.x, blockIdx.y, blockIdx.z, zchunk, kc, smem_raw, uvel);
 }
 
-template <typename S, int TY, bool VEL>
+template <typename S, int TY, bool VEL, bool WRAP = false>
 static cudaError_t launch_fused_t(const void* src, void* dst, int N, int zchunk,
                                   const DugksCoef<typename Traits<S>::C>& k, float* uvel, cudaStream_t stream) {
     const size_t smem = fused_smem_bytes<S, TY>();
@@ -36,7 +40,7 @@ static cudaError_t launch_fused_t(const void* src, void* dst, int N, int zchunk,
     if (e != cudaSuccess) return e;
     const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
     if (!bit || !(configured.load() & bit)) {
-        e = cudaFuncSetAttribute(dugks_fused_kernel<S, TY, VEL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(dugks_fused_kernel<S, TY, VEL, WRAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem);
         if (e != cudaSuccess) return e;
         configured.fetch_or(bit);
@@ -44,8 +48,8 @@ static cudaError_t launch_fused_t(const void* src, void* dst, int N, int zchunk,
     if (zchunk <= 0) zchunk = 32;
     if (zchunk > N) zchunk = N;
     dim3 block(32, TY + 1);
-    dim3 grid((N + 29) / 30, (N + TY - 1) / TY, (N + zchunk - 1) / zchunk);
-    return launch_next(dugks_fused_kernel<S, TY, VEL>, grid, block, smem, stream, (const S*)src, (S*)dst, N, zchunk, k,
+    dim3 grid(WRAP ? 1 : (N + 29) / 30, (N + TY - 1) / TY, (N + zchunk - 1) / zchunk);
+    return launch_next(dugks_fused_kernel<S, TY, VEL, WRAP>, grid, block, smem, stream, (const S*)src, (S*)dst, N, zchunk, k,
                        uvel);
 }
 
@@ -53,8 +57,11 @@ template <typename S, bool VEL>
 static cudaError_t launch_fused_v(const void* src, void* dst, int N, const DugksCoef<typename Traits<S>::C>& k,
                                   int ty, int zchunk, float* uvel, cudaStream_t stream) {
     if constexpr (sizeof(typename Traits<S>::C) == 8) {
-        return launch_fused_t<S, 4, VEL>(src, dst, N, zchunk, k, uvel, stream);
+        if (ty == 3 && whole_rows(N)) return launch_fused_t<S, 3, VEL, true>(src, dst, N, zchunk, k, uvel, stream);
+        if (ty == 3) return launch_fused_t<S, 3, VEL>(src, dst, N, zchunk, k, uvel, stream);
+        return launch_fused_t<S, 7, VEL>(src, dst, N, zchunk, k, uvel, stream);
     } else {
+        if (ty == 8 && whole_rows(N)) return launch_fused_t<S, 8, VEL, true>(src, dst, N, zchunk, k, uvel, stream);
         switch (ty) {
             case 4: return launch_fused_t<S, 4, VEL>(src, dst, N, zchunk, k, uvel, stream);
             case 5: return launch_fused_t<S, 5, VEL>(src, dst, N, zchunk, k, uvel, stream);
@@ -94,12 +101,21 @@ cudaError_t dugks_step_fused(int storage, const void* src, void* dst, int N, dou
 namespace {
 
 // What the launch shape is chosen among, with the measured time of one plane
-// of a block (FP32, us): alone on its SM and with the SM's blocks all there.
+// of a block (us): alone on its SM and with the SM's blocks all there.  FP64: a
+// row costs about 18 us of one scheduler's FP64 pipe a plane, so blocks are 4 or 8
+// warps, one or two a scheduler: five (4-row tiles) took as long as eight
+// (32^3 148 -> 90 us a step, 128^3 4.24 -> 3.55 ms).
 struct TileShape {
     int ty, per_sm;
     double alone, shared;
 };
 constexpr TileShape kShapes[] = {{4, 2, 1.5, 1.85}, {5, 2, 1.28, 2.0}, {8, 1, 1.76, 1.76}, {11, 1, 2.1, 2.1}};
+constexpr TileShape kShapes64[] = {{3, 1, 21.3, 21.3}, {7, 1, 41.5, 41.5}};
+
+long long columns(int N, int ty) {
+    const bool wrap = whole_rows(N) && (ty == 3 || ty == 8);
+    return (long long)(wrap ? 1 : (N + 29) / 30) * ((N + ty - 1) / ty);
+}
 
 // Time (us) of the fused DUGKS launch with tiles of shape t and z chunks of zc
 // planes: blocks are issued chunk by chunk (the grid's z index varies slowest),
@@ -110,7 +126,7 @@ constexpr TileShape kShapes[] = {{4, 2, 1.5, 1.85}, {5, 2, 1.28, 2.0}, {8, 1, 1.
 // incomplete wave that are free earlier.
 double makespan(int N, const TileShape& t, int zc, int nsm) {
     constexpr double kPrologue = 1.1;
-    const long long cols = (long long)((N + 29) / 30) * ((N + t.ty - 1) / t.ty);
+    const long long cols = columns(N, t.ty);
     const int full = N / zc, rest = N - full * zc;
     const double plane = cols * (full + (rest > 0)) <= nsm ? t.alone : t.shared;
     const double a = (zc + kPrologue) * plane, b = (rest + kPrologue) * plane;
@@ -138,16 +154,15 @@ double makespan(int N, const TileShape& t, int zc, int nsm) {
 // last wave nearly empty costs up to a third of it.  Every tile height and
 // chunk length is scored by the schedule above and the shortest taken (the
 // longest chunk among those within 0.5 %: fewer halo planes).  Measured against
-// sweeps of all shapes: 32^3 8 x 2 planes 8.2 us (5 x 3: 10.2), 48^3 8 x 4 12.3
+// sweeps of all shapes: 33^3 8 x 2 planes 7.6 us, 48^3 8 x 4 12.3
 // us (5 x 8: 14.4), 64^3 11 x 8 22.5 us (8 x 11: 23.8), 97^3 11 x 25 61.6 us
 // (5 x 13: 66.6), 128^3 11 x 26 117 us (5 x 19: 119), 256^3 11 x 37 0.777 ms
 // (5 x 52: 0.773).
 void dugks_fused_shape(int storage, int N, int nsm, int want_ty, int want_zc, int* ty, int* zc) {
     constexpr long long kMaxBlocks = 20000;
-    const TileShape f64{4, 1, 1.0, 1.0};
     double best = -1.0;
     auto consider = [&](const TileShape& t) {
-        const long long cols = (long long)((N + 29) / 30) * ((N + t.ty - 1) / t.ty);
+        const long long cols = columns(N, t.ty);
         for (int c = want_zc > 0 ? std::min(want_zc, N) : N; c >= 1; --c) {
             const int nz = (N + c - 1) / c;
             if (want_zc <= 0 && nz > 1 && (nz > 64 || cols * nz > kMaxBlocks)) break;
@@ -163,7 +178,7 @@ void dugks_fused_shape(int storage, int N, int nsm, int want_ty, int want_zc, in
         }
     };
     if (storage == ST_F64) {
-        consider(f64);
+        for (const TileShape& t : kShapes64) consider(t);
         return;
     }
     for (const TileShape& t : kShapes)

@@ -320,6 +320,10 @@ __device__ __forceinline__ void face_values(const Rec<C>& P, const Rec<C>& M, co
 }
 
 template <typename C>
+__device__ __forceinline__ Pr<C> pshfl(Pr<C> v, int lane) {
+    return pmk(__shfl_sync(0xffffffffu, v.x, lane), __shfl_sync(0xffffffffu, v.y, lane));
+}
+template <typename C>
 __device__ __forceinline__ Pr<C> pshfl_down1(Pr<C> v) {
     return pmk(__shfl_down_sync(0xffffffffu, v.x, 1), __shfl_down_sync(0xffffffffu, v.y, 1));
 }
@@ -344,8 +348,9 @@ __device__ __forceinline__ int wrapc(int v, int n) {
 // memory at smem_raw (16-byte aligned).  Also called by the persistent
 // ensemble kernel.  With VEL (FP32-computed storage) the tile also writes
 // rho0 u = sum xi f of the stored new state (Eq. 8) to uvel[3][N^3], summed in
-// population order.
-template <typename S, int TY, bool VEL = false>
+// population order.  With WRAP (N <= 32) a warp holds whole periodic rows, lane
+// = x, and needs no x halo: one tile along x where 31 and 32 cells take two.
+template <typename S, int TY, bool VEL = false, bool WRAP = false>
 __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restrict__ dst, int N,
                                            int bx, int by, int bz, int zchunk,
                                            const DugksCoef<typename Traits<S>::C>& kc,
@@ -365,9 +370,13 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
     const unsigned own = opaque((unsigned)__cvta_generic_to_shared(smem_raw) + row * SM::ROW + lane * (int)sizeof(Q4));
     const int z0 = bz * zchunk;
     const int zend = min(z0 + zchunk, N);
-    const int gxr = bx * 30 - 1 + lane, gyr = by * TY - 1 + row;
+    const int gxr = WRAP ? lane : bx * 30 - 1 + lane, gyr = by * TY - 1 + row;
     const int gx = wrapc(gxr, N), gy = wrapc(gyr, N);
-    const bool valid = lane >= 1 && lane <= 30 && gxr < N && gyr < N;
+    const bool valid = (WRAP || (lane >= 1 && lane <= 30)) && gxr < N && gyr < N;
+    // WRAP: the lanes of the x neighbours and their distance in shared memory
+    [[maybe_unused]] const int right = WRAP ? (lane + 1 == N ? 0 : min(lane + 1, 31)) : 0;
+    [[maybe_unused]] const int left = WRAP ? (lane == 0 ? N - 1 : lane - 1) : 0;
+    [[maybe_unused]] const int to_right = (right - lane) * (int)sizeof(Q4), to_left = (left - lane) * (int)sizeof(Q4);
     const size_t plane = (size_t)N * N * N;
     // cell indices fit in 32 bits (N <= 1024)
     const unsigned nn32 = (unsigned)N * N, col32 = (unsigned)gx + (unsigned)N * gy;
@@ -453,8 +462,13 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
     auto diff_x = [&](auto slc, auto kc2, unsigned own) {
         constexpr int O = SM::XCH + decltype(slc)::value * NXQ * SM::QX + decltype(kc2)::value * SM::QX;
         Q4 p, m;
-        lds<O + (int)sizeof(Q4)>(own, p);
-        lds<O - (int)sizeof(Q4)>(own, m);
+        if constexpr (WRAP) {
+            lds<O>(own + to_right, p);
+            lds<O>(own + to_left, m);
+        } else {
+            lds<O + (int)sizeof(Q4)>(own, p);
+            lds<O - (int)sizeof(Q4)>(own, m);
+        }
         return qsub<C>(p, m);
     };
     auto diff_y = [&](auto slc, auto kc2) {
@@ -654,16 +668,17 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
             const Q4 yp = diff_y(slc, k0);
             const P2 g[NC] = {P2{}, yp.a, yp.b, z56.a, z56.b};
             side_records<0, true, true>(cur, g, qadd<C>(ym, zm), kc, Px, Mx);
+            auto from_right = [&](P2 v) { return WRAP ? pshfl<C>(v, right) : pshfl_down1<C>(v); };
 #pragma unroll
-            for (int k = 0; k < NC; ++k) Mn.r[k] = pshfl_down1<C>(Mx.r[k]);
-            Mn.m0 = pshfl_down1<C>(Mx.m0);
-            Mn.m1 = pshfl_down1<C>(Mx.m1);
+            for (int k = 0; k < NC; ++k) Mn.r[k] = from_right(Mx.r[k]);
+            Mn.m0 = from_right(Mx.m0);
+            Mn.m1 = from_right(Mx.m1);
             P2 ffx[NC];
             face_values<0>(Px, Mn, kc, ffx);
             static_for<0, NC>([&](auto kc2) {
                 constexpr int K = decltype(kc2)::value;
                 constexpr int p = cross_pair(0, K);
-                const P2 fl = pshfl_up1<C>(ffx[K]);
+                const P2 fl = WRAP ? pshfl<C>(ffx[K], left) : pshfl_up1<C>(ffx[K]);
                 // Dhat = e_px (F(x + 1/2) - F(x - 1/2)), the first contribution
                 D[p] = pe(p, 0) > 0 ? psub(ffx[K], fl) : psub(fl, ffx[K]);
             });

@@ -31,7 +31,7 @@ cudaError_t dugks_step(int storage, const void* src, void* dst, void* fbp, int N
 cudaError_t dugks_step_fused(int storage, const void* src, void* dst, int N, double nu, double dt,
                              int tile_y, int zchunk, cudaStream_t stream, float* uvel = nullptr);
 
-// Tile height (FP32-computed storage: 4, 5, 8 or 11 rows; FP64: 4) and planes
+// Tile height (FP32-computed storage: 4, 5, 8 or 11 rows; FP64: 3 or 7) and planes
 // per block of the fused step on nsm multiprocessors; want_ty (4 or 8) and
 // want_zc fix one of them where positive.
 void dugks_fused_shape(int storage, int N, int nsm, int want_ty, int want_zc, int* ty, int* zc);

@@ -1,7 +1,7 @@
 """Launch shapes chosen by the library give the bits of the explicit ones.
 
-The fused DUGKS step picks its tile height (5, 8 or 11 rows) and z chunk, the
-LBE step puts two rows in a block for boxes of 33 to 64; a cell's arithmetic
+The fused DUGKS step picks its tile height (5, 8 or 11 rows; FP64 3 or 7) and z
+chunk, and for N = 31 and 32 may hold whole rows in a warp; the LBE step puts two rows in a block for boxes of 33 to 64; a cell's arithmetic
 does not depend on either, so every choice is compared bitwise with 4-row tiles
 of three planes, or with one-warp LBE blocks.  Odd and ragged sizes leave
 partial tiles, chunks and blocks on every side.
@@ -35,10 +35,19 @@ def _run(kin, N, scheme, storage, steps, **tuning):
 
 
 @pytest.mark.parametrize("storage", [0, 1, 2])
-@pytest.mark.parametrize("N", [2, 11, 30, 31, 45, 61, 64, 97])
+@pytest.mark.parametrize("N", [2, 11, 30, 31, 32, 45, 61, 64, 97])
 def test_dugks_default_shape_is_bitwise_the_small_tiles(kin, N, storage):
     ref = _run(kin, N, kin.DUGKS, storage, 2, tile_y=4, zchunk=3)
     np.testing.assert_array_equal(_run(kin, N, kin.DUGKS, storage, 2), ref)
+
+
+@pytest.mark.parametrize("N", [3, 30, 31, 32, 33, 45])
+def test_dugks_fp64_shapes_agree_bitwise(kin, N):
+    """Chunks of 1, 5 and 16 planes take 3- or 7-row tiles and, at 31 and 32,
+    whole-row warps or 30-column tiles."""
+    ref = _run(kin, N, kin.DUGKS, kin.F64, 2)
+    for zc in (1, 5, 16):
+        np.testing.assert_array_equal(_run(kin, N, kin.DUGKS, kin.F64, 2, zchunk=zc), ref)
 
 
 @pytest.mark.parametrize("storage", [0, 1, 2, 3])
