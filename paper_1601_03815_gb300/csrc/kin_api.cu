@@ -1,5 +1,6 @@
 // C ABI of libkin (declared in include/kin.h).
 #include "kin.h"
+#include "host_pages.h"
 #include "kin_common.cuh"
 #include "kin_init.h"
 #include "kin_internal.h"
@@ -96,6 +97,19 @@ int ensure_u(kin_sim* s) {
         s->red_cap = need;
     }
     if (!s->red_out) CK(cudaMalloc(&s->red_out, sizeof(double) * (16 + kin_num_shells(s->N))));
+    return KIN_OK;
+}
+
+// Enqueue the copy of bytes from dev to offset off of the result array behind
+// pages, each part once its pages are there.
+int copy_out(kin_sim* s, HostPages& pages, char* host, size_t off, const void* dev, size_t bytes) {
+    for (size_t at = 0; at < bytes;) {
+        const size_t end = std::min(off + bytes, (off + at) / HostPages::kPart * HostPages::kPart + HostPages::kPart);
+        const size_t n = end - (off + at);
+        pages.wait(end);
+        CK(cudaMemcpyAsync(host + off + at, static_cast<const char*>(dev) + at, n, cudaMemcpyDeviceToHost, s->stream));
+        at += n;
+    }
     return KIN_OK;
 }
 
@@ -422,12 +436,13 @@ int kin_get_f(kin_sim* s, double* f) {
     if (!f) return fail(KIN_EINVAL, "NULL f");
     DeviceGuard g(s->device);
     if (int r = ensure_u(s)) return r;
-    const size_t n = ncell(s);
+    const size_t n = ncell(s), pb = sizeof(double) * n;
+    HostPages pages(f, Q * pb);
     for (int i = 0; i < Q; ++i) {
         CK(get_population(s->storage, i, s->buf[s->cur], shifted(s), s->N, s->u, s->stream));
-        CK(cudaMemcpyAsync(f + (size_t)i * n, s->u, sizeof(double) * n, cudaMemcpyDeviceToHost, s->stream));
-        CK(cudaStreamSynchronize(s->stream));
+        if (int r = copy_out(s, pages, reinterpret_cast<char*>(f), i * pb, s->u, pb)) return r;
     }
+    CK(cudaStreamSynchronize(s->stream));
     return KIN_OK;
 }
 
@@ -465,8 +480,10 @@ int kin_get_velocity(kin_sim* s, double* u) {
     if (!u) return fail(KIN_EINVAL, "NULL u");
     DeviceGuard g(s->device);
     if (int r = ensure_u(s)) return r;
+    const size_t bytes = sizeof(double) * 3 * ncell(s);
+    HostPages pages(u, bytes);
     CK(velocity_field(s->storage, s->buf[s->cur], shifted(s), s->N, s->u, s->stream));
-    CK(cudaMemcpyAsync(u, s->u, sizeof(double) * 3 * ncell(s), cudaMemcpyDeviceToHost, s->stream));
+    if (int r = copy_out(s, pages, reinterpret_cast<char*>(u), 0, s->u, bytes)) return r;
     CK(cudaStreamSynchronize(s->stream));
     return KIN_OK;
 }
