@@ -41,6 +41,12 @@ __host__ __device__ constexpr int cc(int i, int a) { return a == 0 ? cx(i) : a =
 __host__ __device__ constexpr int w36(int i) { return i == 0 ? 12 : (i <= 6 ? 2 : 1); }
 
 // ---------------------------------------------------------------------------
+// a * b, never contracted with a following addition (code that is inlined in
+// several places has to round the same way in each).
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+// ---------------------------------------------------------------------------
 // Compile-time loop: calls f(std::integral_constant<int, I>) for I in [B, E).
 template <int B, int E, typename F>
 __device__ __forceinline__ void static_for(F&& f) {
@@ -132,88 +138,37 @@ __device__ __forceinline__ void moments(const C (&f)[Q], C& drho, C& jx, C& jy, 
 }
 
 // ---------------------------------------------------------------------------
-// MRT moment rows of Sec. II.B as integer polynomials of the velocity.
-__host__ __device__ constexpr int mrow(int k, int x, int y, int z) {
-    const int r2 = x * x + y * y + z * z;
-    switch (k) {
-        case 0: return 1;
-        case 1: return 19 * r2 - 30;
-        case 2: return (21 * r2 * r2 - 53 * r2 + 24) / 2;
-        case 3: return x;
-        case 4: return (5 * r2 - 9) * x;
-        case 5: return y;
-        case 6: return (5 * r2 - 9) * y;
-        case 7: return z;
-        case 8: return (5 * r2 - 9) * z;
-        case 9: return 3 * x * x - r2;
-        case 10: return (3 * r2 - 5) * (3 * x * x - r2);
-        case 11: return y * y - z * z;
-        case 12: return (3 * r2 - 5) * (y * y - z * z);
-        case 13: return x * y;
-        case 14: return y * z;
-        case 15: return x * z;
-        case 16: return (y * y - z * z) * x;
-        case 17: return (z * z - x * x) * y;
-        default: return (x * x - y * y) * z;
-    }
-}
-// Squared norm of row k over the 19 velocities.
-__host__ __device__ constexpr int mnorm(int k) {
-    int s = 0;
-    for (int i = 0; i < Q; ++i) {
-        int v = mrow(k, cx(i), cy(i), cz(i));
-        s += v * v;
-    }
-    return s;
-}
-// Non-conserved rows whose polynomial is even / odd in xi.
-__host__ __device__ constexpr int even_row(int j) {
-    return j == 0 ? 1 : j == 1 ? 2 : j == 2 ? 9 : j == 3 ? 10 : j == 4 ? 11 : j == 5 ? 12 : j == 6 ? 13
-         : j == 7 ? 14 : 15;
-}
-__host__ __device__ constexpr int odd_row(int j) {
-    return j == 0 ? 4 : j == 1 ? 6 : j == 2 ? 8 : j == 3 ? 16 : j == 4 ? 17 : 18;
-}
-constexpr int NEVEN = 9;
-constexpr int NODD = 6;
+// MRT collision (Sec. II.B, RHS of Eq. 21): f <- f - M^-1 S (M f - m_eq), in place.
+//
+// The rows M_k are orthogonal integer polynomials of the velocity, so M^-1 =
+// M^T diag(1 / |M_k|^2) and the change of f_i is sum_k M_ki g_k with
+// g_k = s_k (m_k - m_eq_k) / |M_k|^2.  Rows are even or odd in xi and enter
+// through the pair sums a_p and differences b_p; of these every row needs only
+// the sums over the axis pairs, over the two diagonal pairs of a plane, and
+// their signed counterparts.  With S_ax, S_d the sums of the axis and diagonal
+// a_p and s_xy, s_xz, s_yz those of a plane:
+//   k  polynomial                 m_k                           |M_k|^2   m_eq_k
+//   1  19 r2 - 30                 -30 f0 - 11 S_ax + 8 S_d        2394    -11 drho + 19 j.j
+//   2  (21 r4 - 53 r2 + 24) / 2    12 f0 - 4 S_ax + S_d             252    -475/63 j.j
+//   4  (5 r2 - 9) x  (6 y, 8 z)   j_x - 5 b_x                       40    -2/3 j_x
+//   9  3 x^2 - r2                 A + B                             36    3 j_x^2 - j.j
+//  10  (3 r2 - 5)(3 x^2 - r2)     B - 2 A                           72    0
+//  11  y^2 - z^2                  A' + B'                           12    j_y^2 - j_z^2
+//  12  (3 r2 - 5)(y^2 - z^2)      B' - 2 A'                         24    0
+//  13  x y  (14 y z, 15 x z)      a_3 - a_4                          4    j_x j_y
+//  16  (y^2 - z^2) x  (17, 18)    x part of the xy pairs - xz pairs   8    0
+// (A = 3 a_x - S_ax, B = S_d - 3 s_yz, A' = a_y - a_z, B' = s_xy - s_xz;
+// omega_eps = omega_xx = 0, omega_epsj = -475/63, rho0 = 1; m_1 - m_eq_1 =
+// 19 (S_d - f0 - j.j)).  About 165 operations a cell, against 290 with every row
+// summed by itself: the 2-byte step and FP64 were bound by them (256^3 FP16
+// 214 -> 184 us, its copy roof; 64^3 FP64 135 -> 78 us).
 
-// Relaxation rates (Sec. II.B, values of Sec. IV.A).
+// s_k / |M_k|^2 (with the constant factors of the table) for the rates of Sec. IV.A.
 template <typename C>
 struct MrtRates {
-    C s1, s2, s4, s9, s10, s13, s16;
+    C c1, c2, c4, c9, c10, c11, c12, c13, c16;
 };
-template <int K, typename C>
-__device__ __forceinline__ C rate(const MrtRates<C>& r) {
-    if constexpr (K == 1) return r.s1;
-    else if constexpr (K == 2) return r.s2;
-    else if constexpr (K == 4 || K == 6 || K == 8) return r.s4;
-    else if constexpr (K == 9 || K == 11) return r.s9;
-    else if constexpr (K == 10 || K == 12) return r.s10;
-    else if constexpr (K == 13 || K == 14 || K == 15) return r.s13;
-    else return r.s16;
-}
 
-// Equilibrium moments (Sec. II.B with omega_eps = omega_xx = 0,
-// omega_epsj = -475/63, rho0 = 1).  Slot 9 holds 3 p_xx.
-template <int K, typename C>
-__device__ __forceinline__ C meq(C drho, C jx, C jy, C jz, C jj) {
-    if constexpr (K == 1) return C(-11) * drho + C(19) * jj;
-    else if constexpr (K == 2) return C(-475.0 / 63.0) * jj;
-    else if constexpr (K == 4) return C(-2.0 / 3.0) * jx;
-    else if constexpr (K == 6) return C(-2.0 / 3.0) * jy;
-    else if constexpr (K == 8) return C(-2.0 / 3.0) * jz;
-    else if constexpr (K == 9) return C(2) * jx * jx - (jy * jy + jz * jz);
-    else if constexpr (K == 11) return jy * jy - jz * jz;
-    else if constexpr (K == 13) return jx * jy;
-    else if constexpr (K == 14) return jy * jz;
-    else if constexpr (K == 15) return jx * jz;
-    else return C(0);  // rows 10, 12 (omega_xx = 0) and 16-18
-}
-
-// One MRT collision in place (RHS of Eq. 21): f <- f - M^-1 S (M f - m_eq).
-// M is orthogonal, so M^-1 = M^T diag(1/|M_k|^2); rows are even or odd in xi,
-// so the work splits into the pair sums a_p = f_{2p+1} + f_{2p+2} (even rows)
-// and differences b_p = f_{2p+1} - f_{2p+2} (odd rows).
 // FIXJ: the equilibrium takes the prescribed momentum (jfx, jfy, jfz) and the
 // momentum rows relax fully to it (the consistent initialisation, Sec. IV.A);
 // otherwise the cell's own momentum, conserved.
@@ -227,82 +182,93 @@ __device__ __forceinline__ void mrt_collide_t(C (&f)[Q], const MrtRates<C>& r, C
         b[p] = f[2 * p + 1] - f[2 * p + 2];
     }
     const C f0 = f[0];
-    const C drho = f0 + ((a[0] + a[1]) + a[2]) + (((a[3] + a[4]) + (a[5] + a[6])) + (a[7] + a[8]));
-    const C jx = (b[0] + b[3]) + (b[4] + (b[5] + b[6]));
-    const C jy = (b[1] + b[3]) - (b[4] - (b[7] + b[8]));
-    const C jz = (b[2] + b[5]) - (b[6] - (b[7] - b[8]));
+    const C sxy = a[3] + a[4], sxz = a[5] + a[6], syz = a[7] + a[8];
+    const C sax = (a[0] + a[1]) + a[2], sd = (sxy + sxz) + syz;
+    // the x, y, z parts of the diagonal pairs of a plane
+    const C xxy = b[3] + b[4], xxz = b[5] + b[6];
+    const C yxy = b[3] - b[4], yyz = b[7] + b[8];
+    const C zxz = b[5] - b[6], zyz = b[7] - b[8];
+    const C drho = f0 + (sax + sd);
+    const C jx = b[0] + (xxy + xxz), jy = b[1] + (yxy + yyz), jz = b[2] + (zxz + zyz);
     drho_out = drho;
     jx_out = jx;
     jy_out = jy;
     jz_out = jz;
-    const C jxe = FIXJ ? jfx : jx, jye = FIXJ ? jfy : jy, jze = FIXJ ? jfz : jz;
-    const C jj = jxe * jxe + jye * jye + jze * jze;
-    // FIXJ: (m - m_eq) / |M_k|^2 of the momentum rows at rate 1 (|M_3|^2 = 10)
-    [[maybe_unused]] const C gjx = (jx - jfx) * C(0.1), gjy = (jy - jfy) * C(0.1), gjz = (jz - jfz) * C(0.1);
+    const C ex = FIXJ ? jfx : jx, ey = FIXJ ? jfy : jy, ez = FIXJ ? jfz : jz;  // momentum of m_eq
+    // (products that meet a plain addition go through mul_rn, so that every
+    // kernel this is inlined in rounds alike)
+    const C xx = mul_rn(ex, ex), yy = mul_rn(ey, ey);
+    const C jj = fma(ez, ez, xx + yy);
 
-    C ge[NEVEN], go[NODD];
-    static_for<0, NEVEN>([&](auto jc) {
-        constexpr int J = decltype(jc)::value;
-        constexpr int K = even_row(J);
-        C m = C(mrow(K, 0, 0, 0)) * f0;
-        static_for<0, NPAIR>([&](auto pc) {
-            constexpr int P = decltype(pc)::value;
-            constexpr int c = mrow(K, pair_x(P), pair_y(P), pair_z(P));
-            if constexpr (c == 1) m += a[P];
-            else if constexpr (c == -1) m -= a[P];
-            else if constexpr (c != 0) m += C(c) * a[P];
-        });
-        ge[J] = rate<K>(r) * (m - meq<K>(drho, jxe, jye, jze, jj)) * (C(1) / C(mnorm(K)));
-    });
-    static_for<0, NODD>([&](auto jc) {
-        constexpr int J = decltype(jc)::value;
-        constexpr int K = odd_row(J);
-        C m = C(0);
-        static_for<0, NPAIR>([&](auto pc) {
-            constexpr int P = decltype(pc)::value;
-            constexpr int c = mrow(K, pair_x(P), pair_y(P), pair_z(P));
-            if constexpr (c == 1) m += b[P];
-            else if constexpr (c == -1) m -= b[P];
-            else if constexpr (c != 0) m += C(c) * b[P];
-        });
-        go[J] = rate<K>(r) * (m - meq<K>(drho, jxe, jye, jze, jj)) * (C(1) / C(mnorm(K)));
-    });
-    // back transform: df_i = sum_k M_k,i g_k
-    {
-        C d0 = C(0);
-        static_for<0, NEVEN>([&](auto jc) {
-            constexpr int J = decltype(jc)::value;
-            constexpr int c = mrow(even_row(J), 0, 0, 0);
-            if constexpr (c != 0) d0 += C(c) * ge[J];
-        });
-        f[0] = f0 - d0;
+    const C g1 = mul_rn(r.c1, ((sd - f0) - jj));
+    const C g2 = mul_rn(r.c2, fma(C(475.0 / 63.0), jj, fma(C(12), f0, fma(C(-4), sax, sd))));
+    const C A9 = fma(C(3), a[0], -sax), B9 = fma(C(-3), syz, sd);
+    const C g9 = mul_rn(r.c9, fma(C(-3), xx, (A9 + B9) + jj));
+    const C g10 = mul_rn(r.c10, fma(C(-2), A9, B9));
+    const C A11 = a[1] - a[2], B11 = sxy - sxz;
+    const C g11 = mul_rn(r.c11, fma(ez, ez, (A11 + B11) - yy));
+    const C g12 = mul_rn(r.c12, fma(C(-2), A11, B11));
+    const C g13 = mul_rn(r.c13, fma(-ex, ey, a[3] - a[4]));
+    const C g14 = mul_rn(r.c13, fma(-ey, ez, a[7] - a[8]));
+    const C g15 = mul_rn(r.c13, fma(-ex, ez, a[5] - a[6]));
+    // c4 carries the factor 5 of j - 5 b
+    C g4, g6, g8;
+    if constexpr (FIXJ) {
+        g4 = mul_rn(r.c4, fma(C(0.2), fma(C(2.0 / 3.0), ex, jx), -b[0]));
+        g6 = mul_rn(r.c4, fma(C(0.2), fma(C(2.0 / 3.0), ey, jy), -b[1]));
+        g8 = mul_rn(r.c4, fma(C(0.2), fma(C(2.0 / 3.0), ez, jz), -b[2]));
+    } else {
+        g4 = mul_rn(r.c4, fma(C(1.0 / 3.0), jx, -b[0]));
+        g6 = mul_rn(r.c4, fma(C(1.0 / 3.0), jy, -b[1]));
+        g8 = mul_rn(r.c4, fma(C(1.0 / 3.0), jz, -b[2]));
     }
-    static_for<0, NPAIR>([&](auto pc) {
-        constexpr int P = decltype(pc)::value;
-        C e = C(0), o = C(0);
-        static_for<0, NEVEN>([&](auto jc) {
-            constexpr int J = decltype(jc)::value;
-            constexpr int c = mrow(even_row(J), pair_x(P), pair_y(P), pair_z(P));
-            if constexpr (c == 1) e += ge[J];
-            else if constexpr (c == -1) e -= ge[J];
-            else if constexpr (c != 0) e += C(c) * ge[J];
-        });
-        static_for<0, NODD>([&](auto jc) {
-            constexpr int J = decltype(jc)::value;
-            constexpr int c = mrow(odd_row(J), pair_x(P), pair_y(P), pair_z(P));
-            if constexpr (c == 1) o += go[J];
-            else if constexpr (c == -1) o -= go[J];
-            else if constexpr (c != 0) o += C(c) * go[J];
-        });
-        if constexpr (FIXJ) {
-            // the momentum rows (M_3,5,7 = xi_x, xi_y, xi_z) relaxed with rate 1
-            if constexpr (pair_x(P) != 0) o += C(pair_x(P)) * gjx;
-            if constexpr (pair_y(P) != 0) o += C(pair_y(P)) * gjy;
-            if constexpr (pair_z(P) != 0) o += C(pair_z(P)) * gjz;
-        }
-        f[2 * P + 1] -= e + o;
-        f[2 * P + 2] -= e - o;
-    });
+    const C g16 = mul_rn(r.c16, xxy - xxz), g17 = mul_rn(r.c16, yyz - yxy), g18 = mul_rn(r.c16, zxz - zyz);
+
+    // back transform: df_i = sum_k M_ki g_k, even part e and odd part o of a pair
+    f[0] = f0 - fma(C(-30), g1, C(12) * g2);
+    C e[NPAIR], o[NPAIR];
+    const C eax = fma(C(-11), g1, C(-4) * g2);
+    const C h9 = fma(C(-2), g10, g9), h11 = fma(C(-2), g12, g11);
+    e[0] = fma(C(2), h9, eax);
+    e[1] = (eax - h9) + h11;
+    e[2] = (eax - h9) - h11;
+    const C ed = fma(C(8), g1, g2);
+    const C k9 = g9 + g10, k11 = g11 + g12;
+    const C exy = (ed + k9) + k11, exz = (ed + k9) - k11, eyz = fma(C(-2), k9, ed);
+    e[3] = exy + g13;
+    e[4] = exy - g13;
+    e[5] = exz + g15;
+    e[6] = exz - g15;
+    e[7] = eyz + g14;
+    e[8] = eyz - g14;
+    o[0] = mul_rn(C(-4), g4);
+    o[1] = mul_rn(C(-4), g6);
+    o[2] = mul_rn(C(-4), g8);
+    C x1 = g4 + g16, x2 = g4 - g16, y1 = g6 - g17, y2 = g6 + g17, z1 = g8 + g18, z2 = g8 - g18;
+    if constexpr (FIXJ) {
+        // the momentum rows (M_3,5,7 = xi_x, xi_y, xi_z) relaxed with rate 1, |M_3|^2 = 10
+        const C gx = mul_rn(jx - jfx, C(0.1)), gy = mul_rn(jy - jfy, C(0.1)), gz = mul_rn(jz - jfz, C(0.1));
+        o[0] += gx;
+        o[1] += gy;
+        o[2] += gz;
+        x1 += gx;
+        x2 += gx;
+        y1 += gy;
+        y2 += gy;
+        z1 += gz;
+        z2 += gz;
+    }
+    o[3] = x1 + y1;
+    o[4] = x1 - y1;
+    o[5] = x2 + z1;
+    o[6] = x2 - z1;
+    o[7] = y2 + z2;
+    o[8] = y2 - z2;
+#pragma unroll
+    for (int p = 0; p < NPAIR; ++p) {
+        f[2 * p + 1] -= e[p] + o[p];
+        f[2 * p + 2] -= e[p] - o[p];
+    }
 }
 
 template <typename C>

@@ -14,17 +14,21 @@
 
 namespace kin {
 
-// Sec. IV.A rates with dt = dx = 1.
+// Sec. IV.A rates with dt = dx = 1: s1 = 1.19, s2 = s10 = 1.4, s4 = 1.2, s16 =
+// 1.98, s9 = s13 = 1 / (3 nu + 1/2), over the rows' squared norms.
 template <typename C>
 inline MrtRates<C> lbe_rates(double nu) {
+    const double s9 = 1.0 / (3.0 * nu + 0.5);
     MrtRates<C> r;
-    r.s1 = C(1.19);
-    r.s2 = C(1.4);
-    r.s4 = C(1.2);
-    r.s9 = C(1.0 / (3.0 * nu + 0.5));
-    r.s10 = C(1.4);
-    r.s13 = r.s9;
-    r.s16 = C(1.98);
+    r.c1 = C(1.19 * 19.0 / 2394.0);
+    r.c2 = C(1.4 / 252.0);
+    r.c4 = C(1.2 * 5.0 / 40.0);
+    r.c9 = C(s9 / 36.0);
+    r.c10 = C(1.4 / 72.0);
+    r.c11 = C(s9 / 12.0);
+    r.c12 = C(1.4 / 24.0);
+    r.c13 = C(s9 / 4.0);
+    r.c16 = C(1.98 / 8.0);
     return r;
 }
 

@@ -79,11 +79,6 @@ __device__ __forceinline__ double2 psub(double2 a, double2 b) {
 }
 __device__ __forceinline__ double2 pneg(double2 a) { return make_double2(-a.x, -a.y); }
 
-// a * b, never contracted with a following addition (code that is inlined in
-// several places has to round the same way in each)
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-
 // acc + SG * v for a compile-time sign SG = +1 or -1
 template <int SG, typename T>
 __device__ __forceinline__ T padd_sg(T acc, T v) {
