@@ -5,6 +5,7 @@
 #include "dugks_tile.cuh"
 #include "kin_internal.h"
 #include "kin_launch.cuh"
+#include "tile_schedule.h"
 
 namespace kin {
 
@@ -118,34 +119,12 @@ long long columns(int N, int ty) {
 }
 
 // Time (us) of the fused DUGKS launch with tiles of shape t and z chunks of zc
-// planes: blocks are issued chunk by chunk (the grid's z index varies slowest),
-// each to the SM slot that frees first, and occupy it for their planes plus
-// about 1.1 plane-times of prologue (two pre-steps and one record before the
-// first face).  All chunks but the last are equal, so whole waves are counted
-// and only the last chunk's blocks are placed, on the slots of the last
-// incomplete wave that are free earlier.
+// planes; a block's prologue (two pre-steps and one record before the first
+// face) takes about 1.1 plane-times.
 double makespan(int N, const TileShape& t, int zc, int nsm) {
-    constexpr double kPrologue = 1.1;
     const long long cols = columns(N, t.ty);
-    const int full = N / zc, rest = N - full * zc;
-    const double plane = cols * (full + (rest > 0)) <= nsm ? t.alone : t.shared;
-    const double a = (zc + kPrologue) * plane, b = (rest + kPrologue) * plane;
-    const long long slots = (long long)nsm * t.per_sm;
-    const long long late = cols * full % slots;  // slots one wave ahead of the others
-    double early_at = (double)(cols * full / slots) * a, late_at = early_at + a;
-    double end = late > 0 ? late_at : early_at;
-    for (long long left = rest > 0 ? cols : 0; left > 0;) {
-        if (late == 0 || early_at <= late_at) {
-            left -= slots - late;
-            early_at += b;
-            end = std::max(end, early_at);
-        } else {
-            left -= late;
-            late_at += b;
-            end = std::max(end, late_at);
-        }
-    }
-    return end;
+    const double plane = cols * ((N + zc - 1) / zc) <= nsm ? t.alone : t.shared;
+    return plane * tile_schedule(cols, N, zc, (long long)nsm * t.per_sm, 1.1);
 }
 
 }  // namespace

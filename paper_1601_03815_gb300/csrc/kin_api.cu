@@ -176,6 +176,24 @@ int launch_step(kin_sim* s, float* uvel = nullptr) {
     return KIN_OK;
 }
 
+// n steps; the last one with uvel as in launch_step.  LBE steps go in pairs where
+// one pass over memory for two of them is the faster way (an explicit block size
+// keeps the single-step kernel it is meant for).
+int launch_steps(kin_sim* s, int n, float* uvel) {
+    int k = 0;
+    if (s->scheme == KIN_LBE_MRT && s->block_lbe == 0 && lbe_pairs(s->storage, s->N))
+        for (; k + 2 <= n; k += 2) {
+            CK(lbe_pair_step(s->buf[s->cur], s->buf[s->cur ^ 1], s->N, s->nu, s->num_sms, s->stream));
+            s->launches += 1;
+            s->cur ^= 1;
+            s->step += 2;
+            s->epoch += 1;
+        }
+    for (; k < n; ++k)
+        if (int r = launch_step(s, k == n - 1 ? uvel : nullptr)) return r;
+    return KIN_OK;
+}
+
 // Enqueue E and eps of the current state into red_out[0..1] (device) and, where
 // host is not NULL, into that device-accessible host memory (with_err: followed
 // by the error word).
@@ -493,9 +511,7 @@ int kin_step(kin_sim* s, int n) {
     if (int r = usable(s)) return r;
     if (n < 0) return fail(KIN_EINVAL, "negative step count");
     DeviceGuard g(s->device);
-    for (int k = 0; k < n; ++k)
-        if (int r = launch_step(s)) return r;
-    return KIN_OK;
+    return launch_steps(s, n, nullptr);
 }
 
 int kin_step_stats(kin_sim* s, int n, double* E, double* eps, double* Ek) {
@@ -505,8 +521,7 @@ int kin_step_stats(kin_sim* s, int n, double* E, double* eps, double* Ek) {
     DeviceGuard g(s->device);
     const bool fuse = n > 0 && fused_velocity_ok(s);
     if (fuse && !s->u32) CK(cudaMalloc(&s->u32, sizeof(float) * 3 * ncell(s)));
-    for (int k = 0; k < n; ++k)
-        if (int r = launch_step(s, fuse && k == n - 1 ? s->u32 : nullptr)) return r;
+    if (int r = launch_steps(s, n, fuse ? s->u32 : nullptr)) return r;
     return kin_stats(s, E, eps, Ek);
 }
 
@@ -531,8 +546,7 @@ int kin_step_stats_async(kin_sim* s, int n, double* out) {
     DeviceGuard g(s->device);
     const bool fuse = n > 0 && fused_velocity_ok(s);
     if (fuse && !s->u32) CK(cudaMalloc(&s->u32, sizeof(float) * 3 * ncell(s)));
-    for (int k = 0; k < n; ++k)
-        if (int r = launch_step(s, fuse && k == n - 1 ? s->u32 : nullptr)) return r;
+    if (int r = launch_steps(s, n, fuse ? s->u32 : nullptr)) return r;
     return kin_stats_async(s, out);
 }
 

@@ -3,8 +3,11 @@
 #include "kin_internal.h"
 #include "kin_launch.cuh"
 #include "lbe_node.cuh"
+#include "lbe_pair.cuh"
+#include "tile_schedule.h"
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 
 namespace kin {
@@ -124,6 +127,42 @@ cudaError_t lbe_consistent_step(int storage, const void* src, void* dst, int N, 
         case ST_F64: return launch_consistent<double>(src, dst, N, nu, u0, stream);
     }
     return cudaErrorInvalidValue;
+}
+
+// Two steps in one pass pay where the state does not stay in L2 between steps:
+// us a step, single / paired: 64^3 5.2 / 7.6 (40 MB of state), 97^3 24.6 / 21.0,
+// 128^3 47.9 / 37.9, 256^3 367 / 257; level between 84^3 and 88^3 (14.1 / 12.2).
+bool lbe_pairs(int storage, int N) { return storage == ST_F32 && N >= 88; }
+
+cudaError_t lbe_pair_step(const void* src, void* dst, int N, double nu, int nsm, cudaStream_t stream) {
+    constexpr int TY = kPairRows;
+    constexpr size_t smem = sizeof(float) * LbePairSmem<TY>::FLOATS;
+    static std::atomic<unsigned long long> configured{0};  // devices whose shared-memory limit is set
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (!bit || !(configured.load() & bit)) {
+        e = cudaFuncSetAttribute(lbe_pair_kernel<TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        configured.fetch_or(bit);
+    }
+    // planes a block: the shortest schedule, of at most 64 chunks (a block relaxes
+    // two planes before its first result)
+    const long long cols = (long long)((N + 29) / 30) * ((N + TY - 1) / TY);
+    int zc = N;
+    double best = -1.0;
+    for (int nz = 1; nz <= 64 && nz <= N; ++nz) {
+        const int c = (N + nz - 1) / nz;
+        const double t = tile_schedule(cols, N, c, (long long)nsm * kPairBlocks, 2.0);
+        if (best < 0.0 || t < best) {
+            best = t;
+            zc = c;
+        }
+    }
+    const dim3 grid((N + 29) / 30, (N + TY - 1) / TY, (N + zc - 1) / zc);
+    return launch_next(lbe_pair_kernel<TY>, grid, dim3(32, TY + 2), smem, stream, (const float*)src, (float*)dst, N,
+                       (size_t)N * N * N, zc, lbe_rates<float>(nu));
 }
 
 KIN_DEBUG_ACCESSOR(debug_word_lbe)

@@ -58,6 +58,16 @@ def test_lbe_default_blocks_are_bitwise_the_one_warp_blocks(kin, N, storage):
     np.testing.assert_array_equal(_run(kin, N, kin.LBE_MRT, storage, 3, block_x=256), ref)
 
 
+@pytest.mark.parametrize("steps", [2, 5])
+@pytest.mark.parametrize("N", [87, 88, 89, 97, 121])
+def test_lbe_step_pairs_are_bitwise_single_steps(kin, N, steps):
+    """From 88^3 on FP32 steps go in pairs (one pass over memory); an explicit
+    block size keeps the single-step kernel.  Edges: tiles of 30 x 6 cells and z
+    chunks with remainders, an odd step left over."""
+    ref = _run(kin, N, kin.LBE_MRT, kin.F32, steps, block_x=128)
+    np.testing.assert_array_equal(_run(kin, N, kin.LBE_MRT, kin.F32, steps), ref)
+
+
 @pytest.mark.parametrize("scheme", [0, 1])
 def test_steps_captured_in_a_graph(kin, scheme):
     """Steps launched to overlap the one before them, replayed from a graph."""
