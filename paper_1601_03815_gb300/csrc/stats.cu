@@ -166,9 +166,11 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// Sums of a and b over the block, in thread 0 (warps, then the block, in order).
+// Sums of a and b over the block, in thread 0: warps by shuffles, then the warps'
+// sums by shuffles of the first (a chain of 8 FP64 additions, each ~60 cycles).
 __device__ __forceinline__ void block_sum2(double& a, double& b) {
-    __shared__ double sh[2][RED_THREADS / 32];
+    constexpr int W = RED_THREADS / 32;
+    __shared__ double sh[2][W];
     a = warp_sum(a);
     b = warp_sum(b);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -178,18 +180,30 @@ __device__ __forceinline__ void block_sum2(double& a, double& b) {
         sh[1][wid] = b;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        a = b = 0.0;
-        for (int w = 0; w < RED_THREADS / 32; ++w) {
-            a += sh[0][w];
-            b += sh[1][w];
+    if (wid == 0) {
+        a = sh[0][lane % W];
+        b = sh[1][lane % W];
+#pragma unroll
+        for (int o = W / 2; o > 0; o >>= 1) {
+            a += __shfl_down_sync(0xffffffffu, a, o);
+            b += __shfl_down_sync(0xffffffffu, b, o);
         }
     }
 }
 
+// E = <u.u> / 2 and eps = 2 nu <s_ab s_ab> of the sums, as factors (two FP64
+// divisions at the end of the reduction took 1.4 us).
+struct EdScale {
+    double E, eps;
+};
+static EdScale ed_scale(int N, double nu) {
+    const double n = (double)N * N * N;
+    return EdScale{0.5 / n, 2.0 * nu / n};
+}
+
 // Fixed-order sum of the block partials {sum |u|^2, sum s_ab s_ab} by one block:
 // thread t takes partials t, t + RED_THREADS, ..., then block_sum2.
-__device__ __forceinline__ void ed_total(const double* partial, int nblocks, size_t n, double nu, const EdSink& sink) {
+__device__ __forceinline__ void ed_total(const double* partial, int nblocks, const EdScale& scale, const EdSink& sink) {
     double a = 0.0, b = 0.0;
     for (int i = threadIdx.x; i < nblocks; i += RED_THREADS) {
         a += __ldcg(partial + 2 * i);
@@ -197,7 +211,7 @@ __device__ __forceinline__ void ed_total(const double* partial, int nblocks, siz
     }
     block_sum2(a, b);
     if (threadIdx.x == 0) {
-        const double E = 0.5 * a / (double)n, eps = 2.0 * nu * b / (double)n;
+        const double E = a * scale.E, eps = b * scale.eps;
         sink.out[0] = E;
         sink.out[1] = eps;
         if (sink.host) {
@@ -211,7 +225,7 @@ __device__ __forceinline__ void ed_total(const double* partial, int nblocks, siz
 // A block's sums into its partial; the last block to get here (counter, which
 // wraps to zero for the next call) forms the total.  One launch instead of two:
 // the one-block total took 6 us of its own.
-__device__ __forceinline__ void ed_block_done(double a, double b, double* partial, size_t n, double nu,
+__device__ __forceinline__ void ed_block_done(double a, double b, double* partial, const EdScale& scale,
                                               const EdSink& sink) {
     block_sum2(a, b);
     if (threadIdx.x == 0) {
@@ -227,7 +241,7 @@ __device__ __forceinline__ void ed_block_done(double a, double b, double* partia
     __syncthreads();
     if (!last) return;
     __threadfence();
-    ed_total(partial, gridDim.x, n, nu, sink);
+    ed_total(partial, gridDim.x, scale, sink);
 }
 
 // Reduction of |u|^2 and s_ab s_ab in FP64; each thread walks a fixed
@@ -235,7 +249,7 @@ __device__ __forceinline__ void ed_block_done(double a, double b, double* partia
 // s_ab s_ab = sum_a g_aa^2 / 4 + sum_{a<b} (g_ab + g_ba)^2 / 8: 21 FP64
 // operations a cell (they are what bounds the kernel), the factors exact.
 __global__ void __launch_bounds__(RED_THREADS)
-    ed_partial_kernel(const double* u, int N, double nu, double* partial, EdSink sink) {
+    ed_partial_kernel(const double* u, int N, EdScale scale, double* partial, EdSink sink) {
     grid_begin();
     const size_t n = (size_t)N * N * N;
     const double* U[3] = {u, u + n, u + 2 * n};
@@ -262,7 +276,7 @@ __global__ void __launch_bounds__(RED_THREADS)
             se = fma(v, v, se);
         }
     }
-    ed_block_done(se, 0.25 * sd + 0.125 * so, partial, n, nu, sink);
+    ed_block_done(se, 0.25 * sd + 0.125 * so, partial, scale, sink);
 }
 
 // One cell's |u|^2 and s_ab s_ab in FP32 (the form of ed_partial_kernel), formed
@@ -280,7 +294,7 @@ __device__ __forceinline__ void add_cell(const float (&g)[3][3], const float (&u
 // |u|^2 and s_ab s_ab are formed in FP32, summed in FP32 over at most 8 rows
 // and then in FP64, in a fixed order.
 __global__ void __launch_bounds__(RED_THREADS)
-    ed32_partial_kernel(const float* u, int N, double nu, double* partial, EdSink sink) {
+    ed32_partial_kernel(const float* u, int N, EdScale scale, double* partial, EdSink sink) {
     grid_begin();
     const size_t n = (size_t)N * N * N;
     // component bases; offsets inside a component fit in 32 bits (N <= 1024)
@@ -315,7 +329,7 @@ __global__ void __launch_bounds__(RED_THREADS)
     }
     se += (double)fe;
     ss += (double)fs;
-    ed_block_done(se, ss, partial, n, nu, sink);
+    ed_block_done(se, ss, partial, scale, sink);
 }
 
 // The same for N a multiple of 4, four cells per thread: a thread reads its
@@ -325,7 +339,7 @@ __global__ void __launch_bounds__(RED_THREADS)
 // terms of a thread's cells are summed in cell order, in FP32 over at most 8
 // row groups and then in FP64.
 __global__ void __launch_bounds__(RED_THREADS)
-    ed32v4_partial_kernel(const float* u, int N, double nu, double* partial, EdSink sink) {
+    ed32v4_partial_kernel(const float* u, int N, EdScale scale, double* partial, EdSink sink) {
     grid_begin();
     const size_t n = (size_t)N * N * N;
     const float* U[3] = {u, u + n, u + 2 * n};
@@ -385,22 +399,21 @@ __global__ void __launch_bounds__(RED_THREADS)
     }
     se += (double)fe;
     ss += (double)fs;
-    ed_block_done(se, ss, partial, n, nu, sink);
+    ed_block_done(se, ss, partial, scale, sink);
 }
 
 __global__ void __launch_bounds__(RED_THREADS)
-    ed_final_kernel(const double* partial, int nblocks, size_t n, double nu, EdSink sink) {
+    ed_final_kernel(const double* partial, int nblocks, EdScale scale, EdSink sink) {
     grid_begin();
-    ed_total(partial, nblocks, n, nu, sink);
+    ed_total(partial, nblocks, scale, sink);
 }
 
 cudaError_t energy_dissipation(const double* u, int N, double nu, double* partials, const EdSink& sink,
                                cudaStream_t stream) {
     const int nb = stats_blocks(N);
-    cudaError_t e = launch_next(ed_partial_kernel, nb, RED_THREADS, 0, stream, u, N, nu, partials, sink);
+    cudaError_t e = launch_next(ed_partial_kernel, nb, RED_THREADS, 0, stream, u, N, ed_scale(N, nu), partials, sink);
     if (e != cudaSuccess || sink.counter) return e;
-    return launch_next(ed_final_kernel, 1, RED_THREADS, 0, stream, (const double*)partials, nb, (size_t)N * N * N, nu,
-                       sink);
+    return launch_next(ed_final_kernel, 1, RED_THREADS, 0, stream, (const double*)partials, nb, ed_scale(N, nu), sink);
 }
 
 cudaError_t energy_dissipation32(const float* u, int N, double nu, double* partials, const EdSink& sink,
@@ -408,10 +421,10 @@ cudaError_t energy_dissipation32(const float* u, int N, double nu, double* parti
     if (N % 4 == 0 && N / 4 <= RED_THREADS) {
         const int rows = RED_THREADS / (N / 4);  // a block's rows at a time
         const int nb = std::min(stats_blocks(N), (N * N + rows - 1) / rows);
-        return launch_next(ed32v4_partial_kernel, nb, RED_THREADS, 0, stream, u, N, nu, partials, sink);
+        return launch_next(ed32v4_partial_kernel, nb, RED_THREADS, 0, stream, u, N, ed_scale(N, nu), partials, sink);
     }
-    return launch_next(ed32_partial_kernel, std::min(stats_blocks(N), N * N), RED_THREADS, 0, stream, u, N, nu, partials,
-                       sink);
+    return launch_next(ed32_partial_kernel, std::min(stats_blocks(N), N * N), RED_THREADS, 0, stream, u, N,
+                       ed_scale(N, nu), partials, sink);
 }
 
 // ---------------------------------------------------------------------------
