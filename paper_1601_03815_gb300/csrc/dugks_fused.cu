@@ -1,8 +1,8 @@
 // Standalone launch of the fused DUGKS step (tile code in dugks_tile.cuh).
 #include <algorithm>
-#include <atomic>
 
 #include "dugks_tile.cuh"
+#include "dugks_tile16.cuh"
 #include "kin_internal.h"
 #include "kin_launch.cuh"
 #include "tile_schedule.h"
@@ -33,25 +33,47 @@ template <typename S, int TY, bool VEL, bool WRAP = false>
 static cudaError_t launch_fused_t(const void* src, void* dst, int N, int zchunk,
                                   const DugksCoef<typename Traits<S>::C>& k, float* uvel, cudaStream_t stream) {
     const size_t smem = fused_smem_bytes<S, TY>();
-    // the shared-memory limit is a per-device attribute of the kernel: set it
-    // once for every device this process launches on
-    static std::atomic<unsigned long long> configured{0};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    const cudaError_t e = allow_smem<dugks_fused_kernel<S, TY, VEL, WRAP>>(smem);
     if (e != cudaSuccess) return e;
-    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
-    if (!bit || !(configured.load() & bit)) {
-        e = cudaFuncSetAttribute(dugks_fused_kernel<S, TY, VEL, WRAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
-        if (e != cudaSuccess) return e;
-        configured.fetch_or(bit);
-    }
     if (zchunk <= 0) zchunk = 32;
     if (zchunk > N) zchunk = N;
     dim3 block(32, TY + 1);
     dim3 grid(WRAP ? 1 : (N + 29) / 30, (N + TY - 1) / TY, (N + zchunk - 1) / zchunk);
     return launch_next(dugks_fused_kernel<S, TY, VEL, WRAP>, grid, block, smem, stream, (const S*)src, (S*)dst, N, zchunk, k,
                        uvel);
+}
+
+// FP16 and BF16 storage.  EVEN = false: odd N, whose tile reads f-tilde from global
+// memory instead of staging it.
+template <typename S, int TY, bool VEL, bool EVEN>
+__global__ void __launch_bounds__(32 * (TY + 2), 1)
+    dugks_fused16_kernel(const S* __restrict__ src, S* __restrict__ dst, int N, int zchunk, DugksCoef<float> kc,
+                         float* __restrict__ uvel) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    two_byte::dugks_tile<S, TY, VEL, EVEN>(src, dst, N, blockIdx.x, blockIdx.y, blockIdx.z, zchunk, kc, smem_raw, uvel);
+}
+
+template <typename S, int TY, bool VEL, bool EVEN>
+static cudaError_t launch_fused16_t(const void* src, void* dst, int N, int zchunk, const DugksCoef<float>& k,
+                                    float* uvel, cudaStream_t stream) {
+    const size_t smem = two_byte::tile_smem_bytes<S, TY>();
+    const cudaError_t e = allow_smem<dugks_fused16_kernel<S, TY, VEL, EVEN>>(smem);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((N + 29) / 30, (N + TY - 1) / TY, (N + zchunk - 1) / zchunk);
+    // an ordinary launch: its copies go through L1
+    dugks_fused16_kernel<S, TY, VEL, EVEN><<<grid, dim3(32, TY + 2), smem, stream>>>((const S*)src, (S*)dst, N, zchunk, k,
+                                                                                    uvel);
+    return cudaGetLastError();
+}
+
+template <typename S, bool VEL>
+static cudaError_t launch_fused16(const void* src, void* dst, int N, const DugksCoef<float>& k, int ty, int zchunk,
+                                  float* uvel, cudaStream_t stream) {
+    if (ty == 4)
+        return N % 2 ? launch_fused16_t<S, 4, VEL, false>(src, dst, N, zchunk, k, uvel, stream)
+                     : launch_fused16_t<S, 4, VEL, true>(src, dst, N, zchunk, k, uvel, stream);
+    return N % 2 ? launch_fused16_t<S, 8, VEL, false>(src, dst, N, zchunk, k, uvel, stream)
+                 : launch_fused16_t<S, 8, VEL, true>(src, dst, N, zchunk, k, uvel, stream);
 }
 
 template <typename S, bool VEL>
@@ -61,6 +83,8 @@ static cudaError_t launch_fused_v(const void* src, void* dst, int N, const Dugks
         if (ty == 3 && whole_rows(N)) return launch_fused_t<S, 3, VEL, true>(src, dst, N, zchunk, k, uvel, stream);
         if (ty == 3) return launch_fused_t<S, 3, VEL>(src, dst, N, zchunk, k, uvel, stream);
         return launch_fused_t<S, 7, VEL>(src, dst, N, zchunk, k, uvel, stream);
+    } else if constexpr (sizeof(S) == 2) {
+        return launch_fused16<S, VEL>(src, dst, N, k, ty, zchunk, uvel, stream);
     } else {
         if (ty == 8 && whole_rows(N)) return launch_fused_t<S, 8, VEL, true>(src, dst, N, zchunk, k, uvel, stream);
         switch (ty) {
@@ -109,12 +133,17 @@ namespace {
 struct TileShape {
     int ty, per_sm;
     double alone, shared;
+    bool wraps;  // has the whole-row form
 };
-constexpr TileShape kShapes[] = {{4, 2, 1.5, 1.85}, {5, 2, 1.28, 2.0}, {8, 1, 1.76, 1.76}, {11, 1, 2.1, 2.1}};
-constexpr TileShape kShapes64[] = {{3, 1, 21.3, 21.3}, {7, 1, 41.5, 41.5}};
+constexpr TileShape kShapes[] = {{4, 2, 1.5, 1.85, false}, {5, 2, 1.28, 2.0, false}, {8, 1, 1.76, 1.76, true}, {11, 1, 2.1, 2.1, false}};
+constexpr TileShape kShapes64[] = {{3, 1, 21.3, 21.3, true}, {7, 1, 41.5, 41.5, false}};
 
-long long columns(int N, int ty) {
-    const bool wrap = whole_rows(N) && (ty == 3 || ty == 8);
+// FP16 and BF16: one block an SM
+constexpr TileShape kShapes16[] = {{8, 1, 1.9, 1.9, false}, {4, 1, 1.3, 1.3, false}};
+
+long long columns(int N, const TileShape& t) {
+    const int ty = t.ty;
+    const bool wrap = whole_rows(N) && t.wraps;
     return (long long)(wrap ? 1 : (N + 29) / 30) * ((N + ty - 1) / ty);
 }
 
@@ -122,7 +151,7 @@ long long columns(int N, int ty) {
 // planes; a block's prologue (two pre-steps and one record before the first
 // face) takes about 1.1 plane-times.
 double makespan(int N, const TileShape& t, int zc, int nsm) {
-    const long long cols = columns(N, t.ty);
+    const long long cols = columns(N, t);
     const double plane = cols * ((N + zc - 1) / zc) <= nsm ? t.alone : t.shared;
     return plane * tile_schedule(cols, N, zc, (long long)nsm * t.per_sm, 1.1);
 }
@@ -141,7 +170,7 @@ void dugks_fused_shape(int storage, int N, int nsm, int want_ty, int want_zc, in
     constexpr long long kMaxBlocks = 20000;
     double best = -1.0;
     auto consider = [&](const TileShape& t) {
-        const long long cols = columns(N, t.ty);
+        const long long cols = columns(N, t);
         for (int c = want_zc > 0 ? std::min(want_zc, N) : N; c >= 1; --c) {
             const int nz = (N + c - 1) / c;
             if (want_zc <= 0 && nz > 1 && (nz > 64 || cols * nz > kMaxBlocks)) break;
@@ -158,6 +187,18 @@ void dugks_fused_shape(int storage, int N, int nsm, int want_ty, int want_zc, in
     };
     if (storage == ST_F64) {
         for (const TileShape& t : kShapes64) consider(t);
+        return;
+    }
+    if (storage != ST_F32) {
+        const TileShape& t = kShapes16[want_ty == 4];
+        const long long cols = (long long)((N + 29) / 30) * ((N + t.ty - 1) / t.ty);
+        if (want_zc <= 0 && 2 * cols >= 3LL * nsm) {
+            // about two waves of blocks (256^3: 240 + 16 planes, the measured optimum)
+            *ty = t.ty;
+            *zc = (int)std::max(8LL, std::min<long long>((long long)N * cols / (2LL * nsm) / 8 * 8, N));
+            return;
+        }
+        consider(t);
         return;
     }
     for (const TileShape& t : kShapes)

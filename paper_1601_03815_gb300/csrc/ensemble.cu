@@ -30,6 +30,7 @@
 // buffer; the member barrier (DUGKS) or the stream order (LBE) makes every
 // read of step s - 1 precede every write of step s + 1 to the same buffer.
 #include "dugks_tile.cuh"
+#include "dugks_tile16.cuh"
 #include "kin.h"
 #include "kin_internal.h"
 #include "kin_sim.h"
@@ -75,6 +76,10 @@ __device__ __forceinline__ int ld_relaxed(const int* p) {
     return v;
 }
 
+// Rows of a 2-byte tile: it has a warp for each of its two halo rows, so the block
+// of a TY-row FP32 tile holds one row less.
+constexpr int rows16(int ty) { return ty - 1; }
+
 // One fused-DUGKS tile t of member M at buffer parity par.
 template <typename S, int TY>
 __device__ __forceinline__ void ensemble_tile(const EnsMember& M, int par, int t, unsigned char* smem_raw) {
@@ -83,8 +88,12 @@ __device__ __forceinline__ void ensemble_tile(const EnsMember& M, int par, int t
     // a local copy of the member's coefficients: passed as a reference into
     // the member table in global memory, the items ran 13 % slower
     const DugksCoef<float> kc = M.coef;
-    dugks_tile<S, TY>(static_cast<const S*>(M.buf[par]), static_cast<S*>(M.buf[par ^ 1]), M.N, r % M.tiles_x,
-                      r / M.tiles_x, bz, M.zchunk, kc, smem_raw);
+    const S* src = static_cast<const S*>(M.buf[par]);
+    S* dst = static_cast<S*>(M.buf[par ^ 1]);
+    if constexpr (sizeof(S) == 2)
+        two_byte::dugks_tile<S, rows16(TY)>(src, dst, M.N, r % M.tiles_x, r / M.tiles_x, bz, M.zchunk, kc, smem_raw);
+    else
+        dugks_tile<S, TY>(src, dst, M.N, r % M.tiles_x, r / M.tiles_x, bz, M.zchunk, kc, smem_raw);
 }
 
 // WIDE: some member has 2-byte storage (even N); without it the kernel holds
@@ -250,7 +259,7 @@ void drop_graphs(kin_ensemble* e) {
 template <int TY, bool WIDE>
 size_t persistent_smem() {
     return WIDE ? std::max(fused_smem_bytes<float, TY>(),
-                           std::max(fused_smem_bytes<__half, TY>(), fused_smem_bytes<__nv_bfloat16, TY>()))
+                           two_byte::tile_smem_bytes<__half, rows16(TY)>())
                 : fused_smem_bytes<float, TY>();
 }
 
@@ -290,7 +299,8 @@ std::vector<EnsMember> dugks_table(const kin_ensemble* e) {
         M.coef = dugks_coef<float>(s->nu, s->dt);
         const int zc = std::min(e->zc, s->N);
         M.tiles_x = (s->N + 29) / 30;
-        M.tiles_y = (s->N + e->tile_y - 1) / e->tile_y;
+        const int rows = s->storage == ST_F32 ? e->tile_y : rows16(e->tile_y);
+        M.tiles_y = (s->N + rows - 1) / rows;
         M.zchunk = zc;
         M.ntiles = M.tiles_x * M.tiles_y * ((s->N + zc - 1) / zc);
     }

@@ -183,7 +183,7 @@ int launch_steps(kin_sim* s, int n, float* uvel) {
     int k = 0;
     if (s->scheme == KIN_LBE_MRT && s->block_lbe == 0 && lbe_pairs(s->storage, s->N))
         for (; k + 2 <= n; k += 2) {
-            CK(lbe_pair_step(s->buf[s->cur], s->buf[s->cur ^ 1], s->N, s->nu, s->num_sms, s->stream));
+            CK(lbe_pair_step(s->storage, s->buf[s->cur], s->buf[s->cur ^ 1], s->N, s->nu, s->num_sms, s->stream));
             s->launches += 1;
             s->cur ^= 1;
             s->step += 2;

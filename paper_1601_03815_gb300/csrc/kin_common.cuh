@@ -160,12 +160,13 @@ __device__ __forceinline__ void moments(const C (&f)[Q], C& drho, C& jx, C& jy, 
 // (A = 3 a_x - S_ax, B = S_d - 3 s_yz, A' = a_y - a_z, B' = s_xy - s_xz;
 // omega_eps = omega_xx = 0, omega_epsj = -475/63, rho0 = 1; m_1 - m_eq_1 =
 // 19 (S_d - f0 - j.j)).  About 165 operations a cell, against 290 with every row
-// summed by itself: the 2-byte step and FP64 were bound by them (256^3 FP16
-// 214 -> 184 us, its copy roof; 64^3 FP64 135 -> 78 us).
+// summed by itself, which bounded FP64 (64^3 135 -> 78 us) and two steps in one
+// pass (lbe_pair.cuh).
 
-// s_k / |M_k|^2 (with the constant factors of the table) for the rates of Sec. IV.A.
+// Rates of Sec. IV.A, and s_k / |M_k|^2 with the constant factors of the table.
 template <typename C>
 struct MrtRates {
+    C s1, s2, s4, s9, s10, s13, s16;
     C c1, c2, c4, c9, c10, c11, c12, c13, c16;
 };
 
@@ -271,10 +272,187 @@ __device__ __forceinline__ void mrt_collide_t(C (&f)[Q], const MrtRates<C>& r, C
     }
 }
 
-template <typename C>
-__device__ __forceinline__ void mrt_collide(C (&f)[Q], const MrtRates<C>& r, C& drho_out, C& jx_out,
-                                            C& jy_out, C& jz_out) {
-    mrt_collide_t<false>(f, r, drho_out, jx_out, jy_out, jz_out, C(0), C(0), C(0));
+// ---------------------------------------------------------------------------
+// MRT collision of 2-byte storage, every row of M summed by itself.  The state of
+// such a run is its storage rounding noise: any other order of the FP32
+// operations reshuffles it, and E of a 32^3 BF16 run moves by 5e-3.  So these
+// runs keep this order, and with it their results bit for bit, at 214 us a
+// 256^3 FP16 step where the order of mrt_collide_t below takes 184.
+//
+// Moment rows of Sec. II.B as integer polynomials of the velocity.
+__host__ __device__ constexpr int mrow(int k, int x, int y, int z) {
+    const int r2 = x * x + y * y + z * z;
+    switch (k) {
+        case 0: return 1;
+        case 1: return 19 * r2 - 30;
+        case 2: return (21 * r2 * r2 - 53 * r2 + 24) / 2;
+        case 3: return x;
+        case 4: return (5 * r2 - 9) * x;
+        case 5: return y;
+        case 6: return (5 * r2 - 9) * y;
+        case 7: return z;
+        case 8: return (5 * r2 - 9) * z;
+        case 9: return 3 * x * x - r2;
+        case 10: return (3 * r2 - 5) * (3 * x * x - r2);
+        case 11: return y * y - z * z;
+        case 12: return (3 * r2 - 5) * (y * y - z * z);
+        case 13: return x * y;
+        case 14: return y * z;
+        case 15: return x * z;
+        case 16: return (y * y - z * z) * x;
+        case 17: return (z * z - x * x) * y;
+        default: return (x * x - y * y) * z;
+    }
+}
+// Squared norm of row k over the 19 velocities.
+__host__ __device__ constexpr int mnorm(int k) {
+    int s = 0;
+    for (int i = 0; i < Q; ++i) {
+        int v = mrow(k, cx(i), cy(i), cz(i));
+        s += v * v;
+    }
+    return s;
+}
+// Non-conserved rows whose polynomial is even / odd in xi.
+__host__ __device__ constexpr int even_row(int j) {
+    return j == 0 ? 1 : j == 1 ? 2 : j == 2 ? 9 : j == 3 ? 10 : j == 4 ? 11 : j == 5 ? 12 : j == 6 ? 13
+         : j == 7 ? 14 : 15;
+}
+__host__ __device__ constexpr int odd_row(int j) {
+    return j == 0 ? 4 : j == 1 ? 6 : j == 2 ? 8 : j == 3 ? 16 : j == 4 ? 17 : 18;
+}
+constexpr int NEVEN = 9;
+constexpr int NODD = 6;
+
+template <int K, typename C>
+__device__ __forceinline__ C rate(const MrtRates<C>& r) {
+    if constexpr (K == 1) return r.s1;
+    else if constexpr (K == 2) return r.s2;
+    else if constexpr (K == 4 || K == 6 || K == 8) return r.s4;
+    else if constexpr (K == 9 || K == 11) return r.s9;
+    else if constexpr (K == 10 || K == 12) return r.s10;
+    else if constexpr (K == 13 || K == 14 || K == 15) return r.s13;
+    else return r.s16;
+}
+
+// Equilibrium moments (Sec. II.B with omega_eps = omega_xx = 0,
+// omega_epsj = -475/63, rho0 = 1).  Slot 9 holds 3 p_xx.
+template <int K, typename C>
+__device__ __forceinline__ C meq(C drho, C jx, C jy, C jz, C jj) {
+    if constexpr (K == 1) return C(-11) * drho + C(19) * jj;
+    else if constexpr (K == 2) return C(-475.0 / 63.0) * jj;
+    else if constexpr (K == 4) return C(-2.0 / 3.0) * jx;
+    else if constexpr (K == 6) return C(-2.0 / 3.0) * jy;
+    else if constexpr (K == 8) return C(-2.0 / 3.0) * jz;
+    else if constexpr (K == 9) return C(2) * jx * jx - (jy * jy + jz * jz);
+    else if constexpr (K == 11) return jy * jy - jz * jz;
+    else if constexpr (K == 13) return jx * jy;
+    else if constexpr (K == 14) return jy * jz;
+    else if constexpr (K == 15) return jx * jz;
+    else return C(0);  // rows 10, 12 (omega_xx = 0) and 16-18
+}
+
+// One MRT collision in place (RHS of Eq. 21): f <- f - M^-1 S (M f - m_eq).
+// M is orthogonal, so M^-1 = M^T diag(1/|M_k|^2); rows are even or odd in xi,
+// so the work splits into the pair sums a_p = f_{2p+1} + f_{2p+2} (even rows)
+// and differences b_p = f_{2p+1} - f_{2p+2} (odd rows).
+// FIXJ: the equilibrium takes the prescribed momentum (jfx, jfy, jfz) and the
+// momentum rows relax fully to it (the consistent initialisation, Sec. IV.A);
+// otherwise the cell's own momentum, conserved.
+template <bool FIXJ, typename C>
+__device__ __forceinline__ void mrt_collide_rows(C (&f)[Q], const MrtRates<C>& r, C& drho_out, C& jx_out,
+                                              C& jy_out, C& jz_out, C jfx, C jfy, C jfz) {
+    C a[NPAIR], b[NPAIR];
+#pragma unroll
+    for (int p = 0; p < NPAIR; ++p) {
+        a[p] = f[2 * p + 1] + f[2 * p + 2];
+        b[p] = f[2 * p + 1] - f[2 * p + 2];
+    }
+    const C f0 = f[0];
+    const C drho = f0 + ((a[0] + a[1]) + a[2]) + (((a[3] + a[4]) + (a[5] + a[6])) + (a[7] + a[8]));
+    const C jx = (b[0] + b[3]) + (b[4] + (b[5] + b[6]));
+    const C jy = (b[1] + b[3]) - (b[4] - (b[7] + b[8]));
+    const C jz = (b[2] + b[5]) - (b[6] - (b[7] - b[8]));
+    drho_out = drho;
+    jx_out = jx;
+    jy_out = jy;
+    jz_out = jz;
+    const C jxe = FIXJ ? jfx : jx, jye = FIXJ ? jfy : jy, jze = FIXJ ? jfz : jz;
+    const C jj = jxe * jxe + jye * jye + jze * jze;
+    // FIXJ: (m - m_eq) / |M_k|^2 of the momentum rows at rate 1 (|M_3|^2 = 10)
+    [[maybe_unused]] const C gjx = (jx - jfx) * C(0.1), gjy = (jy - jfy) * C(0.1), gjz = (jz - jfz) * C(0.1);
+
+    C ge[NEVEN], go[NODD];
+    static_for<0, NEVEN>([&](auto jc) {
+        constexpr int J = decltype(jc)::value;
+        constexpr int K = even_row(J);
+        C m = C(mrow(K, 0, 0, 0)) * f0;
+        static_for<0, NPAIR>([&](auto pc) {
+            constexpr int P = decltype(pc)::value;
+            constexpr int c = mrow(K, pair_x(P), pair_y(P), pair_z(P));
+            if constexpr (c == 1) m += a[P];
+            else if constexpr (c == -1) m -= a[P];
+            else if constexpr (c != 0) m += C(c) * a[P];
+        });
+        ge[J] = rate<K>(r) * (m - meq<K>(drho, jxe, jye, jze, jj)) * (C(1) / C(mnorm(K)));
+    });
+    static_for<0, NODD>([&](auto jc) {
+        constexpr int J = decltype(jc)::value;
+        constexpr int K = odd_row(J);
+        C m = C(0);
+        static_for<0, NPAIR>([&](auto pc) {
+            constexpr int P = decltype(pc)::value;
+            constexpr int c = mrow(K, pair_x(P), pair_y(P), pair_z(P));
+            if constexpr (c == 1) m += b[P];
+            else if constexpr (c == -1) m -= b[P];
+            else if constexpr (c != 0) m += C(c) * b[P];
+        });
+        go[J] = rate<K>(r) * (m - meq<K>(drho, jxe, jye, jze, jj)) * (C(1) / C(mnorm(K)));
+    });
+    // back transform: df_i = sum_k M_k,i g_k
+    {
+        C d0 = C(0);
+        static_for<0, NEVEN>([&](auto jc) {
+            constexpr int J = decltype(jc)::value;
+            constexpr int c = mrow(even_row(J), 0, 0, 0);
+            if constexpr (c != 0) d0 += C(c) * ge[J];
+        });
+        f[0] = f0 - d0;
+    }
+    static_for<0, NPAIR>([&](auto pc) {
+        constexpr int P = decltype(pc)::value;
+        C e = C(0), o = C(0);
+        static_for<0, NEVEN>([&](auto jc) {
+            constexpr int J = decltype(jc)::value;
+            constexpr int c = mrow(even_row(J), pair_x(P), pair_y(P), pair_z(P));
+            if constexpr (c == 1) e += ge[J];
+            else if constexpr (c == -1) e -= ge[J];
+            else if constexpr (c != 0) e += C(c) * ge[J];
+        });
+        static_for<0, NODD>([&](auto jc) {
+            constexpr int J = decltype(jc)::value;
+            constexpr int c = mrow(odd_row(J), pair_x(P), pair_y(P), pair_z(P));
+            if constexpr (c == 1) o += go[J];
+            else if constexpr (c == -1) o -= go[J];
+            else if constexpr (c != 0) o += C(c) * go[J];
+        });
+        if constexpr (FIXJ) {
+            // the momentum rows (M_3,5,7 = xi_x, xi_y, xi_z) relaxed with rate 1
+            if constexpr (pair_x(P) != 0) o += C(pair_x(P)) * gjx;
+            if constexpr (pair_y(P) != 0) o += C(pair_y(P)) * gjy;
+            if constexpr (pair_z(P) != 0) o += C(pair_z(P)) * gjz;
+        }
+        f[2 * P + 1] -= e + o;
+        f[2 * P + 2] -= e - o;
+    });
+}
+
+// The collision of storage type S.
+template <typename S, bool FIXJ, typename C>
+__device__ __forceinline__ void mrt_collide_as(C (&f)[Q], const MrtRates<C>& r, C jfx = C(0), C jfy = C(0), C jfz = C(0)) {
+    C drho, jx, jy, jz;
+    if constexpr (sizeof(S) == 2) mrt_collide_rows<FIXJ>(f, r, drho, jx, jy, jz, jfx, jfy, jfz);
+    else mrt_collide_t<FIXJ>(f, r, drho, jx, jy, jz, jfx, jfy, jfz);
 }
 
 // Periodic neighbour of coordinate v in [0, n).

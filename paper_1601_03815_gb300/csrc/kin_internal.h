@@ -20,10 +20,11 @@ size_t storage_bytes(int storage);
 cudaError_t lbe_step(int storage, const void* src, void* dst, int N, double nu, int block_x,
                      cudaStream_t stream);
 
-// Two steps from src to dst (FP32 storage, nsm multiprocessors), bitwise those of
-// two lbe_step calls; lbe_pairs: whether that is the faster way.
+// Two steps from src to dst in one launch (nsm multiprocessors), bitwise those of
+// two lbe_step calls; lbe_pairs: whether that is the faster way (elsewhere
+// cudaErrorInvalidValue).
 bool lbe_pairs(int storage, int N);
-cudaError_t lbe_pair_step(const void* src, void* dst, int N, double nu, int nsm, cudaStream_t stream);
+cudaError_t lbe_pair_step(int storage, const void* src, void* dst, int N, double nu, int nsm, cudaStream_t stream);
 
 // DUGKS step (Eqs. 9-20).  fbp is scratch of 19 N^3 compute-type values.
 cudaError_t dugks_step(int storage, const void* src, void* dst, void* fbp, int N, double nu,

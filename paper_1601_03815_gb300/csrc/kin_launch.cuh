@@ -15,6 +15,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <utility>
 
 namespace kin {
@@ -22,6 +23,21 @@ namespace kin {
 __device__ __forceinline__ void grid_begin() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Allow KERNEL bytes of dynamic shared memory on the current device; set once per
+// device that this process launches on.
+template <auto KERNEL>
+cudaError_t allow_smem(size_t bytes) {
+    static std::atomic<unsigned long long> configured{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (bit && (configured.load() & bit)) return cudaSuccess;
+    e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) configured.fetch_or(bit);
+    return e;
 }
 
 template <typename... P, typename... A>

@@ -7,7 +7,6 @@
 #include "tile_schedule.h"
 
 #include <algorithm>
-#include <atomic>
 #include <cstring>
 
 namespace kin {
@@ -102,8 +101,7 @@ __global__ void __launch_bounds__(256) lbe_consistent_kernel(const S* __restrict
     C f[Q];
     lbe_gather<S>(src, N, plane, x, y, z, f);
     const size_t c = (size_t)x + (size_t)N * (y + (size_t)N * z);
-    C drho, jx, jy, jz;
-    mrt_collide_t<true>(f, rates, drho, jx, jy, jz, (C)u0[c], (C)u0[plane + c], (C)u0[2 * plane + c]);
+    mrt_collide_as<S, true>(f, rates, (C)u0[c], (C)u0[plane + c], (C)u0[2 * plane + c]);
     lbe_scatter<S>(dst, N, plane, x, y, z, f);
 }
 
@@ -129,24 +127,38 @@ cudaError_t lbe_consistent_step(int storage, const void* src, void* dst, int N, 
     return cudaErrorInvalidValue;
 }
 
-// Two steps in one pass pay where the state does not stay in L2 between steps:
-// us a step, single / paired: 64^3 5.2 / 7.6 (40 MB of state), 97^3 24.6 / 21.0,
-// 128^3 47.9 / 37.9, 256^3 367 / 257; level between 84^3 and 88^3 (14.1 / 12.2).
-bool lbe_pairs(int storage, int N) { return storage == ST_F32 && N >= 88; }
+// Two steps in one launch pay where a step is mostly the hand-over between two
+// grids (us a step, single / paired, FP32: 8^3 1.6 / 1.3, 24^3 2.0 / 1.35, 32^3
+// 3.5 / 1.4), and where the state does not stay in L2 between steps (64^3 5.2 /
+// 7.6, 40 MB of state; 84^3 11.8 / 12.1, 88^3 14.1 / 12.2, 97^3 24.6 / 21.0, 128^3
+// 47.9 / 37.9, 256^3 367 / 257).  2-byte steps of large boxes are bound by their
+// operations, FP64 always is.
+bool lbe_pairs(int storage, int N) { return N <= 32 ? storage != ST_F64 : storage == ST_F32 && N >= 88; }
 
-cudaError_t lbe_pair_step(const void* src, void* dst, int N, double nu, int nsm, cudaStream_t stream) {
+template <typename S>
+static cudaError_t launch_small_pair(const void* src, void* dst, int N, double nu, cudaStream_t stream) {
+    // 96 blocks of 768 threads at 32^3; 6 rows x 1 plane 2.4 us a step, 6 x 2 1.6,
+    // 3 x 2 2.1, 8 x 1 1.5, 2 x 2 1.75
+    constexpr int TY = 4, TZ = 2;
+    constexpr size_t smem = sizeof(float) * Q * 32 * (TY + 2) * (TZ + 2);
+    cudaError_t e = allow_smem<lbe_small_pair_kernel<S, TY, TZ>>(smem);
+    if (e != cudaSuccess) return e;
+    return launch_next(lbe_small_pair_kernel<S, TY, TZ>, dim3((N + TY - 1) / TY, (N + TZ - 1) / TZ),
+                       dim3(32, TY + 2, TZ + 2), smem, stream, (const S*)src, (S*)dst, N, (size_t)N * N * N,
+                       lbe_rates<float>(nu));
+}
+
+cudaError_t lbe_pair_step(int storage, const void* src, void* dst, int N, double nu, int nsm, cudaStream_t stream) {
+    if (!lbe_pairs(storage, N)) return cudaErrorInvalidValue;
+    if (N <= 32) {
+        if (storage == ST_F32) return launch_small_pair<float>(src, dst, N, nu, stream);
+        if (storage == ST_F16) return launch_small_pair<__half>(src, dst, N, nu, stream);
+        return launch_small_pair<__nv_bfloat16>(src, dst, N, nu, stream);
+    }
     constexpr int TY = kPairRows;
     constexpr size_t smem = sizeof(float) * LbePairSmem<TY>::FLOATS;
-    static std::atomic<unsigned long long> configured{0};  // devices whose shared-memory limit is set
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    cudaError_t e = allow_smem<lbe_pair_kernel<TY>>(smem);
     if (e != cudaSuccess) return e;
-    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
-    if (!bit || !(configured.load() & bit)) {
-        e = cudaFuncSetAttribute(lbe_pair_kernel<TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        configured.fetch_or(bit);
-    }
     // planes a block: the shortest schedule, of at most 64 chunks (a block relaxes
     // two planes before its first result)
     const long long cols = (long long)((N + 29) / 30) * ((N + TY - 1) / TY);

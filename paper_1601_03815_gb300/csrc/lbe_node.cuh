@@ -20,6 +20,13 @@ template <typename C>
 inline MrtRates<C> lbe_rates(double nu) {
     const double s9 = 1.0 / (3.0 * nu + 0.5);
     MrtRates<C> r;
+    r.s1 = C(1.19);
+    r.s2 = C(1.4);
+    r.s4 = C(1.2);
+    r.s9 = C(s9);
+    r.s10 = C(1.4);
+    r.s13 = r.s9;
+    r.s16 = C(1.98);
     r.c1 = C(1.19 * 19.0 / 2394.0);
     r.c2 = C(1.4 / 252.0);
     r.c4 = C(1.2 * 5.0 / 40.0);
@@ -66,8 +73,7 @@ __device__ __forceinline__ void lbe_node(const S* __restrict__ src, S* __restric
     using C = typename Traits<S>::C;
     C f[Q];
     lbe_gather<S>(src, N, plane, x, y, z, f);
-    C drho, jx, jy, jz;
-    mrt_collide(f, rates, drho, jx, jy, jz);
+    mrt_collide_as<S, false>(f, rates);
     lbe_scatter<S>(dst, N, plane, x, y, z, f);
 }
 
@@ -205,8 +211,7 @@ __device__ __forceinline__ void lbe_vnode4p(const S* __restrict__ src, S* __rest
         float f[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) f[i] = Half1<S>::get(w[i][k >> 1], k & 1);
-        float drho, jx, jy, jz;
-        mrt_collide(f, rates, drho, jx, jy, jz);
+        mrt_collide_as<S, false>(f, rates);
 #pragma unroll
         for (int i = 0; i < Q; ++i) w[i][k >> 1] = Half1<S>::put(w[i][k >> 1], k & 1, f[i]);
     }
@@ -248,8 +253,7 @@ __device__ __forceinline__ void lbe_vnode(const S* __restrict__ src, S* __restri
     });
 #pragma unroll
     for (int k = 0; k < V; ++k) {
-        float drho, jx, jy, jz;
-        mrt_collide(f[k], rates, drho, jx, jy, jz);
+        mrt_collide_as<S, false>(f[k], rates);
     }
     const int c = x + N * (y + N * z);
     if (!KIN_CHECK((size_t)c + V <= plane, DBG_LBE_STORE, c)) return;

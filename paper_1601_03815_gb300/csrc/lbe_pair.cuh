@@ -88,8 +88,7 @@ __global__ void __launch_bounds__(32 * (TY + 2), kPairBlocks)
     int up_last = 0;
     load();
     for (int k = z0 - 1; k <= zend; ++k) {
-        float d0, d1, d2, d3;
-        mrt_collide(f, rates, d0, d1, d2, d3);
+        mrt_collide_as<float, false>(f, rates);
         static_for<0, Q>([&](auto ic) {
             constexpr int I = decltype(ic)::value;
             if constexpr (lbe_moves(I)) {
@@ -116,7 +115,7 @@ __global__ void __launch_bounds__(32 * (TY + 2), kPairBlocks)
                     if constexpr (cz(I) < 0) g[I] = own[SM::DOWN + O + down];
                 }
             });
-            mrt_collide(g, rates, d0, d1, d2, d3);
+            mrt_collide_as<float, false>(g, rates);
             if (valid) {
                 const int c = x + y * N + (k - 1) * nn;
                 if (KIN_CHECK(c >= 0 && (size_t)c < plane, DBG_LBE_STORE, c)) {
@@ -135,6 +134,42 @@ __global__ void __launch_bounds__(32 * (TY + 2), kPairBlocks)
         flat = flat == 2 * 8 * SM::POP ? 0 : flat + 8 * SM::POP;
         down = 4 * SM::POP - down;
     }
+}
+
+// Two steps of a box of at most 32 (FP32, FP16 or BF16 storage): such a step is
+// latency, not bytes (32^3: 3.5 us, of which ~1.7 are the hand-over from one grid
+// to the next; in pairs 1.4 us a step).  A warp holds a whole periodic row, a block TY rows and TZ planes
+// with a rim of one, one node a thread: every thread relaxes its node, the inner
+// ones again from shared memory.  Most of the first step is done by several
+// blocks, which costs less than a second launch.
+template <typename S, int TY, int TZ>
+__global__ void __launch_bounds__(32 * (TY + 2) * (TZ + 2), 1)
+    lbe_small_pair_kernel(const S* src, S* dst, int N, size_t plane, MrtRates<float> rates) {
+    constexpr int ROWS = TY + 2, PLANES = TZ + 2;
+    extern __shared__ __align__(16) float smem_f[];  // [population][plane][row][lane]
+    const int lane = threadIdx.x, row = threadIdx.y, pl = threadIdx.z;
+    const int yr = blockIdx.x * TY - 1 + row, zr = blockIdx.y * TZ - 1 + pl;
+    const int x = min(lane, N - 1), y = (yr + N) % N, z = (zr + N) % N;
+    grid_begin();
+    float f[Q];
+    lbe_gather<S>(src, N, plane, x, y, z, f);
+    mrt_collide_as<S, false>(f, rates);
+    // what storing the state and reading it back gives
+#pragma unroll
+    for (int i = 0; i < Q; ++i) f[i] = (float)S(f[i]);
+    constexpr int POP = PLANES * ROWS * 32;
+    const int at = (pl * ROWS + row) * 32;
+#pragma unroll
+    for (int i = 1; i < Q; ++i) smem_f[i * POP + at + lane] = f[i];
+    __syncthreads();
+    if (row < 1 || row > TY || pl < 1 || pl > TZ || lane >= N || yr >= N || zr >= N) return;
+    const int xs[3] = {wrap_dec(lane, N), lane, wrap_inc(lane, N)};
+    static_for<1, Q>([&](auto ic) {
+        constexpr int I = decltype(ic)::value;
+        f[I] = smem_f[I * POP + at - (cz(I) * ROWS + cy(I)) * 32 + xs[1 - cx(I)]];
+    });
+    mrt_collide_as<S, false>(f, rates);
+    lbe_scatter<S>(dst, N, plane, lane, yr, zr, f);
 }
 
 }  // namespace kin

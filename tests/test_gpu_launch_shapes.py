@@ -68,6 +68,14 @@ def test_lbe_step_pairs_are_bitwise_single_steps(kin, N, steps):
     np.testing.assert_array_equal(_run(kin, N, kin.LBE_MRT, kin.F32, steps), ref)
 
 
+@pytest.mark.parametrize("storage", [0, 1, 2])
+@pytest.mark.parametrize("N", [2, 3, 4, 5, 17, 31, 32])
+def test_lbe_small_step_pairs_are_bitwise_single_steps(kin, N, storage):
+    """Up to 32^3 steps go in pairs of one launch (4 rows x 2 planes a block)."""
+    ref = _run(kin, N, kin.LBE_MRT, storage, 5, block_x=32)
+    np.testing.assert_array_equal(_run(kin, N, kin.LBE_MRT, storage, 5), ref)
+
+
 @pytest.mark.parametrize("scheme", [0, 1])
 def test_steps_captured_in_a_graph(kin, scheme):
     """Steps launched to overlap the one before them, replayed from a graph."""
