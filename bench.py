@@ -84,8 +84,8 @@ def _sm_max_mhz():
 # The fused DUGKS kernel's translation unit, its headers and the build flags:
 # DRAM traffic and instruction counts recorded from an ncu capture hold only
 # while these are unchanged.
-KERNEL_SOURCES = ("dugks_fused.cu", "dugks_tile.cuh", "dugks_face.cuh", "pair_math.cuh", "kin_common.cuh",
-                  "kin_internal.h")
+KERNEL_SOURCES = ("dugks_fused.cu", "dugks_tile.cuh", "dugks_face.cuh", "tile_schedule.h", "pair_math.cuh",
+                  "kin_common.cuh", "kin_launch.cuh", "kin_internal.h")
 COUNTERS_RECORD = "profiles/dugks_fused_kernel_256_f32_counters.md"
 SMS, SCHEDULERS = 152, 4  # GB300: streaming multiprocessors, warp schedulers per SM
 

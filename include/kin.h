@@ -236,7 +236,9 @@ int kin_num_shells(int N);
 /* Launch-shape tuning (all values <= 0 keep the current setting):
  *   block_x  threads per block along x (multiple of 32, <= 1024) of the
  *            LBE step (used up to 256) and of the two-launch DUGKS form
- *            (up to 128); with FP16/BF16 storage and even N an LBE thread
+ *            (up to 128); LBE steps then run one to a launch (by default
+ *            kin_step takes them in pairs where that is faster, with bitwise
+ *            the same results); with FP16/BF16 storage and even N an LBE thread
  *            takes 4 cells, or 2 when N % 4 != 0
  *   tile_y   DUGKS fused kernel: rows per tile, 4 or 8 (by default 5, 8 or 11,
  *            chosen with zchunk)

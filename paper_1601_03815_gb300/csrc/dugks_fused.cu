@@ -162,7 +162,8 @@ double makespan(int N, const TileShape& t, int zc, int nsm) {
 // last wave nearly empty costs up to a third of it.  Every tile height and
 // chunk length is scored by the schedule above and the shortest taken (the
 // longest chunk among those within 0.5 %: fewer halo planes).  Measured against
-// sweeps of all shapes: 33^3 8 x 2 planes 7.6 us, 48^3 8 x 4 12.3
+// sweeps of all shapes (before steps overlapped the end of the step before,
+// which took ~2 us off the small ones): 33^3 8 x 2 planes 7.6 us, 48^3 8 x 4 12.3
 // us (5 x 8: 14.4), 64^3 11 x 8 22.5 us (8 x 11: 23.8), 97^3 11 x 25 61.6 us
 // (5 x 13: 66.6), 128^3 11 x 26 117 us (5 x 19: 119), 256^3 11 x 37 0.777 ms
 // (5 x 52: 0.773).

@@ -36,10 +36,10 @@
 // Dhat_p = (D_{2p+1}, -D_{2p+2}), so a face adds the same signed value to
 // both members.
 //
-// What bounds it, 128^3 FP32: the shared-memory and shuffle pipe, 67 % of its
-// wavefront rate (FMA pipe 40 %, issue 45 %); every row's exchange is ~200
-// wavefronts a plane.  Against the form that staged f-tilde in shared memory
-// and summed the moments of every difference: 96.3 -> 59 M warp instructions,
+// What bounds it, 128^3 FP32 (11-row tiles): the shared-memory and shuffle pipe,
+// 58 % of its wavefront rate, and latency between the two barriers (FMA pipe
+// 42 %, issue 47 %).  Against the form that staged f-tilde in shared memory
+// and summed the moments of every difference: 96.3 -> 62.1 M warp instructions,
 // 154 -> 117 us at 128^3, 0.961 -> 0.773 ms at 256^3 (2.65 -> 3.30 TB/s
 // algorithmic).  The steps of that: moments from f-tilde and f-tilde kept in
 // registers 0.961 -> 0.928; two 6-warp blocks on an SM, which drift apart so that
@@ -186,51 +186,6 @@ constexpr size_t fused_smem_bytes() {
     return FusedSmem<typename Traits<S>::C, TY>::BYTES;
 }
 
-// ------------------------------------------------------------------ global loads
-// f-tilde is read once, in L2 (the persistent ensemble kernel reads what other
-// blocks wrote earlier in the same launch, so never through the read-only
-// path), and kept raw until the pre-step.
-template <typename S>
-struct RawOf {
-    using T = S;
-    static __device__ __forceinline__ T load(const S* p) { return __ldcg(p); }
-    static __device__ __forceinline__ typename Traits<S>::C get(T v) { return v; }
-    template <typename P>
-    static __device__ __forceinline__ P store2(S* p0, S* p1, P v) {
-        __stcg(p0, v.x);
-        __stcg(p1, v.y);
-        return v;
-    }
-};
-template <>
-struct RawOf<__half> {
-    using T = unsigned short;
-    static __device__ __forceinline__ T load(const __half* p) {
-        return __ldcg(reinterpret_cast<const unsigned short*>(p));
-    }
-    static __device__ __forceinline__ float get(T v) { return __half2float(__ushort_as_half(v)); }
-    static __device__ __forceinline__ float2 store2(__half* p0, __half* p1, float2 v) {
-        const __half2 h = __floats2half2_rn(v.x, v.y);
-        __stcg(reinterpret_cast<unsigned short*>(p0), __half_as_ushort(__low2half(h)));
-        __stcg(reinterpret_cast<unsigned short*>(p1), __half_as_ushort(__high2half(h)));
-        return make_float2(__low2float(h), __high2float(h));
-    }
-};
-template <>
-struct RawOf<__nv_bfloat16> {
-    using T = unsigned short;
-    static __device__ __forceinline__ T load(const __nv_bfloat16* p) {
-        return __ldcg(reinterpret_cast<const unsigned short*>(p));
-    }
-    static __device__ __forceinline__ float get(T v) { return __bfloat162float(__ushort_as_bfloat16(v)); }
-    static __device__ __forceinline__ float2 store2(__nv_bfloat16* p0, __nv_bfloat16* p1, float2 v) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
-        __stcg(reinterpret_cast<unsigned short*>(p0), __bfloat16_as_ushort(__low2bfloat16(h)));
-        __stcg(reinterpret_cast<unsigned short*>(p1), __bfloat16_as_ushort(__high2bfloat16(h)));
-        return make_float2(__low2float(h), __high2float(h));
-    }
-};
-
 // ------------------------------------------------------------------ cells
 // f-bar-plus of one cell with its moments.
 template <typename C>
@@ -359,6 +314,7 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
     using P2 = Pr<C>;
     using Q4 = Quad<C>;
     using SM = FusedSmem<C, TY>;
+    static_assert(std::is_same<S, C>::value, "FP32 or FP64 storage (FP16 and BF16: dugks_tile16.cuh)");
     static_assert(!VEL || std::is_same<C, float>::value, "the fused velocity serves FP32-computed storage");
 
     // read once: recomputed from the special registers and the layout, the
@@ -383,27 +339,27 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
 
     auto zwrap = [&](int z) { return z < 0 ? z + N : (z >= N ? z - N : z); };
 
-    // raw f-tilde of this thread's column at plane z
-    using Raw = typename RawOf<S>::T;
-    auto load_plane = [&](int z, unsigned col, Raw (&fr)[Q]) {
+    // f-tilde of a column at plane z, from L2 (kin_launch.cuh; in the persistent
+    // ensemble kernel other blocks wrote it earlier in the same launch)
+    auto load_plane = [&](int z, unsigned col, C (&fr)[Q]) {
         const unsigned o = (unsigned)zwrap(z) * nn32 + col;
         if (!KIN_CHECK(o < plane, DBG_DUGKS_LOAD, o)) return;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) fr[i] = RawOf<S>::load(src + i * plane + o);
+        for (int i = 0; i < Q; ++i) fr[i] = Traits<S>::load_l2(src + i * plane + o);
     };
 
-    // Eq. 19 of the column's raw values: fbp = f + b (f_eq - f), f_eq of a pair
+    // Eq. 19 of the column's values: fbp = f + b (f_eq - f), f_eq of a pair
     // = q +/- l (Eq. 7), with the moments of fbp: delta-rho and j are those of
     // f, Pi = Pi_f + b (Pi_eq - Pi_f) with Pi_eq = delta-rho / 3 I + j j.  The
     // exchange record goes to slot SL.  With KEEP also f-tilde-plus = 4/3 fbp -
     // 1/3 f-tilde (Eq. 20), kept in the column's own slot until the update.
-    auto prestep = [&](auto slc, auto keepc, unsigned own, const Raw (&fr)[Q], Cell<C>& n) {
+    auto prestep = [&](auto slc, auto keepc, unsigned own, const C (&fr)[Q], Cell<C>& n) {
         constexpr int SL = decltype(slc)::value;
         constexpr bool keep = decltype(keepc)::value;
         P2 f[NPAIR];
 #pragma unroll
-        for (int q = 0; q < NPAIR; ++q) f[q] = pmk(RawOf<S>::get(fr[2 * q + 1]), RawOf<S>::get(fr[2 * q + 2]));
-        const C f0 = RawOf<S>::get(fr[0]);
+        for (int q = 0; q < NPAIR; ++q) f[q] = pmk(fr[2 * q + 1], fr[2 * q + 2]);
+        const C f0 = fr[0];
         C a[NPAIR], b[NPAIR];
 #pragma unroll
         for (int q = 0; q < NPAIR; ++q) {
@@ -507,7 +463,7 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
         const unsigned ownr[2] = {own, own + (TY + 1) * SM::ROW};
         const unsigned col[2] = {col32, (unsigned)gx + (unsigned)N * wrapc(by * TY + TY, N)};
         Cell<C> A[2], B[2];
-        Raw fr[2][Q];
+        C fr[2][Q];
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             load_plane(z0 - 1, col[r], fr[r]);
@@ -552,7 +508,7 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
     }
 
     Cell<C> A, B;          // planes z and z - 1, in turn
-    Raw fr[Q];
+    C fr[Q];
     Rec<C> Pz;             // P^z record of plane z - 1
     P2 ffy[NC] = {};       // upper y-face values of plane z - 1
     P2 D[NPAIR];           // sign-folded flux sums of plane z - 1, still missing z and y faces
@@ -640,10 +596,10 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
                 Traits<S>::store(dst + c, t[NPAIR].x);
                 static_for<0, NPAIR>([&](auto pc) {
                     constexpr int PP = decltype(pc)::value;
-                    // f-tilde-plus minus dt times the flux sum (Eq. 9), both members rounded
-                    // by one paired conversion for 2-byte storage
-                    [[maybe_unused]] const P2 r = RawOf<S>::store2(
-                        dst + (2 * PP + 1) * plane + c, dst + (2 * PP + 2) * plane + c, pfma(kc.dts, D[PP], t[PP]));
+                    // f-tilde-plus minus dt times the flux sum (Eq. 9)
+                    const P2 r = pfma(kc.dts, D[PP], t[PP]);
+                    __stcg(dst + (2 * PP + 1) * plane + c, r.x);
+                    __stcg(dst + (2 * PP + 2) * plane + c, r.y);
                     if constexpr (VEL) {
                         vel_add(std::integral_constant<int, 2 * PP + 1>{}, r.x);
                         vel_add(std::integral_constant<int, 2 * PP + 2>{}, r.y);

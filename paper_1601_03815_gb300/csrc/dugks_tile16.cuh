@@ -58,6 +58,21 @@ __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gsrc) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
+// The two members of a pair, rounded by one paired conversion (the rounding of two
+// single ones), to p0 and p1; returns what loads would return.
+__device__ __forceinline__ float2 store2(__half* p0, __half* p1, float2 v) {
+    const __half2 h = __floats2half2_rn(v.x, v.y);
+    *p0 = __low2half(h);
+    *p1 = __high2half(h);
+    return make_float2(__low2float(h), __high2float(h));
+}
+__device__ __forceinline__ float2 store2(__nv_bfloat16* p0, __nv_bfloat16* p1, float2 v) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
+    *p0 = __low2bfloat16(h);
+    *p1 = __high2bfloat16(h);
+    return make_float2(__low2float(h), __high2float(h));
+}
+
 template <typename S, int TY>
 constexpr size_t tile_smem_bytes() {
     return sizeof(FusedSmem<float, TY>) + sizeof(RawStage16<S, TY>);
@@ -519,7 +534,7 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
                     const P2 o = pfma(kc.dts, Dprev[PP], t);
                     // both members rounded by one paired conversion for 2-byte storage
                     [[maybe_unused]] const P2 r =
-                        RawOf<S>::store2(dst + (2 * PP + 1) * plane + c, dst + (2 * PP + 2) * plane + c, o);
+                        store2(dst + (2 * PP + 1) * plane + c, dst + (2 * PP + 2) * plane + c, o);
                     if constexpr (VEL) {
                         vel_add(std::integral_constant<int, 2 * PP + 1>{}, r.x);
                         vel_add(std::integral_constant<int, 2 * PP + 2>{}, r.y);

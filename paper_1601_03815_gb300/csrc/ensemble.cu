@@ -349,8 +349,8 @@ int launch_persistent_config(kin_ensemble* e) {
 // Planes per item when the caller has not chosen: a step takes about its items'
 // planes (and 1.1 plane-times of prologue each) spread over the resident
 // blocks, but no less than its longest item, which the next step of that
-// member waits for.  The reference mix gets 64 planes (0.373 ms a step of its
-// DUGKS members; 16: 0.421, 32: 0.385, 128: 0.366).
+// member waits for.  The reference mix gets whole columns, at most 128 planes
+// (0.366 ms a step of its DUGKS members; 16 planes: 0.421, 32: 0.385, 64: 0.373).
 int default_zchunk(const kin_ensemble* e) {
     int nsm = 0;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, e->device) != cudaSuccess || nsm <= 0) nsm = 152;

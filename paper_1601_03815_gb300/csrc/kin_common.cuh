@@ -277,7 +277,7 @@ __device__ __forceinline__ void mrt_collide_t(C (&f)[Q], const MrtRates<C>& r, C
 // such a run is its storage rounding noise: any other order of the FP32
 // operations reshuffles it, and E of a 32^3 BF16 run moves by 5e-3.  So these
 // runs keep this order, and with it their results bit for bit, at 214 us a
-// 256^3 FP16 step where the order of mrt_collide_t below takes 184.
+// 256^3 FP16 step where the order of mrt_collide_t takes 184.
 //
 // Moment rows of Sec. II.B as integer polynomials of the velocity.
 __host__ __device__ constexpr int mrow(int k, int x, int y, int z) {

@@ -83,8 +83,9 @@ __global__ void velocity_kernel(const S* __restrict__ st, bool shifted, int N, s
 // u in FP32 for storage computed in FP32, the populations of a cell added in
 // their order (the fused DUGKS step forms the same sums).  SHIFTED: the LBE
 // pull layout; its row offsets are formed once per cell, which with the index
-// arithmetic of stored_index took as long as the loads (256^3 LBE: FP32
-// 250 -> 218 us, FP16 254 -> 130 us with four cells a thread).
+// arithmetic of stored_index took as long as the loads (256^3 LBE, velocity and
+// reduction together, a step with E and eps less the step: FP32 317 -> 260 us,
+// FP16 330 -> 176 us with four cells a thread).
 template <int I>
 __device__ __forceinline__ void add_velocity(float (&j)[3], float v) {
     if constexpr (cx(I) > 0) j[0] += v;
