@@ -225,17 +225,27 @@ int enqueue_energy_dissipation(kin_sim* s, double* host, bool with_err) {
     return KIN_OK;
 }
 
-// The address under which kernels may write doubles to this host memory, or
-// NULL: aligned page-locked memory of this process.  Looked up on every call
-// (the memory may have been released and the address reused since).
+// The address under which kernels may write the two doubles of a result to this
+// host memory, or NULL: aligned page-locked memory of this process, both of them
+// in it and not registered as read-only for the device (the copy then gives the
+// error it always gave).  Looked up on every call (the memory may have been
+// released and the address reused since).
 double* device_view(double* host) {
     if (reinterpret_cast<uintptr_t>(host) % sizeof(double)) return nullptr;
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
+    cudaPointerAttributes a, b;
+    unsigned flags = 0;
+    if (cudaPointerGetAttributes(&a, host) != cudaSuccess || cudaPointerGetAttributes(&b, host + 1) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
-    return a.type == cudaMemoryTypeHost ? static_cast<double*>(a.devicePointer) : nullptr;
+    double* view = static_cast<double*>(a.devicePointer);
+    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !view || b.devicePointer != view + 1)
+        return nullptr;
+    if (cudaHostGetFlags(&flags, host) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return flags & cudaHostRegisterReadOnly ? nullptr : view;
 }
 
 }  // namespace
