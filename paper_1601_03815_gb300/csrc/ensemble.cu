@@ -39,6 +39,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <cmath>
 #include <climits>
 #include <cstddef>
 #include <map>
@@ -348,22 +349,27 @@ int launch_persistent_config(kin_ensemble* e) {
 
 // Planes per item when the caller has not chosen: a step takes about its items'
 // planes (and 1.1 plane-times of prologue each) spread over the resident
-// blocks, but no less than its longest item, which the next step of that
-// member waits for.  The reference mix gets whole columns, at most 128 planes
-// (0.366 ms a step of its DUGKS members; 16 planes: 0.421, 32: 0.385, 64: 0.373).
+// blocks, but no less than any member's own items take on all of them, round by
+// round: that member's next step waits for the last.  Without the second bound a
+// mix with one large member gets a nearly empty second round (us a step, one
+// 96^3 and one 24^3 DUGKS member beside LBE: 24 planes 122, the 14 chosen now 89.5,
+// the best of a sweep 82 with 32; one of 50^3: 3 planes 22.3, 4 16.4).  The reference mix gets whole columns, at
+// most 128 planes (0.366 ms a step of its DUGKS members; 16 planes: 0.421, 32:
+// 0.385, 64: 0.373).
 int default_zchunk(const kin_ensemble* e) {
-    int nsm = 0;
+    int nsm = 0, top = 1;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, e->device) != cudaSuccess || nsm <= 0) nsm = 152;
     const double slots = nsm * (e->tile_y <= 5 ? 2.0 : 1.0);
+    for (int m : e->dugks_ids) top = std::max(top, e->members[m]->N);
     int best = 1;
     double best_cost = -1.0;
-    for (int zc : {1024, 512, 256, 128, 96, 64, 48, 32, 24, 16, 11, 8, 6, 4, 3, 2, 1}) {
+    for (int zc = top; zc >= 1; --zc) {
         double sum = 0.0, longest = 0.0;
         for (int m : e->dugks_ids) {
-            const int N = e->members[m]->N, c = std::min(zc, N);
+            const int N = e->members[m]->N, c = std::min(zc, N), nz = (N + c - 1) / c;
             const double cols = (double)((N + 29) / 30) * ((N + e->tile_y - 1) / e->tile_y);
-            sum += cols * (N + 1.1 * ((N + c - 1) / c));
-            longest = std::max(longest, c + 1.1);
+            sum += cols * (N + 1.1 * nz);
+            longest = std::max(longest, std::ceil(cols * nz / slots) * (c + 1.1));
         }
         const double cost = std::max(sum / slots, longest);
         if (best_cost < 0.0 || cost < best_cost) {
