@@ -127,7 +127,11 @@ int kin_get_velocity(kin_sim* sim, double* u);
  * KIN_EINVAL for max_iter < 1; KIN_ENONFINITE if it diverges. */
 int kin_init_consistent(kin_sim* sim, int max_iter, double tol, int* iters, double* residual);
 
-/* Enqueue n >= 0 time steps on the simulation's stream and return. */
+/* Enqueue n >= 0 time steps on the simulation's stream and return.  The stream
+ * may be capturing a graph: with an even n each replay advances the state by n
+ * steps from where it is (an odd n leaves the state in the buffer that the next
+ * replay does not read; kin_get_step counts the captured call once, replays not
+ * at all). */
 int kin_step(kin_sim* sim, int n);
 
 /* Statistics of the current state (synchronises the stream):

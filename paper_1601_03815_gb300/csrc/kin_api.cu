@@ -176,19 +176,34 @@ int launch_step(kin_sim* s, float* uvel = nullptr) {
     return KIN_OK;
 }
 
+bool capturing(cudaStream_t stream) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &status) != cudaSuccess) {
+        cudaGetLastError();  // the launch returns the error of such a stream
+        return false;
+    }
+    return status == cudaStreamCaptureStatusActive;
+}
+
 // n steps; the last one with uvel as in launch_step.  LBE steps go in pairs where
 // one pass over memory for two of them is the faster way (an explicit block size
-// keeps the single-step kernel it is meant for).
+// keeps the single-step kernel it is meant for).  Every launch moves the state to
+// the other buffer, and a graph reads the buffer it was captured on at every
+// replay: under capture the launches are made an even number, one pair taken as two
+// single steps if need be, so that a replay continues where the last one ended.
 int launch_steps(kin_sim* s, int n, float* uvel) {
     int k = 0;
-    if (s->scheme == KIN_LBE_MRT && s->block_lbe == 0 && lbe_pairs(s->storage, s->N))
-        for (; k + 2 <= n; k += 2) {
+    if (s->scheme == KIN_LBE_MRT && s->block_lbe == 0 && lbe_pairs(s->storage, s->N)) {
+        int pairs = n / 2;
+        if (pairs > 0 && (n - pairs) % 2 && capturing(s->stream)) --pairs;
+        for (; k < 2 * pairs; k += 2) {
             CK(lbe_pair_step(s->storage, s->buf[s->cur], s->buf[s->cur ^ 1], s->N, s->nu, s->num_sms, s->stream));
             s->launches += 1;
             s->cur ^= 1;
             s->step += 2;
             s->epoch += 1;
         }
+    }
     for (; k < n; ++k)
         if (int r = launch_step(s, k == n - 1 ? uvel : nullptr)) return r;
     return KIN_OK;
