@@ -52,9 +52,12 @@ public:
         for (std::thread& t : threads_) t.join();
     }
 
+    // Whether threads are at work on the pages.
+    bool pending() const { return !threads_.empty(); }
+
     // Returns once [p, p + end) may be overwritten.
     void wait(size_t end) const {
-        if (threads_.empty()) return;
+        if (!pending()) return;
         const size_t parts = std::min(parts_, (end + kPart - 1) / kPart);
         for (size_t k = 0; k < parts; ++k)
             while (!done_[k].load(std::memory_order_acquire)) std::this_thread::yield();

@@ -101,10 +101,12 @@ int ensure_u(kin_sim* s) {
 }
 
 // Enqueue the copy of bytes from dev to offset off of the result array behind
-// pages, each part once its pages are there.
+// pages, each part once its pages are there; in one piece where they are there
+// already (parts into a reused array: 256^3 populations 14.9 -> 16.1 ms).
 int copy_out(kin_sim* s, HostPages& pages, char* host, size_t off, const void* dev, size_t bytes) {
     for (size_t at = 0; at < bytes;) {
-        const size_t end = std::min(off + bytes, (off + at) / HostPages::kPart * HostPages::kPart + HostPages::kPart);
+        const size_t part = (off + at) / HostPages::kPart * HostPages::kPart + HostPages::kPart;
+        const size_t end = pages.pending() ? std::min(off + bytes, part) : off + bytes;
         const size_t n = end - (off + at);
         pages.wait(end);
         CK(cudaMemcpyAsync(host + off + at, static_cast<const char*>(dev) + at, n, cudaMemcpyDeviceToHost, s->stream));

@@ -40,6 +40,8 @@ int main() {
         h.wait(n);
         g.wait(n);
     }
+    // what is there needs no parts: the copy is one
+    if (kin::HostPages(a, n).pending()) return 4;
     for (size_t k = 0; k < n; k += 64)
         if (q[k] != 1) return 2;
     for (size_t k = page; k < n; k += 2 * page)
