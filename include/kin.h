@@ -219,8 +219,8 @@ int kin_energy_dissipation_noalloc(const double* u, int N, double nu, double* ou
  * the buffer, side and first changed byte (a kernel wrote outside the state).
  * Synchronous.
  * kin_debug_status: *is_debug (may be NULL) = 1 when this library was built
- * with KIN_DEBUG, whose stencil kernels check every global offset
- * and row index before use, skip an access that fails
+ * with KIN_DEBUG, whose stencil kernels check every global offset and the
+ * shared-memory slots, rows and indices before use, skip an access that fails
  * and record the first failure (bits 40..47: check site, bits 0..39: the
  * offending value) instead of trapping.  *word (may be NULL) receives that
  * record, 0 if every check passed (always 0 in the release build); reset != 0

@@ -322,7 +322,14 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
     const int lane = opaque((int)threadIdx.x);
     const bool halo = threadIdx.y == TY;
     const int row = opaque(halo ? 0 : (int)threadIdx.y + 1);
+    // Every shared-memory access is own (or own + (TY + 1) rows in the halo warp) plus a
+    // constant.  Of the arrays of TY + 2 rows that reaches one row up or down of rows 1
+    // to TY and one quad beside a row; of the bases rows 1 to TY.
+    static_assert(SM::XCH >= (int)sizeof(Q4) && SM::MY == SM::XCH + 2 * NXQ * SM::QX && SM::FY == SM::MY + 4 * SM::QX &&
+                      SM::BASE + SM::ROW == SM::FY + 3 * SM::QX && SM::BYTES == SM::BASE + SM::ROW + 2 * NBQ * SM::QB,
+                  "the arrays follow one another");
     (void)KIN_CHECK((int)threadIdx.y <= TY && lane < 32, DBG_DUGKS_ROW, threadIdx.y);
+    (void)KIN_CHECK(row >= 0 && row <= TY && (halo ? row == 0 : row >= 1), DBG_DUGKS_SLOT, row);
     const unsigned own = opaque((unsigned)__cvta_generic_to_shared(smem_raw) + row * SM::ROW + lane * (int)sizeof(Q4));
     const int z0 = bz * zchunk;
     const int zend = min(z0 + zchunk, N);
@@ -332,6 +339,7 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
     // WRAP: the lanes of the x neighbours and their distance in shared memory
     [[maybe_unused]] const int right = WRAP ? (lane + 1 == N ? 0 : min(lane + 1, 31)) : 0;
     [[maybe_unused]] const int left = WRAP ? (lane == 0 ? N - 1 : lane - 1) : 0;
+    (void)KIN_CHECK(right >= 0 && right < 32 && left >= 0 && left < 32, DBG_DUGKS_SLOT, right * 64 + left);
     [[maybe_unused]] const int to_right = (right - lane) * (int)sizeof(Q4), to_left = (left - lane) * (int)sizeof(Q4);
     const size_t plane = (size_t)N * N * N;
     // cell indices fit in 32 bits (N <= 1024)

@@ -298,7 +298,7 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
 #pragma unroll
                     for (int i = 0; i < Q; ++i)
                         if (KIN_CHECK(o + i * plane + 1 < Q * plane, DBG_DUGKS_LOAD, o + i * plane + 1) &&
-                            KIN_CHECK(s >= 0 && s < 4, DBG_DUGKS_ROW, s))
+                            KIN_CHECK(s >= 0 && s < 4, DBG_DUGKS_SLOT, s))
                             cp_async4(&stage16->raw[s][i][r2][2 * lane], src + o + i * plane);
                 }
             }
@@ -422,7 +422,7 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
 
     for (int z = z0; z <= zend; ++z) {
         const bool last = z == zend;
-        if (!KIN_CHECK(s_m1 >= 0 && s_m1 < 3 && s_0 >= 0 && s_0 < 3 && s_p1 >= 0 && s_p1 < 3, DBG_DUGKS_ROW,
+        if (!KIN_CHECK(s_m1 >= 0 && s_m1 < 3 && s_0 >= 0 && s_0 < 3 && s_p1 >= 0 && s_p1 < 3, DBG_DUGKS_SLOT,
                        s_m1 * 100 + s_0 * 10 + s_p1))
             break;
         __syncthreads();  // fy of plane z - 1 complete; my of plane z - 1 consumed

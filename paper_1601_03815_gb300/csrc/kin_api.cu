@@ -846,11 +846,14 @@ int kin_debug_status(int* is_debug, unsigned long long* word, int reset) {
 #else
     if (is_debug) *is_debug = 0;
 #endif
-    unsigned long long w[3] = {0, 0, 0};
+    unsigned long long w[4] = {0, 0, 0, 0};
     CK(debug_word_dugks(&w[0], reset != 0));
     CK(debug_word_lbe(&w[1], reset != 0));
     CK(debug_word_ensemble(&w[2], reset != 0));
-    const unsigned long long first = w[0] ? w[0] : (w[1] ? w[1] : w[2]);
+    CK(debug_word_stats(&w[3], reset != 0));
+    unsigned long long first = 0;
+    for (unsigned long long v : w)
+        if (!first) first = v;
     if (word) *word = first;
     if (first)
         return fail(KIN_EDEBUG, "index check failed at site %llu with value %llu", first >> 40,

@@ -1,7 +1,7 @@
 // Index checks of the KIN_DEBUG build (compute-sanitizer's substitute).
 //
-// With KIN_DEBUG defined, the stencil kernels check the global offsets and
-// row indices they are about to use.  A failed check
+// With KIN_DEBUG defined, the stencil kernels check the global offsets and the
+// shared-memory slots, rows and indices they are about to use.  A failed check
 // skips that access (no trap, no fault: the kernel runs on and the context
 // stays usable) and records the first failure of the translation unit in a
 // device word: bits 40..47 the check site, bits 0..39 the offending value.
@@ -17,9 +17,11 @@ namespace kin {
 enum : unsigned {
     DBG_DUGKS_LOAD = 1,   // global f-tilde read of the DUGKS tile (copy or load)
     DBG_DUGKS_STORE = 2,  // global store of the new f-tilde / velocity
+    DBG_DUGKS_SLOT = 3,   // ring or staging slot, or shared-memory address
     DBG_DUGKS_ROW = 4,    // row index of a warp of the DUGKS tile
     DBG_LBE_LOAD = 5,     // global pull of the LBE node
     DBG_LBE_STORE = 6,    // global store of the LBE node
+    DBG_LBE_SLOT = 7,     // shared-memory index of a pair of LBE steps
 };
 
 #ifdef KIN_DEBUG

@@ -117,11 +117,12 @@ cudaError_t sample_cells(int storage, const void* state, bool shifted, int N,
                          const int64_t* cells, int64_t n, double* out, cudaStream_t stream);
 
 // First failed index check of a KIN_DEBUG build in the translation units of
-// the fused DUGKS step, the LBE step and the ensemble kernel (0: none, or not
-// a debug build); reset clears it.
+// the fused DUGKS step, the LBE step, the ensemble kernel and the statistics (0:
+// none, or not a debug build); reset clears it.
 cudaError_t debug_word_dugks(unsigned long long* word, bool reset);
 cudaError_t debug_word_lbe(unsigned long long* word, bool reset);
 cudaError_t debug_word_ensemble(unsigned long long* word, bool reset);
+cudaError_t debug_word_stats(unsigned long long* word, bool reset);
 
 // Non-finite check of a double array: flag[0] |= 1 if any element is NaN/Inf.
 cudaError_t scan_nonfinite(const double* v, size_t n, int* flag, cudaStream_t stream);

@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(32 * (TY + 2), kPairBlocks)
     const int nn = N * N, n3 = nn * N;  // N <= 1024
     float* const own = smem_f + row * 32 + lane;
     grid_begin();
+    (void)KIN_CHECK(row < SM::ROWS && lane < 32, DBG_LBE_SLOT, row * 64 + lane);
 
     // plane offsets of planes k - 1, k, k + 1 of the next load (N >= 2)
     int zo[3];
@@ -102,6 +103,11 @@ __global__ void __launch_bounds__(32 * (TY + 2), kPairBlocks)
         if (k < zend) load();
         __syncthreads();
         if (k > z0 && yin) {
+            // the slots' first words; a row, and a word beside it, each way is inside (yin)
+            (void)KIN_CHECK(up >= 0 && up < SM::FLAT - SM::UP && up_before >= 0 && up_before < SM::FLAT - SM::UP &&
+                                flat >= 0 && flat < SM::DOWN - SM::FLAT && flat_before >= 0 &&
+                                flat_before < SM::DOWN - SM::FLAT && down >= 0 && down < 8 * SM::POP,
+                            DBG_LBE_SLOT, up);
             float g[Q];
             g[0] = rest;
             g[5] = z5b;
@@ -166,7 +172,8 @@ __global__ void __launch_bounds__(32 * (TY + 2) * (TZ + 2), 1)
     const int xs[3] = {wrap_dec(lane, N), lane, wrap_inc(lane, N)};
     static_for<1, Q>([&](auto ic) {
         constexpr int I = decltype(ic)::value;
-        f[I] = smem_f[I * POP + at - (cz(I) * ROWS + cy(I)) * 32 + xs[1 - cx(I)]];
+        const int idx = I * POP + at - (cz(I) * ROWS + cy(I)) * 32 + xs[1 - cx(I)];
+        if (KIN_CHECK(idx >= I * POP && idx < (I + 1) * POP, DBG_LBE_SLOT, idx)) f[I] = smem_f[idx];
     });
     mrt_collide_as<S, false>(f, rates);
     lbe_scatter<S>(dst, N, plane, lane, yr, zr, f);

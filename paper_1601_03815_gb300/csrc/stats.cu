@@ -96,6 +96,8 @@ __device__ __forceinline__ void add_velocity(float (&j)[3], float v) {
     if constexpr (cz(I) < 0) j[2] -= v;
 }
 
+KIN_DEBUG_ACCESSOR(debug_word_stats)
+
 template <typename S, bool SHIFTED>
 __global__ void velocity32_kernel(const S* st, int N, size_t plane, float* __restrict__ u) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
