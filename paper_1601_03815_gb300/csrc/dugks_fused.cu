@@ -60,7 +60,7 @@ static cudaError_t launch_fused16_t(const void* src, void* dst, int N, int zchun
     const cudaError_t e = allow_smem<dugks_fused16_kernel<S, TY, VEL, EVEN>>(smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((N + 29) / 30, (N + TY - 1) / TY, (N + zchunk - 1) / zchunk);
-    // an ordinary launch: its copies go through L1
+    // an ordinary launch: its copies and, for odd N, its loads go through L1
     dugks_fused16_kernel<S, TY, VEL, EVEN><<<grid, dim3(32, TY + 2), smem, stream>>>((const S*)src, (S*)dst, N, zchunk, k,
                                                                                     uvel);
     return cudaGetLastError();

@@ -305,6 +305,9 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
         }
         cp_async_commit();
     };
+    // Odd N reads a value again at each use, through the read-only path: only ordinary
+    // launches run this form, whose source no kernel writes meanwhile (97^3 FP16 92 us
+    // a step; from L2 each time 146).
     auto raw_pair = [&](int z, int q) -> P2 {
         if constexpr (use16) {
             const int s = rslot_of(z);
@@ -314,7 +317,7 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
             const size_t o = (size_t)zwrap(z) * nn + colidx;
             if (!KIN_CHECK(o + (2 * q + 2) * plane < Q * plane, DBG_DUGKS_LOAD, o + (2 * q + 2) * plane))
                 return pmk(C(0), C(0));
-            return pmk(Traits<S>::load_l2(src + o + (2 * q + 1) * plane), Traits<S>::load_l2(src + o + (2 * q + 2) * plane));
+            return pmk(Traits<S>::load(src + o + (2 * q + 1) * plane), Traits<S>::load(src + o + (2 * q + 2) * plane));
         }
     };
     auto raw_rest = [&](int z) -> C {
@@ -323,7 +326,7 @@ __device__ __forceinline__ void dugks_tile(const S* __restrict__ src, S* __restr
         } else {
             const size_t o = (size_t)zwrap(z) * nn + colidx;
             if (!KIN_CHECK(o < plane, DBG_DUGKS_LOAD, o)) return C(0);
-            return Traits<S>::load_l2(src + o);
+            return Traits<S>::load(src + o);
         }
     };
 
