@@ -138,8 +138,7 @@ struct TileShape {
 constexpr TileShape kShapes[] = {{4, 2, 1.5, 1.85, false}, {5, 2, 1.28, 2.0, false}, {8, 1, 1.76, 1.76, true}, {11, 1, 2.1, 2.1, false}};
 constexpr TileShape kShapes64[] = {{3, 1, 21.3, 21.3, true}, {7, 1, 41.5, 41.5, false}};
 
-// FP16 and BF16: one block an SM
-constexpr TileShape kShapes16[] = {{8, 1, 1.9, 1.9, false}, {4, 1, 1.3, 1.3, false}};
+constexpr long long kMaxBlocks = 20000;  // of a grid that is considered
 
 long long columns(int N, const TileShape& t) {
     const int ty = t.ty;
@@ -156,6 +155,30 @@ double makespan(int N, const TileShape& t, int zc, int nsm) {
     return plane * tile_schedule(cols, N, zc, (long long)nsm * t.per_sm, 1.1);
 }
 
+// Planes per block of the FP16 and BF16 step, one block an SM with a prologue of 1.5
+// plane-times: from 1.5 waves of columns on chunks that make about two waves of
+// blocks (256^3: 240 + 16 planes, the measured optimum), else the length with the
+// shortest schedule.  Lengths that leave a shorter last chunk are tried too: its
+// blocks fill the last wave (us a step against even chunks: 88^3 47.3 / 51.4, 128^3
+// 155 / 165, 192^3 439 / 455).
+int two_byte_zchunk(int N, int ty, int nsm) {
+    const long long cols = (long long)((N + 29) / 30) * ((N + ty - 1) / ty);
+    if (2 * cols >= 3LL * nsm)
+        return (int)std::max(8LL, std::min<long long>((long long)N * cols / (2LL * nsm) / 8 * 8, N));
+    double best = -1.0;
+    int zc = N;
+    for (int c = N; c >= 1; --c) {
+        const int nz = (N + c - 1) / c;
+        if (nz > 1 && (nz > 64 || cols * nz > kMaxBlocks)) break;
+        const double m = tile_schedule(cols, N, c, nsm, 1.5);
+        if (best < 0.0 || m < best * (1.0 - 0.005)) {
+            best = m;
+            zc = c;
+        }
+    }
+    return zc;
+}
+
 }  // namespace
 
 // The step lasts as long as its busiest SM, so a chunk length that leaves the
@@ -168,7 +191,6 @@ double makespan(int N, const TileShape& t, int zc, int nsm) {
 // (5 x 13: 66.6), 128^3 11 x 26 117 us (5 x 19: 119), 256^3 11 x 37 0.777 ms
 // (5 x 52: 0.773).
 void dugks_fused_shape(int storage, int N, int nsm, int want_ty, int want_zc, int* ty, int* zc) {
-    constexpr long long kMaxBlocks = 20000;
     double best = -1.0;
     auto consider = [&](const TileShape& t) {
         const long long cols = columns(N, t);
@@ -191,15 +213,8 @@ void dugks_fused_shape(int storage, int N, int nsm, int want_ty, int want_zc, in
         return;
     }
     if (storage != ST_F32) {
-        const TileShape& t = kShapes16[want_ty == 4];
-        const long long cols = (long long)((N + 29) / 30) * ((N + t.ty - 1) / t.ty);
-        if (want_zc <= 0 && 2 * cols >= 3LL * nsm) {
-            // about two waves of blocks (256^3: 240 + 16 planes, the measured optimum)
-            *ty = t.ty;
-            *zc = (int)std::max(8LL, std::min<long long>((long long)N * cols / (2LL * nsm) / 8 * 8, N));
-            return;
-        }
-        consider(t);
+        *ty = want_ty == 4 ? 4 : 8;
+        *zc = want_zc > 0 ? std::min(want_zc, N) : two_byte_zchunk(N, *ty, nsm);
         return;
     }
     for (const TileShape& t : kShapes)
