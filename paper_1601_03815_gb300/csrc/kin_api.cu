@@ -161,7 +161,7 @@ int launch_step(kin_sim* s, float* uvel = nullptr) {
     void* dst = s->buf[s->cur ^ 1];
     cudaError_t e;
     if (s->scheme == KIN_LBE_MRT)
-        e = lbe_step(s->storage, src, dst, s->N, s->nu, s->block_lbe, s->stream);
+        e = lbe_step(s->storage, src, dst, s->N, s->nu, s->block_lbe, s->num_sms, s->stream);
     else if (s->variant == 1)
         e = dugks_step(s->storage, src, dst, s->fbp, s->N, s->nu, s->dt, s->block_dugks, s->stream);
     else {

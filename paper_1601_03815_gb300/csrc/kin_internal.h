@@ -16,8 +16,9 @@ size_t storage_bytes(int storage);
 // MRT-LBE step (Eq. 21) in the pull arrangement: the buffer holds
 // buf_i(y) = f_i(y + xi_i, t) (pre-collision populations displaced by -xi_i);
 // one launch reads buf_i(x - xi_i) = f_i(x, t), collides and writes the
-// post-collision f*_i(x) to dst, which then holds buf for t + 1.
-cudaError_t lbe_step(int storage, const void* src, void* dst, int N, double nu, int block_x,
+// post-collision f*_i(x) to dst, which then holds buf for t + 1.  nsm:
+// multiprocessors of the device.
+cudaError_t lbe_step(int storage, const void* src, void* dst, int N, double nu, int block_x, int nsm,
                      cudaStream_t stream);
 
 // Two steps from src to dst in one launch (nsm multiprocessors), bitwise those of

@@ -70,8 +70,20 @@ static cudaError_t launch_lbe_v(const S* src, S* dst, int N, const MrtRates<floa
     else return launch_next(lbe_stepv_kernel<S, V>, grid, block, 0, stream, src, dst, N, plane, r);
 }
 
+// An FP64 step of a few warps an SM is bound by the busiest scheduler's FP64 pipe.
+// Blocks that wait beside the grid before them are placed around its warps, so that
+// some schedulers get several and others none; the ordinary launch spreads them
+// evenly.  us a step overlapped / ordinary: 16^3 6.7 / 8.2, 19^3 6.8 / 9.1, 20^3 28.8 /
+// 8.2, 24^3 29.2 / 10.3, 32^3 30.2 / 14.4, 34^3 31.1 / 26.8, 35^3 31.2 / 32.8, 48^3
+// 48.6 / 51.2, 64^3 84.0 / 86.1 (361 warps at 19^3, 400 at 20^3, 2312 at 34^3, 2520 at
+// 35^3; 2.5 and 16 warps an SM are 380 and 2432).
+static bool overlap_unbalances(const dim3& grid, const dim3& block, int nsm) {
+    const long long warps = (long long)grid.x * grid.y * grid.z * (block.x * block.y / 32);
+    return 2 * warps > 5LL * nsm && warps < 16LL * nsm;
+}
+
 template <typename S>
-static cudaError_t launch_lbe(const void* src, void* dst, int N, double nu, int bx,
+static cudaError_t launch_lbe(const void* src, void* dst, int N, double nu, int bx, int nsm,
                               cudaStream_t stream) {
     using C = typename Traits<S>::C;
     const MrtRates<C> r = lbe_rates<C>(nu);
@@ -83,6 +95,10 @@ static cudaError_t launch_lbe(const void* src, void* dst, int N, double nu, int 
     if (bx > 256) bx = 256;  // the kernel's launch bounds
     dim3 block, grid;
     step_shape(N, N, bx, block, grid);
+    if (sizeof(C) == 8 && overlap_unbalances(grid, block, nsm)) {
+        lbe_step_kernel<S><<<grid, block, 0, stream>>>((const S*)src, (S*)dst, N, (size_t)N * N * N, r);
+        return cudaGetLastError();
+    }
     return launch_next(lbe_step_kernel<S>, grid, block, 0, stream, (const S*)src, (S*)dst, N, (size_t)N * N * N, r);
 }
 
@@ -179,13 +195,13 @@ cudaError_t lbe_pair_step(int storage, const void* src, void* dst, int N, double
 
 KIN_DEBUG_ACCESSOR(debug_word_lbe)
 
-cudaError_t lbe_step(int storage, const void* src, void* dst, int N, double nu, int block_x,
+cudaError_t lbe_step(int storage, const void* src, void* dst, int N, double nu, int block_x, int nsm,
                      cudaStream_t stream) {
     switch (storage) {
-        case ST_F32: return launch_lbe<float>(src, dst, N, nu, block_x, stream);
-        case ST_F16: return launch_lbe<__half>(src, dst, N, nu, block_x, stream);
-        case ST_BF16: return launch_lbe<__nv_bfloat16>(src, dst, N, nu, block_x, stream);
-        case ST_F64: return launch_lbe<double>(src, dst, N, nu, block_x, stream);
+        case ST_F32: return launch_lbe<float>(src, dst, N, nu, block_x, nsm, stream);
+        case ST_F16: return launch_lbe<__half>(src, dst, N, nu, block_x, nsm, stream);
+        case ST_BF16: return launch_lbe<__nv_bfloat16>(src, dst, N, nu, block_x, nsm, stream);
+        case ST_F64: return launch_lbe<double>(src, dst, N, nu, block_x, nsm, stream);
     }
     return cudaErrorInvalidValue;
 }
