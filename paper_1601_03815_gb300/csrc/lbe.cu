@@ -15,10 +15,12 @@ namespace kin {
 // share a block (64^3 FP32 5.4 us a step instead of 6.1, 48^3 4.35 instead of
 // 4.45); one-warp rows stay apart (32^3 3.5 us against 4.0 with four rows a
 // block), and in larger boxes a row fills a block or the rows are many
-// (256^3 FP16: 214 us either way).
-static void step_shape(int nx, int N, int b, dim3& block, dim3& grid) {
+// (256^3 FP16: 214 us either way).  Where 32 threads are asked for in a longer row,
+// warps is the rows that share a block (one cell a thread, FP32: 4; blocks of one warp
+// each pay the overlapped start, 256^3 529 us, 372 with four rows).
+static void step_shape(int nx, int N, int b, int warps, dim3& block, dim3& grid) {
     const int bx = std::min(b, ((nx + 31) / 32) * 32);
-    const int by = bx >= 64 && N <= 64 ? std::max(1, b / bx) : 1;
+    const int by = bx >= 64 && N <= 64 ? std::max(1, b / bx) : bx == 32 && nx > 32 ? warps : 1;
     block = dim3(bx, by);
     grid = dim3((nx + bx - 1) / bx, (N + by - 1) / by, N);
 }
@@ -64,7 +66,7 @@ static cudaError_t launch_lbe_v(const S* src, S* dst, int N, const MrtRates<floa
     const int nv = N / V;
     int b = bx > 0 ? std::min(bx, 256) : 128;
     dim3 block, grid;
-    step_shape(nv, N, b, block, grid);
+    step_shape(nv, N, b, 1, block, grid);
     const size_t plane = (size_t)N * N * N;
     if constexpr (V == 4) return launch_next(lbe_stepv4_kernel<S>, grid, block, 0, stream, src, dst, N, plane, r);
     else return launch_next(lbe_stepv_kernel<S, V>, grid, block, 0, stream, src, dst, N, plane, r);
@@ -94,7 +96,7 @@ static cudaError_t launch_lbe(const void* src, void* dst, int N, double nu, int 
     if (bx <= 0) bx = 128;
     if (bx > 256) bx = 256;  // the kernel's launch bounds
     dim3 block, grid;
-    step_shape(N, N, bx, block, grid);
+    step_shape(N, N, bx, sizeof(C) == 8 ? 1 : 4, block, grid);
     if (sizeof(C) == 8 && overlap_unbalances(grid, block, nsm)) {
         lbe_step_kernel<S><<<grid, block, 0, stream>>>((const S*)src, (S*)dst, N, (size_t)N * N * N, r);
         return cudaGetLastError();
