@@ -301,10 +301,11 @@ typedef struct kin_ensemble kin_ensemble;
  * keeps ownership and must destroy the ensemble before any member). */
 int kin_ensemble_create(kin_sim* const* members, int n, kin_ensemble** out);
 
-/* Work decomposition: tile_y (4, 6 or 8; the default is 5-row tiles) and
- * zchunk of the DUGKS tiles (by default chosen for the members), lbe_block
- * (a multiple of 32, at most 128) threads
- * per block of the batched LBE launches; values <= 0 keep the setting. */
+/* Work decomposition: tile_y (4, 6 or 8; by default 5 for FP32 DUGKS members, 8
+ * for one 2-byte type, 6 for a mixture) and zchunk of the DUGKS tiles (by default
+ * chosen for the members), lbe_block (a multiple of 32, at most 128) threads per
+ * block of the batched LBE launches; values <= 0 keep the setting.  FP32 members
+ * beside 2-byte ones have tiles of one row more. */
 int kin_ensemble_set_tuning(kin_ensemble* ens, int tile_y, int zchunk, int lbe_block);
 
 /* Advance every member by nsteps (synchronous): one graph launch, or one per

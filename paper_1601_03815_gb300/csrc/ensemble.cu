@@ -77,12 +77,23 @@ __device__ __forceinline__ int ld_relaxed(const int* p) {
     return v;
 }
 
-// Rows of a 2-byte tile: it has a warp for each of its two halo rows, so the block
-// of a TY-row FP32 tile holds one row less.
-constexpr int rows16(int ty) { return ty - 1; }
+// Storage types of the DUGKS members of a kernel: one, or any mixture.  A kernel of
+// its own for each, since three tiles in one body spill where the registers of a block
+// are capped (8 rows: 664 bytes; one 2-byte type: none.  Four 64^3 FP16 members, 16
+// planes: 184 against 100 us a step).
+enum { HAS_F32 = 1, HAS_F16 = 2, HAS_BF16 = 4, HAS_MIXED = 7 };
+
+// Warps of a block and rows of its FP32 tiles at tile height ty.  A 2-byte tile has a
+// warp for each of its two halo rows, an FP32 tile one for both: in a kernel that
+// runs 2-byte members the block holds their ty rows, and FP32 tiles of one row more.
+constexpr int block_warps(int ty, int has) { return has == HAS_F32 ? ty + 1 : ty + 2; }
+constexpr int rows32(int ty, int has) { return block_warps(ty, has) - 1; }
+
+// Blocks an SM that the registers of a thread are held to.
+constexpr int blocks_an_sm(int ty, int has) { return ty <= 5 && has == HAS_F32 ? 2 : 1; }
 
 // One fused-DUGKS tile t of member M at buffer parity par.
-template <typename S, int TY>
+template <typename S, int TY, int HAS>
 __device__ __forceinline__ void ensemble_tile(const EnsMember& M, int par, int t, unsigned char* smem_raw) {
     const int per = M.tiles_x * M.tiles_y;
     const int bz = t / per, r = t % per;
@@ -92,14 +103,20 @@ __device__ __forceinline__ void ensemble_tile(const EnsMember& M, int par, int t
     const S* src = static_cast<const S*>(M.buf[par]);
     S* dst = static_cast<S*>(M.buf[par ^ 1]);
     if constexpr (sizeof(S) == 2)
-        two_byte::dugks_tile<S, rows16(TY)>(src, dst, M.N, r % M.tiles_x, r / M.tiles_x, bz, M.zchunk, kc, smem_raw);
+        two_byte::dugks_tile<S, TY>(src, dst, M.N, r % M.tiles_x, r / M.tiles_x, bz, M.zchunk, kc, smem_raw);
     else
-        dugks_tile<S, TY>(src, dst, M.N, r % M.tiles_x, r / M.tiles_x, bz, M.zchunk, kc, smem_raw);
+        dugks_tile<S, rows32(TY, HAS)>(src, dst, M.N, r % M.tiles_x, r / M.tiles_x, bz, M.zchunk, kc, smem_raw);
 }
 
-// WIDE: some member has 2-byte storage (even N); without it the kernel holds
-// only the FP32 tile and its registers.
-template <int TY, bool WIDE>
+// The tile as a function of its own: in the mixed kernel of 8-row tiles it spills at
+// most 268 bytes (64^3: 3 FP32, 2 FP16 members and 48^3 BF16 beside LBE, 64 planes: 297
+// -> 237 us a step).
+template <typename S, int TY, int HAS>
+__device__ __noinline__ void called_tile(const EnsMember& M, int par, int t, unsigned char* smem_raw) {
+    ensemble_tile<S, TY, HAS>(M, par, t, smem_raw);
+}
+
+template <int TY, int HAS>
 __device__ __forceinline__ void ensemble_body(const EnsMember* __restrict__ mem, const int2* __restrict__ items,
                                               int nitems, int nsteps, unsigned* done, unsigned* next_item,
                                               int* status, long long wait_cycles, int stall_test) {
@@ -145,12 +162,16 @@ __device__ __forceinline__ void ensemble_body(const EnsMember* __restrict__ mem,
             __syncthreads();
             if (s_abort) return;
             const int par = (M.cur + s) & 1;
-            if constexpr (WIDE) {
-                if (M.storage == ST_F16) ensemble_tile<__half, TY>(M, par, item.y, smem_raw);
-                else if (M.storage == ST_BF16) ensemble_tile<__nv_bfloat16, TY>(M, par, item.y, smem_raw);
-                else ensemble_tile<float, TY>(M, par, item.y, smem_raw);
+            if constexpr (HAS == HAS_MIXED && TY == 8) {
+                if (M.storage == ST_F16) called_tile<__half, TY, HAS>(M, par, item.y, smem_raw);
+                else if (M.storage == ST_BF16) called_tile<__nv_bfloat16, TY, HAS>(M, par, item.y, smem_raw);
+                else called_tile<float, TY, HAS>(M, par, item.y, smem_raw);
+            } else if (HAS == HAS_F16 || (HAS == HAS_MIXED && M.storage == ST_F16)) {
+                ensemble_tile<__half, TY, HAS>(M, par, item.y, smem_raw);
+            } else if (HAS == HAS_BF16 || (HAS == HAS_MIXED && M.storage == ST_BF16)) {
+                ensemble_tile<__nv_bfloat16, TY, HAS>(M, par, item.y, smem_raw);
             } else {
-                ensemble_tile<float, TY>(M, par, item.y, smem_raw);
+                ensemble_tile<float, TY, HAS>(M, par, item.y, smem_raw);
             }
             __syncthreads();
             if (tid == 0) red_release_add(&done[item.x], 1u);
@@ -162,9 +183,9 @@ __device__ __forceinline__ void ensemble_body(const EnsMember* __restrict__ mem,
     const EnsMember *__restrict__ mem, const int2 *__restrict__ items, int nitems, int nsteps, unsigned *done, \
         unsigned *next_item, int *status, long long wait_cycles, int stall_test
 
-template <int TY, bool WIDE>
-__global__ void __launch_bounds__(32 * (TY + 1), TY <= 5 ? 2 : 1) ensemble_kernel(KIN_ENSEMBLE_PARAMS) {
-    ensemble_body<TY, WIDE>(mem, items, nitems, nsteps, done, next_item, status, wait_cycles, stall_test);
+template <int TY, int HAS>
+__global__ void __launch_bounds__(32 * block_warps(TY, HAS), blocks_an_sm(TY, HAS)) ensemble_kernel(KIN_ENSEMBLE_PARAMS) {
+    ensemble_body<TY, HAS>(mem, items, nitems, nsteps, done, next_item, status, wait_cycles, stall_test);
 }
 
 // One LBE step of every member in tab[0 .. nmem) (one storage type): block b
@@ -210,13 +231,11 @@ using namespace kin;
 struct kin_ensemble {
     std::vector<kin_sim*> members;
     std::vector<int> dugks_ids, lbe_ids;  // members of each scheme, in member order
-    bool wide = false;                    // a DUGKS member has 2-byte storage
+    int has = 0;                          // the DUGKS members' storage types (HAS_*)
     int device = 0;
     cudaStream_t stream = nullptr;  // persistent DUGKS launch (and the graph's origin)
     cudaStream_t side = nullptr;    // batched LBE launches inside the graph
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    // 5-row tiles, two 6-warp blocks an SM: 0.366 ms a step for the DUGKS members
-    // of the reference mix, against 0.402 (4 rows), 0.568 (6), 0.436 (8)
     int tile_y = 5, lbe_block = 128;
     int zchunk = 0;  // 0: chosen for the members (default_zchunk)
     int zc = 1;      // planes per item in use
@@ -257,25 +276,43 @@ void drop_graphs(kin_ensemble* e) {
     e->graphs.clear();
 }
 
-template <int TY, bool WIDE>
+template <int TY, int HAS>
 size_t persistent_smem() {
-    return WIDE ? std::max(fused_smem_bytes<float, TY>(),
-                           two_byte::tile_smem_bytes<__half, rows16(TY)>())
-                : fused_smem_bytes<float, TY>();
+    const size_t fp32 = fused_smem_bytes<float, rows32(TY, HAS)>();
+    return HAS == HAS_F32 ? fp32 : std::max(fp32, two_byte::tile_smem_bytes<__half, TY>());
 }
 
-template <int TY, bool WIDE>
+template <int TY, int HAS>
 int configure(kin_ensemble* e) {
-    const size_t smem = persistent_smem<TY, WIDE>();
-    ECK(cudaFuncSetAttribute(ensemble_kernel<TY, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const size_t smem = persistent_smem<TY, HAS>();
+    ECK(cudaFuncSetAttribute(ensemble_kernel<TY, HAS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem));
     int per_sm = 0, nsm = 0;
-    ECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ensemble_kernel<TY, WIDE>, 32 * (TY + 1),
+    ECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ensemble_kernel<TY, HAS>, 32 * block_warps(TY, HAS),
                                                       smem));
     ECK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, e->device));
     if (per_sm < 1) return set_error(KIN_ECUDA, "ensemble kernel does not fit on an SM");
     e->grid = std::min(per_sm * nsm, std::max(e->nitems, 1));
     return KIN_OK;
+}
+
+// f(tile height, storage types) of the kernel that this ensemble runs, as constants.
+template <typename F>
+auto with_kernel(const kin_ensemble* e, F&& f) {
+    auto of_height = [&](auto ty) {
+        switch (e->has) {
+            case HAS_F32: return f(ty, std::integral_constant<int, HAS_F32>{});
+            case HAS_F16: return f(ty, std::integral_constant<int, HAS_F16>{});
+            case HAS_BF16: return f(ty, std::integral_constant<int, HAS_BF16>{});
+        }
+        return f(ty, std::integral_constant<int, HAS_MIXED>{});
+    };
+    switch (e->tile_y) {
+        case 4: return of_height(std::integral_constant<int, 4>{});
+        case 5: return of_height(std::integral_constant<int, 5>{});
+        case 6: return of_height(std::integral_constant<int, 6>{});
+    }
+    return of_height(std::integral_constant<int, 8>{});
 }
 
 int storage_group(int storage) { return storage == ST_F16 ? 1 : storage == ST_BF16 ? 2 : 0; }
@@ -284,6 +321,19 @@ int storage_group(int storage) { return storage == ST_F16 ? 1 : storage == ST_BF
 int lbe_vector(const kin_sim* s) {
     if (s->storage == ST_F32) return 1;
     return s->N % 4 == 0 ? 4 : s->N % 2 == 0 ? 2 : 1;
+}
+
+// Rows of the tiles when the caller has not chosen.  FP32: 5, two 6-warp blocks an SM
+// (0.366 ms a step for the DUGKS members of the reference mix, against 0.402 with 4
+// rows, 0.568 with 6, 0.436 with 8).  One 2-byte type: 8, as stand-alone (the DUGKS and
+// LBE members of half the reference mix in FP16: 575 us, 4 rows 765, 5 rows 760, 6 rows
+// 695).  A mixture: 6, the most rows whose block takes 255 registers (2 FP32 and 2 FP16
+// 96^3 members of each scheme: 376 us, 4 rows 457, 5 rows 422, 8 rows 557).
+int default_tile_y(int has) { return has == HAS_F32 ? 5 : has == HAS_MIXED ? 6 : 8; }
+
+// Rows of the tiles of a DUGKS member.
+int tile_rows(const kin_ensemble* e, const kin_sim* s) {
+    return s->storage == ST_F32 ? rows32(e->tile_y, e->has) : e->tile_y;
 }
 
 // DUGKS table from the members' current state (buffers, parity, nu, dt).
@@ -300,7 +350,7 @@ std::vector<EnsMember> dugks_table(const kin_ensemble* e) {
         M.coef = dugks_coef<float>(s->nu, s->dt);
         const int zc = std::min(e->zc, s->N);
         M.tiles_x = (s->N + 29) / 30;
-        const int rows = s->storage == ST_F32 ? e->tile_y : rows16(e->tile_y);
+        const int rows = tile_rows(e, s);
         M.tiles_y = (s->N + rows - 1) / rows;
         M.zchunk = zc;
         M.ntiles = M.tiles_x * M.tiles_y * ((s->N + zc - 1) / zc);
@@ -341,10 +391,7 @@ int launch_persistent_config(kin_ensemble* e) {
         e->grid = 0;
         return KIN_OK;
     }
-    if (e->tile_y == 5) return e->wide ? configure<5, true>(e) : configure<5, false>(e);
-    if (e->tile_y == 4) return e->wide ? configure<4, true>(e) : configure<4, false>(e);
-    if (e->tile_y == 6) return e->wide ? configure<6, true>(e) : configure<6, false>(e);
-    return e->wide ? configure<8, true>(e) : configure<8, false>(e);
+    return with_kernel(e, [&](auto ty, auto has) { return configure<ty(), has()>(e); });
 }
 
 // Planes per item when the caller has not chosen: a step takes about its items'
@@ -359,7 +406,7 @@ int launch_persistent_config(kin_ensemble* e) {
 int default_zchunk(const kin_ensemble* e) {
     int nsm = 0, top = 1;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, e->device) != cudaSuccess || nsm <= 0) nsm = 152;
-    const double slots = nsm * (e->tile_y <= 5 ? 2.0 : 1.0);
+    const double slots = (double)nsm * blocks_an_sm(e->tile_y, e->has);
     for (int m : e->dugks_ids) top = std::max(top, e->members[m]->N);
     int best = 1;
     double best_cost = -1.0;
@@ -367,7 +414,8 @@ int default_zchunk(const kin_ensemble* e) {
         double sum = 0.0, longest = 0.0;
         for (int m : e->dugks_ids) {
             const int N = e->members[m]->N, c = std::min(zc, N), nz = (N + c - 1) / c;
-            const double cols = (double)((N + 29) / 30) * ((N + e->tile_y - 1) / e->tile_y);
+            const int rows = tile_rows(e, e->members[m]);
+            const double cols = (double)((N + 29) / 30) * ((N + rows - 1) / rows);
             sum += cols * (N + 1.1 * nz);
             longest = std::max(longest, std::ceil(cols * nz / slots) * (c + 1.1));
         }
@@ -412,12 +460,12 @@ long long wait_cycles(const kin_ensemble* e) {
     return (long long)(e->wait_seconds * 1e3 * khz);
 }
 
-template <int TY, bool WIDE>
+template <int TY, int HAS>
 cudaError_t launch_persistent_t(kin_ensemble* e, int nsteps, int stall_test) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(e->grid);
-    cfg.blockDim = dim3(32, TY + 1);
-    cfg.dynamicSmemBytes = persistent_smem<TY, WIDE>();
+    cfg.blockDim = dim3(32, block_warps(TY, HAS));
+    cfg.dynamicSmemBytes = persistent_smem<TY, HAS>();
     cfg.stream = e->stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -425,25 +473,14 @@ cudaError_t launch_persistent_t(kin_ensemble* e, int nsteps, int stall_test) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const int nd = (int)e->dugks_ids.size();
-    return cudaLaunchKernelEx(&cfg, ensemble_kernel<TY, WIDE>, (const EnsMember*)e->d_mem,
+    return cudaLaunchKernelEx(&cfg, ensemble_kernel<TY, HAS>, (const EnsMember*)e->d_mem,
                               (const int2*)e->d_items, e->nitems, nsteps, e->d_done, e->d_done + nd, e->d_status,
                               wait_cycles(e), stall_test);
 }
 
 int launch_persistent(kin_ensemble* e, int nsteps, int stall_test) {
-    cudaError_t err;
-    if (e->tile_y == 4)
-        err = e->wide ? launch_persistent_t<4, true>(e, nsteps, stall_test)
-                      : launch_persistent_t<4, false>(e, nsteps, stall_test);
-    else if (e->tile_y == 5)
-        err = e->wide ? launch_persistent_t<5, true>(e, nsteps, stall_test)
-                      : launch_persistent_t<5, false>(e, nsteps, stall_test);
-    else if (e->tile_y == 6)
-        err = e->wide ? launch_persistent_t<6, true>(e, nsteps, stall_test)
-                      : launch_persistent_t<6, false>(e, nsteps, stall_test);
-    else
-        err = e->wide ? launch_persistent_t<8, true>(e, nsteps, stall_test)
-                      : launch_persistent_t<8, false>(e, nsteps, stall_test);
+    const cudaError_t err = with_kernel(
+        e, [&](auto ty, auto has) { return launch_persistent_t<ty(), has()>(e, nsteps, stall_test); });
     if (err != cudaSuccess) return ens_fail(KIN_ECUDA, "ensemble launch", err);
     return KIN_OK;
 }
@@ -582,11 +619,13 @@ int kin_ensemble_create(kin_sim* const* members, int n, kin_ensemble** out) {
     for (int m = 0; m < n; ++m) {
         if (members[m]->scheme == KIN_DUGKS) {
             e->dugks_ids.push_back(m);
-            if (members[m]->storage != ST_F32) e->wide = true;
+            e->has |= members[m]->storage == ST_F16 ? HAS_F16 : members[m]->storage == ST_BF16 ? HAS_BF16 : HAS_F32;
         } else {
             e->lbe_ids.push_back(m);
         }
     }
+    if (e->has & (e->has - 1)) e->has = HAS_MIXED;
+    e->tile_y = default_tile_y(e->has);
     e->device = dev;
     int prev = 0;
     cudaGetDevice(&prev);
