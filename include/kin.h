@@ -256,6 +256,9 @@ int kin_num_shells(int N);
  * Other variant values return KIN_EINVAL. */
 int kin_set_tuning(kin_sim* sim, int block_x, int tile_y, int zchunk, int variant);
 
+/* Back to the library's own choice of everything that kin_set_tuning sets. */
+int kin_reset_tuning(kin_sim* sim);
+
 /* Number of kernel launches one kin_step(sim, 1) enqueues. */
 int kin_step_launches(const kin_sim* sim);
 
@@ -307,6 +310,9 @@ int kin_ensemble_create(kin_sim* const* members, int n, kin_ensemble** out);
  * block of the batched LBE launches; values <= 0 keep the setting.  FP32 members
  * beside 2-byte ones have tiles of one row more. */
 int kin_ensemble_set_tuning(kin_ensemble* ens, int tile_y, int zchunk, int lbe_block);
+
+/* Back to the defaults of everything that kin_ensemble_set_tuning sets. */
+int kin_ensemble_reset_tuning(kin_ensemble* ens);
 
 /* Advance every member by nsteps (synchronous): one graph launch, or one per
  * 256 steps when there are LBE members (a graph holds one LBE launch per

@@ -85,6 +85,7 @@ def _declare(lib):
         "kin_sync": (c_int, [P]),
         "kin_step_launches": (c_int, [P]),
         "kin_set_tuning": (c_int, [P, c_int, c_int, c_int, c_int]),
+        "kin_reset_tuning": (c_int, [P]),
         "kin_kernel_launches": (c_i64, [P]),
         "kin_get_nu": (c_double, [P]),
         "kin_get_dt": (c_double, [P]),
@@ -102,6 +103,7 @@ def _declare(lib):
         "kin_debug_status": (c_int, [P, P, c_int]),
         "kin_ensemble_create": (c_int, [P, c_int, P]),
         "kin_ensemble_set_tuning": (c_int, [P, c_int, c_int, c_int]),
+        "kin_ensemble_reset_tuning": (c_int, [P]),
         "kin_ensemble_step": (c_int, [P, c_int]),
         "kin_ensemble_test_timeout": (c_int, [P, c_double]),
         "kin_ensemble_info": (c_int, [P, P, P, P]),
@@ -320,6 +322,10 @@ class Sim:
         _check(lib().kin_set_tuning(self._h, int(block_x), int(tile_y), int(zchunk), int(variant)),
                "kin_set_tuning")
 
+    def reset_tuning(self):
+        """kin_reset_tuning: back to the library's own choices."""
+        _check(lib().kin_reset_tuning(self._h), "kin_reset_tuning")
+
     @property
     def step_launches(self) -> int:
         return int(lib().kin_step_launches(self._h))
@@ -375,6 +381,10 @@ class Ensemble:
     def set_tuning(self, tile_y: int = 0, zchunk: int = 0, lbe_block: int = 0):
         _check(lib().kin_ensemble_set_tuning(self._h, int(tile_y), int(zchunk), int(lbe_block)),
                "kin_ensemble_set_tuning")
+
+    def reset_tuning(self):
+        """kin_ensemble_reset_tuning: back to the defaults."""
+        _check(lib().kin_ensemble_reset_tuning(self._h), "kin_ensemble_reset_tuning")
 
     def step(self, n: int = 1):
         _check(lib().kin_ensemble_step(self._h, int(n)), "kin_ensemble_step")

@@ -228,6 +228,9 @@ KIN_DEBUG_ACCESSOR(debug_word_ensemble)
 
 using namespace kin;
 
+// Threads per block of the batched LBE launches when the caller has not chosen.
+constexpr int kLbeBlock = 128;
+
 struct kin_ensemble {
     std::vector<kin_sim*> members;
     std::vector<int> dugks_ids, lbe_ids;  // members of each scheme, in member order
@@ -236,7 +239,7 @@ struct kin_ensemble {
     cudaStream_t stream = nullptr;  // persistent DUGKS launch (and the graph's origin)
     cudaStream_t side = nullptr;    // batched LBE launches inside the graph
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    int tile_y = 5, lbe_block = 128;
+    int tile_y = 5, lbe_block = kLbeBlock;
     int zchunk = 0;  // 0: chosen for the members (default_zchunk)
     int zc = 1;      // planes per item in use
     EnsMember* d_mem = nullptr;
@@ -453,6 +456,16 @@ int build_tables(kin_ensemble* e) {
     return launch_persistent_config(e);
 }
 
+// The tables for a changed tuning.
+int retuned(kin_ensemble* e) {
+    int prev = 0;
+    cudaGetDevice(&prev);
+    cudaSetDevice(e->device);
+    const int r = build_tables(e);
+    cudaSetDevice(prev);
+    return r;
+}
+
 long long wait_cycles(const kin_ensemble* e) {
     int khz = 0;
     cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, e->device);
@@ -664,12 +677,15 @@ int kin_ensemble_set_tuning(kin_ensemble* e, int tile_y, int zchunk, int lbe_blo
     if (tile_y > 0) e->tile_y = tile_y;
     if (zchunk > 0) e->zchunk = zchunk;
     if (lbe_block > 0) e->lbe_block = lbe_block;
-    int prev = 0;
-    cudaGetDevice(&prev);
-    cudaSetDevice(e->device);
-    const int r = build_tables(e);
-    cudaSetDevice(prev);
-    return r;
+    return retuned(e);
+}
+
+int kin_ensemble_reset_tuning(kin_ensemble* e) {
+    if (!e) return set_error(KIN_EINVAL, "NULL ensemble");
+    e->tile_y = default_tile_y(e->has);
+    e->zchunk = 0;
+    e->lbe_block = kLbeBlock;
+    return retuned(e);
 }
 
 int kin_ensemble_step(kin_ensemble* e, int nsteps) {

@@ -776,6 +776,14 @@ int kin_set_tuning(kin_sim* s, int block_x, int tile_y, int zchunk, int variant)
     return KIN_OK;
 }
 
+int kin_reset_tuning(kin_sim* s) {
+    if (int r = valid(s)) return r;
+    s->block_lbe = s->block_dugks = 0;
+    s->tile_y = s->zchunk = s->variant = 0;
+    s->fused_ty = 0;
+    return KIN_OK;
+}
+
 int64_t kin_kernel_launches(const kin_sim* s) { return s ? s->launches : 0; }
 
 int kin_sync(kin_sim* s) {
