@@ -23,10 +23,11 @@ import time
 
 import numpy as np
 
-from . import DUGKS, F32, LBE_MRT, Ensemble, Sim
+from . import DUGKS, F32, LBE_MRT, STORAGE_NAMES, Ensemble, Sim
 
 REFERENCE_SIZES = ((32, 8), (64, 8), (96, 6), (128, 2))
-TUNE_TILE_Y = (0,)  # the library's 5-row tiles: 4, 6 and 8 rows were slower on every mix measured
+DEFAULT_TUNING = (0, 0, 0)  # the library's own choices
+TUNE_TILE_Y = (0,)  # the library's tile height: on the mixes measured others gain 2 % at most
 TUNE_ZCHUNK = (8, 16, 32, 64, 128)
 TUNE_LBE_BLOCK = (64, 128)
 
@@ -62,15 +63,23 @@ def _signature(sims):
     import torch
 
     dev = torch.cuda.get_device_name() if torch.cuda.is_available() else "cpu"
-    sizes = sorted((s.N, s.scheme) for s in sims)
-    # "d": tunings of the 5-row tiles
-    return "d|%s|%s" % (dev, ",".join("%d%s" % (n, "L" if sc == LBE_MRT else "D") for n, sc in sizes))
+    sizes = sorted((s.N, s.scheme, s.storage) for s in sims)
+    # "e": tunings beside the library's own choices, storage types told apart
+    return "e|%s|%s" % (dev, ",".join("%d%s%s" % (n, "L" if sc == LBE_MRT else "D", STORAGE_NAMES[st])
+                                      for n, sc, st in sizes))
+
+
+def set_tuning(ens: Ensemble, tuning):
+    """`tuning` (tile_y, zchunk, lbe_block), where 0 is the library's own choice."""
+    ens.reset_tuning()
+    if tuple(tuning) != DEFAULT_TUNING:
+        ens.set_tuning(*tuning)
 
 
 def autotune(ens: Ensemble, steps: int = 10, use_cache: bool = True, verbose: bool = False):
-    """Time every (tile_y, zchunk, lbe_block) candidate on this ensemble and
-    leave the fastest set.  The members advance while tuning.  Results are
-    cached per device and member mix."""
+    """Time the library's own choices and every (tile_y, zchunk, lbe_block)
+    candidate on this ensemble and leave the fastest set.  The members advance
+    while tuning.  Results are cached per device and member mix."""
     sig = _signature(ens.members)
     path = _cache_path()
     cache = {}
@@ -82,11 +91,11 @@ def autotune(ens: Ensemble, steps: int = 10, use_cache: bool = True, verbose: bo
             cache = {}
     if use_cache and sig in cache:
         best = cache[sig]
-        ens.set_tuning(*best["tuning"])
+        set_tuning(ens, best["tuning"])
         return best
     timings = []
-    for ty, zc, ln in itertools.product(TUNE_TILE_Y, TUNE_ZCHUNK, TUNE_LBE_BLOCK):
-        ens.set_tuning(ty, zc, ln)
+    for ty, zc, ln in [DEFAULT_TUNING, *itertools.product(TUNE_TILE_Y, TUNE_ZCHUNK, TUNE_LBE_BLOCK)]:
+        set_tuning(ens, (ty, zc, ln))
         ens.step(2)  # capture the graph and warm up
         t0 = time.perf_counter()
         ens.step(steps)
@@ -95,7 +104,7 @@ def autotune(ens: Ensemble, steps: int = 10, use_cache: bool = True, verbose: bo
         if verbose:
             print("tile_y=%d zchunk=%d lbe_block=%d: %.3f ms/step" % (ty, zc, ln, 1e3 * dt / steps))
     dt, tuning = min(timings)
-    ens.set_tuning(*tuning)
+    set_tuning(ens, tuning)
     best = {"tuning": list(tuning), "ms_per_step": 1e3 * dt / steps,
             "candidates": [[list(t), 1e3 * d / steps] for d, t in timings]}
     if use_cache:
@@ -164,13 +173,14 @@ def measure(steps: int = 500, seed: int = 1400, tune: bool = True, verbose: bool
 
 
 def just_step(steps: int, tuning, seed: int = 1400):
-    """Build the reference ensemble, set `tuning` (tile_y, zchunk, lbe_block)
-    and advance it `steps` steps in one call, untimed (for profilers)."""
+    """Build the reference ensemble, set `tuning` (tile_y, zchunk, lbe_block; 0:
+    the library's choice) and advance it `steps` steps in one call, untimed (for
+    profilers)."""
     import torch
 
     sims = make_members(member_specs(seed=seed))
     ens = Ensemble(sims)
-    ens.set_tuning(*tuning)
+    set_tuning(ens, tuning)
     ens.step(steps)
     torch.cuda.synchronize()
     info = ens.info()
@@ -188,7 +198,7 @@ def main():
     ap.add_argument("--verbose", action="store_true")
     ap.add_argument("--just-step", type=int, default=0, metavar="K",
                     help="only advance the reference ensemble K steps in one call (for profilers)")
-    ap.add_argument("--tuning", type=int, nargs=3, default=[6, 128, 128], metavar=("TILE_Y", "ZCHUNK", "LBE_BLOCK"))
+    ap.add_argument("--tuning", type=int, nargs=3, default=list(DEFAULT_TUNING), metavar=("TILE_Y", "ZCHUNK", "LBE_BLOCK"))
     a = ap.parse_args()
     if a.just_step > 0:
         print(json.dumps(just_step(a.just_step, a.tuning, a.seed)))
