@@ -245,7 +245,8 @@ int kin_num_shells(int N);
  *            the same results); with FP16/BF16 storage and even N an LBE thread
  *            takes 4 cells, or 2 when N % 4 != 0
  *   tile_y   DUGKS fused kernel: rows per tile, 4 or 8 (by default 5, 8 or 11,
- *            chosen with zchunk)
+ *            chosen with zchunk; FP16 and BF16 8; FP64 has tiles of 3 or 7 rows
+ *            whatever is set)
  *   zchunk   DUGKS fused kernel: planes each thread block marches through
  *            (default: the tile height and length whose schedule on the
  *            device's multiprocessors ends first)

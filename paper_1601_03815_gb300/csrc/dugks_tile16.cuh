@@ -6,8 +6,11 @@
 // field holds another sample of the noise (E of a 32^3 BF16 run moves by 5e-3).
 // The moments of f-bar-plus are therefore summed from its rounded populations
 // here, and their differences from population differences, so that results stay
-// the same bit for bit; dugks_tile.cuh forms them from f-tilde and is 20 % faster
-// (256^3 FP16: 0.79 against 0.97 ms).
+// the same bit for bit (256^3: 0.97 ms).  With FP16 storage the FP32 tile
+// (dugks_tile.cuh) took 0.79 ms, but not all of that is its order of operations: in
+// FP32 that gave 0.961 -> 0.928 ms and its schedule (two blocks an SM, one warp for
+// both halo rows, one address base, the z loop unrolled by two) the rest, to 0.773.
+// This tile has the former schedule.
 //
 // Each CTA owns a 30 x TY column of cells and marches along z; its 32 x (TY + 2)
 // threads cover the columns plus a one-cell halo.  Every thread runs the pre-step

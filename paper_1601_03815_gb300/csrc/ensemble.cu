@@ -18,10 +18,10 @@
 // stream of the same graph.  The two kernels never wait on each other;
 // consecutive LBE steps are ordered by their stream.  Two persistent blocks of
 // 5-row tiles fill an SM's registers, so the LBE launches get the SMs before or
-// after them: for the 24-member reference mix 0.366 ms a step of the DUGKS
-// members plus 0.137 ms of the LBE members, 0.502 together.  Tiles that leave
+// after them: for the 24-member reference mix 0.347 ms a step of the DUGKS
+// members plus 0.139 ms of the LBE members, 0.485 together.  Tiles that leave
 // registers for LBE blocks beside them overlap and are still slower (one block
-// of 7-row tiles at 160 registers: 0.520 ms alone, 0.601 together).
+// of 7-row tiles at 160 registers: 0.601 together, where these took 0.502).
 //
 // Which block runs an item does not change what it computes: a member's
 // results are bitwise those of stepping it alone.
@@ -327,8 +327,8 @@ int lbe_vector(const kin_sim* s) {
 }
 
 // Rows of the tiles when the caller has not chosen.  FP32: 5, two 6-warp blocks an SM
-// (0.366 ms a step for the DUGKS members of the reference mix, against 0.402 with 4
-// rows, 0.568 with 6, 0.436 with 8).  One 2-byte type: 8, as stand-alone (the DUGKS and
+// (0.347 ms a step for the DUGKS members of the reference mix, against 0.369 with 4
+// rows, 0.362 with 6, 0.404 with 8).  One 2-byte type: 8, as stand-alone (the DUGKS and
 // LBE members of half the reference mix in FP16: 575 us, 4 rows 765, 5 rows 760, 6 rows
 // 695).  A mixture: 6, the most rows whose block takes 255 registers (2 FP32 and 2 FP16
 // 96^3 members of each scheme: 376 us, 4 rows 457, 5 rows 422, 8 rows 557).
@@ -403,9 +403,9 @@ int launch_persistent_config(kin_ensemble* e) {
 // round: that member's next step waits for the last.  Without the second bound a
 // mix with one large member gets a nearly empty second round (us a step, one
 // 96^3 and one 24^3 DUGKS member beside LBE: 24 planes 122, the 14 chosen now 89.5,
-// the best of a sweep 82 with 32; one of 50^3: 3 planes 22.3, 4 16.4).  The reference mix gets whole columns, at
-// most 128 planes (0.366 ms a step of its DUGKS members; 16 planes: 0.421, 32:
-// 0.385, 64: 0.373).
+// the best of a sweep 82 with 32; one of 50^3: 3 planes 22.3, 4 16.4).  The reference
+// mix gets whole columns, at most 128 planes (0.347 ms a step of its DUGKS members; 16
+// planes: 0.388, 32: 0.358, 64: 0.347).
 int default_zchunk(const kin_ensemble* e) {
     int nsm = 0, top = 1;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, e->device) != cudaSuccess || nsm <= 0) nsm = 152;

@@ -12,8 +12,8 @@
 namespace kin {
 
 // Blocks of b threads along x.  In boxes of up to 64 two rows of 33..64 threads
-// share a block (64^3 FP32 5.4 us a step instead of 6.1, 48^3 4.35 instead of
-// 4.45); one-warp rows stay apart (32^3 3.5 us against 4.0 with four rows a
+// share a block (64^3 FP32 5.2 us a step instead of 6.2, 48^3 3.8 instead of
+// 3.9); one-warp rows stay apart (32^3 3.5 us against 4.0 with four rows a
 // block), and in larger boxes a row fills a block or the rows are many
 // (256^3 FP16: 214 us either way).  Where 32 threads are asked for in a longer row,
 // warps is the rows that share a block (one cell a thread, FP32: 4; blocks of one warp
