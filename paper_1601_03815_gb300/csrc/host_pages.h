@@ -4,7 +4,7 @@
 // faults every page in, one at a time, at 25 GB/s where the copy itself runs at
 // 180 (403 MB: 14.7 ms).  Four threads asking for the pages ahead of the copy take
 // 4.6 ms for the same array, and the copy of a part starts once that part is
-// there (256^3 velocity 17.3 -> 6.9 ms, populations 114 -> 33).
+// there (256^3 velocity 16.5 -> 6.7 ms, populations 109 -> 33).
 #pragma once
 
 #include <sys/mman.h>
@@ -21,7 +21,10 @@ namespace kin {
 
 class HostPages {
 public:
-    static constexpr size_t kPart = size_t(16) << 20;
+    // Arrays below kLeast are left to the copy.  A copy takes a part once its pages are
+    // there: parts of 8 MB 128^3 velocity 1.21 ms, 160^3 1.99 (16 MB 1.39 and 2.15, 2 MB
+    // 1.21 and 2.13).
+    static constexpr size_t kLeast = size_t(32) << 20, kPart = size_t(8) << 20;
     // Threads, and bytes asked for at a time.  403 MB, pages alone: four threads 4.6 ms,
     // eight 14 (they wait for each other in the kernel); four with ranges of 64 KB
     // 5.7, of 16 MB 5.1.  With the copy: two threads 9.2, three 7.3, four 6.9.
@@ -31,7 +34,7 @@ public:
     // [p, p + bytes) is about to be overwritten.  Below 32 MB, or where the pages
     // are there already, nothing is done (6 MB: 0.35 ms either way).
     HostPages(void* p, size_t bytes) : p_(static_cast<char*>(p)), bytes_(bytes) {
-        if (bytes < 2 * kPart || resident()) return;
+        if (bytes < kLeast || resident()) return;
         const size_t parts = (bytes + kPart - 1) / kPart;
         const unsigned cores = std::max(1u, std::thread::hardware_concurrency());
         const size_t threads = std::min<size_t>({kThreads, parts, std::max(1u, cores / 2)});
